@@ -19,19 +19,24 @@ struct alignas(4 * sizeof(T)) QV {
 };
 
 // Tile TM x TN of C per CTA of 256 threads: thread (ty, tx) owns column j0 + tx and rows
-// i0 + ty + 4 s, s < 8, so each row of the tile is written by 64 consecutive threads (coalesced
+// i0 + ty + ROWSTEP s, so each row of the tile is written by TN consecutive threads (coalesced
 // row-major stores).  U diag(S) and V come through shared memory KC rank columns at a time.
-constexpr int CM_TM = 32, CM_TN = 64, CM_THREADS = 256;
-constexpr int CM_ROWSTEP = CM_THREADS / CM_TN;    // 4
-constexpr int CM_RPT = CM_TM / CM_ROWSTEP;        // 8 rows per thread
+// FP32: 32 x 64 tiles, 8 rows a thread.  FP64: the pipe's rate (under two multiply-adds per SM and
+// cycle) is the bound, so small tiles that spread a small matrix over every SM: 8 x 32, one row a
+// thread (256 x 192, k = 10: 192 CTAs instead of 24, 177 -> 42 us).
+constexpr int CM_THREADS = 256;
 
 template <class T>
 __global__ void __launch_bounds__(CM_THREADS) complete_update_kernel(CompleteArgs a) {
+  constexpr int CM_TM = (sizeof(T) == 4) ? 32 : 8, CM_TN = (sizeof(T) == 4) ? 64 : 32;
+  constexpr int CM_ROWSTEP = CM_THREADS / CM_TN;
+  constexpr int CM_RPT = CM_TM / CM_ROWSTEP;        // rows per thread
   constexpr int KC = (sizeof(T) == 4) ? 16 : 8;
   __shared__ QV<T> Us[KC][CM_TM];
   __shared__ QV<T> Vs[KC][CM_TN];
   const int t = threadIdx.x, tx = t % CM_TN, ty = t / CM_TN;
-  const int64_t i0 = (int64_t)blockIdx.y * CM_TM, j0 = (int64_t)blockIdx.x * CM_TN;
+  const int64_t gx = (a.n + CM_TN - 1) / CM_TN;
+  const int64_t i0 = blockIdx.x / gx * CM_TM, j0 = blockIdx.x % gx * CM_TN;
   const T* u[4];
   const T* v[4];
 #pragma unroll
@@ -111,10 +116,12 @@ __global__ void __launch_bounds__(CM_THREADS) complete_update_kernel(CompleteArg
 
 int complete_update(qlr_ctx* ctx, const CompleteArgs& a, int dtype) {
   if (a.m == 0 || a.n == 0) return QLR_OK;
-  const int64_t gy = (a.m + CM_TM - 1) / CM_TM, gx = (a.n + CM_TN - 1) / CM_TN;
-  if (gy > 65535 || gx > 0x7fffffff) return QLR_EUNSUPPORTED;
+  if ((a.m + 31) / 32 > 65535) return QLR_EUNSUPPORTED;
+  const int tm = dtype == QLR_F64 ? 8 : 32, tn = dtype == QLR_F64 ? 32 : 64;
+  const int64_t gy = (a.m + tm - 1) / tm, gx = (a.n + tn - 1) / tn;
+  if (gx * gy > 0x7fffffff) return QLR_EUNSUPPORTED;
   KTimer kt(ctx, QLR_KID_COMPLETE);
-  const dim3 grid((unsigned)gx, (unsigned)gy);
+  const unsigned grid = (unsigned)(gx * gy);
   if (dtype == QLR_F64) complete_update_kernel<double><<<grid, CM_THREADS, 0, ctx->stream>>>(a);
   else complete_update_kernel<float><<<grid, CM_THREADS, 0, ctx->stream>>>(a);
   qlr_count_launch();

@@ -23,77 +23,6 @@ __device__ __forceinline__ int2 upper_tri_entry(int e) {
   return make_int2(e - b * (b + 1) / 2, b);
 }
 
-// ---------------------------------------------------------------------------------------
-// Gram partial sums: part[chunk] = sum over the chunk's rows r of conj(y_ri) y_rj, for tiles
-// (ti <= tj) of the upper triangle.  32 x 32 quaternion tiles, 256 threads, 2 x 2 per thread.
-constexpr int GT = 32, GR = 16;
-
-template <class TY>
-__global__ void __launch_bounds__(256) gram_partial_kernel(const TY* __restrict__ y0, const TY* __restrict__ y1,
-                                                           const TY* __restrict__ y2, const TY* __restrict__ y3,
-                                                           int64_t m, int l, int64_t ld, int64_t rows_per_chunk,
-                                                           double* __restrict__ part) {
-  __shared__ double Yi[4][GR][GT + 1];
-  __shared__ double Yj[4][GR][GT + 1];
-  const int t = threadIdx.x, tx = t % 16, ty = t / 16;
-  const int2 tile = upper_tri_entry((int)blockIdx.x);
-  const int i0 = tile.x * GT, j0 = tile.y * GT;
-  const int64_t r_begin = (int64_t)blockIdx.y * rows_per_chunk;
-  const int64_t r_end = min(m, r_begin + rows_per_chunk);
-  const TY* yp[4] = {y0, y1, y2, y3};
-  Quat<double> acc[2][2];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 2; ++b) acc[a][b] = {0, 0, 0, 0};
-
-  for (int64_t r0 = r_begin; r0 < r_end; r0 += GR) {
-    // load GR rows x GT columns for both column blocks: thread t -> (row t%16, col t/16 (+16))
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        int rr = t % GR, cc = t / GR + 16 * h;
-        int64_t gr = r0 + rr;
-        double vi = 0.0, vj = 0.0;
-        if (gr < r_end) {
-          if (i0 + cc < l) vi = to_d(yp[c][gr + (int64_t)(i0 + cc) * ld]);
-          if (j0 + cc < l) vj = to_d(yp[c][gr + (int64_t)(j0 + cc) * ld]);
-        }
-        Yi[c][rr][cc] = vi;
-        Yj[c][rr][cc] = vj;
-      }
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int rr = 0; rr < GR; ++rr) {
-      Quat<double> a[2], b[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        int ci = tx + 16 * h, cj = ty + 16 * h;
-        a[h] = {Yi[0][rr][ci], Yi[1][rr][ci], Yi[2][rr][ci], Yi[3][rr][ci]};
-        b[h] = {Yj[0][rr][cj], Yj[1][rr][cj], Yj[2][rr][cj], Yj[3][rr][cj]};
-      }
-#pragma unroll
-      for (int x = 0; x < 2; ++x)
-#pragma unroll
-        for (int z = 0; z < 2; ++z) {
-          Quat<double> p = qcmul(a[x], b[z]);
-          acc[x][z].w += p.w; acc[x][z].x += p.x; acc[x][z].y += p.y; acc[x][z].z += p.z;
-        }
-    }
-    __syncthreads();
-  }
-  double* P = part + (size_t)blockIdx.y * 4 * l * l;
-#pragma unroll
-  for (int x = 0; x < 2; ++x)
-#pragma unroll
-    for (int z = 0; z < 2; ++z) {
-      int i = i0 + tx + 16 * x, j = j0 + ty + 16 * z;
-      if (i < l && j < l) st_small(P, l, i, j, acc[x][z]);
-    }
-}
-
 // Sum the chunk partials in a fixed order; write the full Hermitian matrix.
 __global__ void gram_reduce_kernel(const double* __restrict__ part, int nchunks, int l, double* __restrict__ G) {
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1847,35 +1776,25 @@ int gram(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws) {
   const int l = (int)Y.cols;
   const int64_t m = Y.rows;
   if (l == 0) return QLR_OK;
-  const int nt = (l + GT - 1) / GT;
-  const int64_t ntiles = (int64_t)nt * (nt + 1) / 2;
-  int target = 2 * (ctx->num_sms > 0 ? ctx->num_sms : 148);
+  // FP64: row chunks until the upper-triangle tiles give every SM about four CTAs (the FP64 pipe
+  // is the bound, so an even spread is what counts), at least 32 rows each: 350 -> 8 us at 256 x 15
+  const int64_t per = (l > 64) ? 16 * 8 : 8 * 4;
+  const int64_t ntiles = std::max<int64_t>(1, (int64_t)l * l / (2 * per));
+  const int64_t target = 4 * (int64_t)(ctx->num_sms > 0 ? ctx->num_sms : 148);
   int64_t chunks = (target + ntiles - 1) / ntiles;
-  chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, (m + 63) / 64));
+  chunks = std::max<int64_t>(1, std::min<int64_t>(chunks, (m + 31) / 32));
   chunks = std::min<int64_t>(chunks, std::max<int64_t>(1, ((int64_t)64 << 20) / ((int64_t)32 * l * l)));
-  int64_t rpc = ((m + chunks - 1) / chunks + GR - 1) / GR * GR;
-  if (rpc == 0) rpc = GR;
+  chunks = std::min<int64_t>(chunks, 65535);
+  int64_t rpc = ((m + chunks - 1) / chunks + 31) / 32 * 32;
+  if (rpc == 0) rpc = 32;
   chunks = (m + rpc - 1) / rpc;
   if (chunks == 0) chunks = 1;
   size_t mark = ws.off;
   double* part = ws.take<double>((size_t)chunks * 4 * l * l);
   if (!ws.ok) return QLR_ENOMEM;
-  dim3 grid((unsigned)ntiles, (unsigned)chunks);
+  if (Y.dtype == QLR_BF16) return QLR_EINVAL;
   KTimer kt(ctx, QLR_KID_GRAM);
-  if (Y.dtype == QLR_F64) {
-    const double* p[4];
-    for (int c = 0; c < 4; ++c) p[c] = static_cast<const double*>(Y.plane[c]);
-    gram_partial_kernel<double><<<grid, 256, 0, ctx->stream>>>(p[0], p[1], p[2], p[3], m, l, Y.ld, rpc, part);
-    qlr_count_launch();
-  } else if (Y.dtype == QLR_F32) {
-    const float* p[4];
-    for (int c = 0; c < 4; ++c) p[c] = static_cast<const float*>(Y.plane[c]);
-    gram_partial_kernel<float><<<grid, 256, 0, ctx->stream>>>(p[0], p[1], p[2], p[3], m, l, Y.ld, rpc, part);
-    qlr_count_launch();
-  } else {
-    return QLR_EINVAL;
-  }
-  QLR_CUDA_TRY(cudaGetLastError());
+  QLR_TRY(gram_f64_partials(ctx, Y, chunks, rpc, part));
   int64_t tot = (int64_t)l * l;
   gram_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, ctx->stream>>>(part, (int)chunks, l, G);
   qlr_count_launch();

@@ -170,6 +170,8 @@ struct GemmArgs {
   int kid = QLR_KID_APPLY;   // statistics class of the launch
 };
 int gemm_simt(qlr_ctx* ctx, const GemmArgs& g);
+// FP64 Gram partial sums over row chunks (upper triangle), reduced by gram() in orth.cu.
+int gram_f64_partials(qlr_ctx* ctx, const qlr_qmat& Y, int64_t chunks, int64_t rpc, double* part);
 
 // tcgen05 sketch products (see sketch_tc.cu)
 int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qmat& Y, int compute, WsArena& ws);
