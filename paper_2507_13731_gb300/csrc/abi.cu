@@ -22,9 +22,11 @@ size_t gram_ws_bound(int64_t rows, int64_t l) {
 }
 
 size_t cholqr_ws_bound(int64_t rows, int64_t l, size_t esz) {
-  // + the double-FP32 copies of R and the diagonal-block inverses (FP32 sketches)
+  // + the double-FP32 copies of R and the diagonal-block inverses (FP32 sketches); the Gram's
+  // slices and the tall product's splits take turns
+  const size_t tall = (esz == 4 && l < (1 << 20) && tall_gemm_wanted(rows, l, (int)l)) ? tall_gemm_ws(rows, l, (int)l) : 0;
   return (size_t)12 * 32 * l * l + (size_t)8 * l * l + (size_t)4 * (rows + 4) * l * esz + (size_t)16 * l * l +
-         gram_ws_bound(rows, l) + (size_t)32 * l * l + (size_t)8 * 1024 * ((l + 15) / 16) + 17 * 256;
+         std::max(gram_ws_bound(rows, l), tall) + (size_t)32 * l * l + (size_t)8 * 1024 * ((l + 15) / 16) + 17 * 256;
 }
 
 size_t tsvd_ws_bound(int64_t l) { return core_tsvd_ws((int)l) + 16384; }
@@ -228,6 +230,13 @@ int deflate_block(Sched& S, qlr_qmat& K, int64_t c0, int l) {
   const qlr_qmat slot = col_slice(K, c0, l);
   {
     QLR_TRY(qlr::gram(S.ctx, KB, G, *S.ws));
+    if (K.dtype == QLR_F32 && qlr::tall_gemm_wanted(K.rows, l, (int)c0)) {
+      const double* coef[4];                          // (B^H Y)(t, j) = G(t, c0 + j)
+      for (int c = 0; c < 4; ++c) coef[c] = G + (size_t)c * w * w + (size_t)c0 * w;
+      qlr_qmat dst = slot;
+      const int rc = qlr::tall_gemm(S.ctx, col_slice(K, 0, c0), coef, w, l, -1.f, 1.f, false, dst, *S.ws);
+      if (rc != QLR_ENOMEM) { S.ws->off = mark; return rc; }
+    }
     qlr::GemmArgs g{};
     for (int c = 0; c < 4; ++c) {
       g.a[c] = K.plane[c];                          // B(i, t) at plane + i + t ld
@@ -331,7 +340,21 @@ size_t lowrank_ws(int64_t m, int64_t n, int k, int p, int v, int algo, int compu
   b += (size_t)32 * L * L * 3 + (size_t)64 * L * k + 8 * k;   // + the Gram of a deflated stack
   b += cholqr_ws_bound(rows, L, esz) + tsvd_ws_bound(L);
   b += qlr::sketch_tc_ws(rows, L, 160);           // tensor-core operand staging + stream-K partials
-  return b + ((size_t)4 << 20);
+  b += (size_t)4 << 20;
+  // matrix completion's masked update, between the approximations
+  if (compute != QLR_COMPUTE_F64 && qlr::masked_update_tc_wanted(m, n, k)) b = std::max(b, qlr::masked_update_tc_ws(m, n, k));
+  return b;
+}
+
+// The masked update; FP32 updates on the tensor cores where the workspace holds their operands.
+int masked_update(qlr_ctx* ctx, const qlr::CompleteArgs& a, int dtype) {
+  if (dtype == QLR_F32 && qlr::masked_update_tc_wanted(a.m, a.n, a.k) &&
+      qlr_try_ws(ctx, qlr::masked_update_tc_ws(a.m, a.n, a.k))) {
+    WsArena ws(ctx->ws, ctx->ws_bytes);
+    const int rc = qlr::masked_update_tc(ctx, a, ws);
+    if (rc != QLR_ENOMEM) return rc;
+  }
+  return qlr::complete_update(ctx, a, dtype);
 }
 
 }  // namespace
@@ -397,6 +420,22 @@ int qlr_ensure_ws(qlr_ctx* ctx, size_t bytes) {
   }
   ctx->ws_bytes = want;
   return QLR_OK;
+}
+
+bool qlr_try_ws(qlr_ctx* ctx, size_t bytes) {
+  if (ctx->ws_bytes >= bytes) return true;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  void* p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) { cudaFree(p); return false; }
+  if (ctx->ws) cudaFree(ctx->ws);
+  ctx->ws = p;
+  ctx->ws_bytes = bytes;
+  return true;
 }
 
 extern "C" {
@@ -738,7 +777,7 @@ int qlr_qcomplete_update(qlr_ctx* ctx, const qlr_qmat* M, const uint8_t* mask, i
   qlr::CompleteArgs a;
   QLR_TRY(complete_args(M, mask, mask_ld, U, S, V, k, C, a));
   DeviceGuard g(ctx->device);
-  return qlr::complete_update(ctx, a, C->dtype);
+  return masked_update(ctx, a, C->dtype);
 }
 
 int qlr_qcomplete(qlr_ctx* ctx, const qlr_qmat* M, const uint8_t* mask, int64_t mask_ld, int k, int p, int passes,
@@ -753,7 +792,7 @@ int qlr_qcomplete(qlr_ctx* ctx, const qlr_qmat* M, const uint8_t* mask, int64_t 
   QLR_TRY(qlr::complete_update(ctx, start, C->dtype));                        // C = P_Omega(M)
   for (int it = 0; it < iters; ++it) {
     QLR_TRY(lowrank_impl(ctx, C, k, p, passes, algo, omega, opts, U, S, V));   // eq. Step1
-    QLR_TRY(qlr::complete_update(ctx, update, C->dtype));                     // eq. Step2
+    QLR_TRY(masked_update(ctx, update, C->dtype));                     // eq. Step2
   }
   return QLR_OK;
 }

@@ -56,6 +56,9 @@ struct WsArena {
 };
 
 int qlr_ensure_ws(qlr_ctx* ctx, size_t bytes);
+// The same for a workspace that the call can do without: false, with the present workspace kept,
+// when it cannot grow (stream capture, no memory).
+bool qlr_try_ws(qlr_ctx* ctx, size_t bytes);
 
 // Failing CUDA calls are reported on stderr when QLR_DEBUG_CUDA is set in the environment.
 void qlr_report_cuda(cudaError_t e, const char* expr, const char* file, int line);
@@ -291,6 +294,17 @@ size_t tsvd_ws_bound(int64_t l);
 int batch_create(qlr_ctx* ctx, int count, const qlr_qmat* A, const int* k, const int* p, int passes,
                  const qlr_qmat* omega, const qlr_opts* opts, qlr_qmat* U, double* const* S, qlr_qmat* V,
                  bool tune, bool use_graph, qlr_batch** out);
+
+// FP32-accurate tensor-core products of a tall FP32 matrix (thin_tc.cu); ENOMEM (nothing launched)
+// when the arena cannot hold the operands' BF16 splits.
+//   tall_gemm: C = alpha T S + beta C, S an l x N FP64 factor (planes, column pitch lds).
+bool tall_gemm_wanted(int64_t rows, int64_t N, int l);
+size_t tall_gemm_ws(int64_t rows, int64_t N, int l);
+int tall_gemm(qlr_ctx* ctx, const qlr_qmat& T, const double* const S[4], int64_t lds, int64_t N, float alpha, float beta,
+              bool upper, qlr_qmat& C, WsArena& ws);
+bool masked_update_tc_wanted(int64_t m, int64_t n, int k);
+size_t masked_update_tc_ws(int64_t m, int64_t n, int k);
+int masked_update_tc(qlr_ctx* ctx, const CompleteArgs& a, WsArena& ws);
 
 // utilities (util.cu)
 int convert_qmat(qlr_ctx* ctx, const qlr_qmat& src, qlr_qmat& dst);  // elementwise dtype change

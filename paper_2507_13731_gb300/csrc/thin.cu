@@ -1,9 +1,8 @@
 // Thin x small products C = T S: T (rows x l) a tall quaternion basis stored column-major, S a
 // small l x k factor (R^{-1} of a CholeskyQR step, or the core QSVD's singular vectors for the
 // lifts U = Q1 U_hat, V = Q2 V_hat).  FP32 operands run on thin_small_kernel; FP64 operands on
-// the generic SIMT GEMM.  The tensor-core sketch kernel was measured on this shape (4096 x 110 x
-// 110) and gained nothing: with K = l its CTAs run a dozen pipeline stages each and the 3xTF32
-// split costs three MMAs.
+// the generic SIMT GEMM; FP32 products from tall_gemm_wanted()'s size on run on the tensor cores
+// (thin_tc.cu).
 #include <algorithm>
 
 #include "qlr_internal.h"
@@ -145,6 +144,12 @@ int thin_times_small(qlr_ctx* ctx, const qlr_qmat& T, const double* S, int l, in
   // convert its FP64 tile of S again, on the slow FP64 pipe)
   const bool f32 = (T.dtype != QLR_F64 && C.dtype != QLR_F64);
   const size_t mark = ws.off;
+  if (T.dtype == QLR_F32 && C.dtype == QLR_F32 && T.plane[0] != nullptr && tall_gemm_wanted(T.rows, k, l)) {
+    const double* s[4];
+    for (int c = 0; c < 4; ++c) s[c] = S + (size_t)c * l * k;
+    const int rc = tall_gemm(ctx, T, s, l, k, 1.f, 0.f, S_upper, C, ws);
+    if (rc != QLR_ENOMEM) return rc;
+  }
   float* s32 = f32 ? ws.take<float>((size_t)4 * l * k) : nullptr;
   if (s32) {
     const int64_t n = (int64_t)4 * l * k;
