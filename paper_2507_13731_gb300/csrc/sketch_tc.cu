@@ -18,9 +18,15 @@
 // its rows: for BF16 the MMA consumes the MN-major tile directly; for the 4-byte modes the tile is
 // loaded unswizzled and the worker warps transpose it into the K-major swizzled layout (splitting
 // it into hi / lo on the way for 3xTF32).
-// Warp roles: 0 = TMA producer, 1 = MMA issuer (owns TMEM), 2-3 = workers (hi/lo split,
+// Warp roles: 0 = TMA producer, 1 = MMA issuer (owns TMEM), 2-3 = a pair of workers (hi/lo split,
 // rounding and/or transpose of A), 4-7 = epilogue (TMEM -> registers -> global, or a stream-K
-// partial + the last piece's reduction).
+// partial + the last piece's reduction); with 384 threads, 8-11 = two more worker pairs or four more
+// epilogue warps.
+// The MMA issuer is one thread, and what it does between two stages' MMAs leaves the tensor pipe
+// idle: its ring and chunk positions are counters (the integer divisions they replace took 300 of a
+// stage's 1700 cycles in plain TF32).  Measured (Y = A X and Z = A^H W together, with the staging):
+// 3xTF32 4096 x 4096 x 110 761 -> 630 us, BF16 16384 x 8192 x 220 1638 -> 1522 us, TF32 pure
+// 20000 x 10000 x 60 1431 -> 1348 us, rounded TF32 x 180 5021 -> 4736 us.
 //
 // Precision modes: BF16 (kind::f16, A stored BF16, X rounded to BF16), TF32 (kind::tf32, one
 // product on FP32 data, which the tensor cores truncate to TF32), rounded TF32 (one product, A and
@@ -42,7 +48,11 @@ namespace {
 
 using namespace qlr_tc;
 
-constexpr int TC_THREADS = 256;
+constexpr int TC_THREADS = 256;      // 2 special warps, a pair of workers, 4 epilogue warps
+// Single-problem launches of the modes whose workers touch every A stage: two more worker pairs, or
+// (3xTF32 whose chunk sums go through global memory) four more epilogue warps.  384 threads still
+// leave the 138 registers that the epilogue needs.
+constexpr int TC_THREADS_WIDE = 384;
 constexpr int TBM = 128;          // output rows per CTA (MMA M)
 constexpr int MAX_STAGES = 8;    // pipeline stages (as many as fit in shared memory, at most 8)
 constexpr int PMAX_STAGES = MAX_STAGES;
@@ -77,6 +87,7 @@ struct TcParams {
   int fd;                   // 1: fused output planes (one MMA per input plane, N = 4 nb; see issue_stage)
   int rn;                   // 1 (TF32): A rounded to nearest TF32 in shared memory before the MMAs read it
   int cgroup;               // stream-K in column-block groups (gridDim.x a multiple of ncb)
+  int epi2;                 // warps 8-11 are epilogue warps (384 threads)
 };
 
 // The scalar part of TcParams, copied into registers once: with the parameters in global memory
@@ -91,7 +102,7 @@ struct TcScalars {
   int l, nb, ncb, kiters, c_first, stages;
   uint32_t neg_mask, idesc_base, tmem_cols;
   int* err;
-  int flush, nbuf, ttotal, apl, fd, rn;
+  int flush, nbuf, ttotal, apl, fd, rn, epi2;
   __device__ __forceinline__ float* y(int d) const { return d == 0 ? y0 : d == 1 ? y1 : d == 2 ? y2 : y3; }
 };
 __device__ __forceinline__ TcScalars tc_scalars(const TcParams& p) {
@@ -101,7 +112,7 @@ __device__ __forceinline__ TcScalars tc_scalars(const TcParams& p) {
   v.kiters = p.kiters; v.c_first = p.c_first; v.stages = p.stages;
   v.neg_mask = p.neg_mask; v.idesc_base = p.idesc_base; v.tmem_cols = p.tmem_cols; v.err = p.err;
   v.flush = p.flush; v.nbuf = p.nbuf < 1 ? 1 : p.nbuf; v.ttotal = p.ttotal; v.apl = p.apl == 3 ? 3 : 4; v.fd = p.fd;
-  v.rn = p.rn;
+  v.rn = p.rn; v.epi2 = p.epi2;
   return v;
 }
 
@@ -312,6 +323,9 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
   const int NBUF = pv.nbuf;
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int EPI = pv.epi2 ? 2 : 1;                     // epilogue warps per lane quarter
+  // worker pairs: warps 2-3, then those from warp 8 on that are not epilogue warps
+  const int NPAIR = WORKERS ? 1 + ((int)blockDim.x - TC_THREADS - (pv.epi2 ? 128 : 0)) / 64 : 0;
   const int64_t m0 = (int64_t)mt * TBM;
   const int j0 = cb * nb;
   const int it0 = sg.it0;
@@ -329,11 +343,11 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
     for (int s = 0; s < MAX_STAGES; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
-      mbar_init(&ready[s], 64);
+      mbar_init(&ready[s], 2 * (4 - pv.c_first));   // two worker warps per plane
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tmem_full[b], 1);
-      mbar_init(&tmem_empty[b], 128);
+      mbar_init(&tmem_empty[b], 4 * EPI);           // one arrival per epilogue warp
     }
     *abort_flag = 0;
     *last_flag = 0;
@@ -361,10 +375,9 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
       // groups), so their loads keep the default priority.
       const bool hint = (pv.ncb == 1);
       const uint64_t pol_a = l2_evict_first_policy(), pol_x = l2_evict_last_policy();
-      int issued = 0;
+      int issued = 0, s = 0;
+      uint32_t ph = 0;
       for (int i = 0; i < nit; ++i) {
-        const int s = i % STAGES;
-        const uint32_t ph = (uint32_t)(i / STAGES) & 1u;
         if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, pv.err)) break;
         mbar_expect_tx(&full[s], tx);
         const int k0 = (it0 + i) * C::BK;
@@ -394,6 +407,7 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
           }
         }
         ++issued;
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
       // drain: every issued stage must have landed before the CTA may exit
       for (int i = max(0, issued - STAGES); i < issued; ++i) {
@@ -407,94 +421,100 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
       bool ok = true;
-      int chunk = 0;
+      int chunk = 0, buf = 0, ic = 0, s = 0;       // chunk, its buffer, stage within it, ring slot
+      uint32_t ph = 0;
+      const int nb_log = NBUF - 1;                 // NBUF is 1 or 2
       const StageDescs D = make_stage_descs<KIND, AMODE, WIDE>(smem_u32(smem), stage_bytes, HI_OFF - C0 * A_BYTES,
                                                                A_BYTES, A_SET, X_BYTES, APL, NXP);
-      for (int i = 0; i < nit && ok; ++i) {
-        const int ic = i % F;                      // stage within the accumulation chunk
-        if (i > 0 && ic == 0) {                    // chunk boundary: hand the finished chunk over
-          umma_commit(&tmem_full[chunk % NBUF]);
+#pragma unroll 1
+      for (int i = 0; i < nit; ++i) {
+        if (ic == F) {                             // chunk boundary: hand the finished chunk over
+          umma_commit(&tmem_full[buf]);
           ++chunk;
+          buf = chunk & nb_log;
+          ic = 0;
           if (chunk >= NBUF) {                     // its buffer must have been drained first
-            ok = mbar_wait(&tmem_empty[chunk % NBUF], (uint32_t)((chunk / NBUF) - 1) & 1u, abort_flag, pv.err);
+            ok = mbar_wait(&tmem_empty[buf], (uint32_t)((chunk >> nb_log) - 1) & 1u, abort_flag, pv.err);
             if (!ok) break;
             tc_fence_after();
           }
         }
-        const uint32_t abase = tmem + (uint32_t)((chunk % NBUF) * 4 * nb);
-        const int s = i % STAGES;
-        const uint32_t ph = (uint32_t)(i / STAGES) & 1u;
+        const uint32_t abase = tmem + (uint32_t)(buf * 4 * nb);
         ok = mbar_wait(WORKERS ? &ready[s] : &full[s], ph, abort_flag, pv.err);
         if (!ok) break;
         tc_fence_after();
         issue_stage<KIND, AMODE, WIDE>(D, s, abase, nb, pv.c_first, pv.idesc_base, pv.neg_mask, ic == 0, pv.fd, C0);
         umma_commit(&empty[s]);   // frees the stage once these MMAs have read it
+        ++ic;
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
-      umma_commit(&tmem_full[chunk % NBUF]);   // last chunk complete (also fires after an abort)
+      umma_commit(&tmem_full[buf]);   // last chunk complete (also fires after an abort)
     }
-  } else if (warp < 4) {
+  } else if (warp < 4 || warp >= (pv.epi2 ? 12 : 8)) {
     // ---------------- workers: hi/lo split (3xTF32) and/or transpose of A ----------------
+    // A pair of warps takes one plane of one stage at a time, the pairs in turn.
     if (WORKERS) {
-      const int st = threadIdx.x - 64;   // 0..63
-      for (int i = 0; i < nit; ++i) {
-        const int s = i % STAGES;
-        const uint32_t ph = (uint32_t)(i / STAGES) & 1u;
+      const int pair = warp < 4 ? 0 : (warp - (pv.epi2 ? 12 : 8)) / 2 + 1;
+      const int st = (warp & 1) * 32 + lane;   // 0..63 within the pair
+      const int np = 4 - pv.c_first;
+      int i = 0, c = pair, s = 0;
+      uint32_t ph = 0;
+      auto settle = [&]() {                     // (stage, plane) from a plane count beyond the stage's
+        while (c >= np) {
+          c -= np;
+          ++i;
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
+        }
+      };
+      settle();
+#pragma unroll 1
+      for (; i < nit; c += NPAIR, settle()) {
         if (!mbar_wait(&full[s], ph, abort_flag, pv.err)) break;
-        for (int c = pv.c_first; c < 4; ++c) {
-          uint4* hi = reinterpret_cast<uint4*>(a_plane(s, c));
-          uint4* lo = reinterpret_cast<uint4*>(alo_plane(s, c));
-          if (TR) {
-            // raw[k][r] (k < BK, r < 128) -> row r of the K-major tile, 16-byte chunk cch holding
-            // k = 4 cch .. 4 cch + 3, stored at chunk position cch ^ swizzle(r).  In place: the
-            // workers read the whole raw plane into registers, meet at a named barrier, then write.
-            const uint32_t* raw = reinterpret_cast<const uint32_t*>(raw_plane(s, c));
-            constexpr int NPER = TBM * CH / 64;
-            uint4 vv[NPER];
+        uint4* hi = reinterpret_cast<uint4*>(a_plane(s, pv.c_first + c));
+        uint4* lo = reinterpret_cast<uint4*>(alo_plane(s, pv.c_first + c));
+        // all of the plane's loads before its first store: in place, and in flight together
+        constexpr int NPER = TBM * CH / 64;
+        uint4 vv[NPER];
+        if (TR) {
+          // raw[k][r] (k < BK, r < 128) -> row r of the K-major tile, 16-byte chunk cch holding
+          // k = 4 cch .. 4 cch + 3, stored at chunk position cch ^ swizzle(r).  In place: the
+          // pair reads the whole raw plane into registers, meets at a named barrier, then writes.
+          const uint32_t* raw = reinterpret_cast<const uint32_t*>(raw_plane(s, pv.c_first + c));
 #pragma unroll
-            for (int q = 0; q < NPER; ++q) {
-              const int e = st + 64 * q, r = e % TBM, cch = e / TBM;
-              vv[q].x = raw[(4 * cch + 0) * TBM + r];
-              vv[q].y = raw[(4 * cch + 1) * TBM + r];
-              vv[q].z = raw[(4 * cch + 2) * TBM + r];
-              vv[q].w = raw[(4 * cch + 3) * TBM + r];
-            }
-            asm volatile("bar.sync 2, 64;" ::: "memory");
+          for (int q = 0; q < NPER; ++q) {
+            const int e = st + 64 * q, r = e % TBM, cch = e / TBM;
+            vv[q].x = raw[(4 * cch + 0) * TBM + r];
+            vv[q].y = raw[(4 * cch + 1) * TBM + r];
+            vv[q].z = raw[(4 * cch + 2) * TBM + r];
+            vv[q].w = raw[(4 * cch + 3) * TBM + r];
+          }
+          asm volatile("bar.sync %0, 64;" ::"r"(2 + pair) : "memory");
+        } else {
 #pragma unroll
-            for (int q = 0; q < NPER; ++q) {
-              const int e = st + 64 * q, r = e % TBM, cch = e / TBM;
-              const int sw = (CH == 2) ? ((r >> 2) & 1) : (CH == 4) ? ((r >> 1) & 3) : (r & 7);
-              const uint4 v = vv[q];
-              const int o = r * CH + (cch ^ sw);
-              if (X3) {
-                uint4 h, rr;
-                h.x = v.x & 0xFFFFE000u; h.y = v.y & 0xFFFFE000u; h.z = v.z & 0xFFFFE000u; h.w = v.w & 0xFFFFE000u;
-                rr.x = __float_as_uint(__uint_as_float(v.x) - __uint_as_float(h.x));
-                rr.y = __float_as_uint(__uint_as_float(v.y) - __uint_as_float(h.y));
-                rr.z = __float_as_uint(__uint_as_float(v.z) - __uint_as_float(h.z));
-                rr.w = __float_as_uint(__uint_as_float(v.w) - __uint_as_float(h.w));
-                hi[o] = h;
-                lo[o] = rr;
-              } else {
-                hi[o] = RN ? tf32_rna4(v) : v;
-              }
-            }
-          } else if (!X3) {   // RN: round the K-major tile in place
-            for (int e = st; e < A_BYTES / 16; e += 64) hi[e] = tf32_rna4(hi[e]);
+          for (int q = 0; q < NPER; ++q) vv[q] = hi[st + 64 * q];
+        }
+#pragma unroll
+        for (int q = 0; q < NPER; ++q) {
+          const int e = st + 64 * q, r = e % TBM, cch = e / TBM;
+          const int sw = (CH == 2) ? ((r >> 2) & 1) : (CH == 4) ? ((r >> 1) & 3) : (r & 7);
+          const uint4 v = vv[q];
+          const int o = TR ? r * CH + (cch ^ sw) : e;
+          if (X3) {
+            uint4 h, rr;
+            h.x = v.x & 0xFFFFE000u; h.y = v.y & 0xFFFFE000u; h.z = v.z & 0xFFFFE000u; h.w = v.w & 0xFFFFE000u;
+            rr.x = __float_as_uint(__uint_as_float(v.x) - __uint_as_float(h.x));
+            rr.y = __float_as_uint(__uint_as_float(v.y) - __uint_as_float(h.y));
+            rr.z = __float_as_uint(__uint_as_float(v.z) - __uint_as_float(h.z));
+            rr.w = __float_as_uint(__uint_as_float(v.w) - __uint_as_float(h.w));
+            hi[o] = h;
+            lo[o] = rr;
           } else {
-            for (int e = st; e < A_BYTES / 16; e += 64) {
-              uint4 v = hi[e], h, r;
-              h.x = v.x & 0xFFFFE000u; h.y = v.y & 0xFFFFE000u; h.z = v.z & 0xFFFFE000u; h.w = v.w & 0xFFFFE000u;
-              r.x = __float_as_uint(__uint_as_float(v.x) - __uint_as_float(h.x));
-              r.y = __float_as_uint(__uint_as_float(v.y) - __uint_as_float(h.y));
-              r.z = __float_as_uint(__uint_as_float(v.z) - __uint_as_float(h.z));
-              r.w = __float_as_uint(__uint_as_float(v.w) - __uint_as_float(h.w));
-              hi[e] = h;
-              lo[e] = r;
-            }
+            hi[o] = RN ? tf32_rna4(v) : v;
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive(&ready[s]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ready[s]);
       }
     }
   } else {
@@ -505,10 +525,11 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
     const int tile = mt * pv.ncb + cb;
     const size_t tile_elems = (size_t)4 * TBM * nb;
     const int nchunks = (nit > 0) ? (nit + F - 1) / F : 1;
+    const int nb_log = NBUF - 1, eh = warp >= 8 ? 1 : 0;   // NBUF is 1 or 2; this warp's half of the columns
     bool ok = true;
     for (int ch = 0; ch < nchunks && ok; ++ch) {
-      const int b = ch % NBUF;
-      ok = mbar_wait(&tmem_full[b], (uint32_t)(ch / NBUF) & 1u, abort_flag, pv.err) && !*abort_flag;
+      const int b = ch & nb_log;
+      ok = mbar_wait(&tmem_full[b], (uint32_t)(ch >> nb_log) & 1u, abort_flag, pv.err) && !*abort_flag;
       tc_fence_after();
       if (!ok || nit == 0) break;
       const bool first = (ch == 0);
@@ -517,6 +538,7 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
       const uint32_t tbase = tmem + (uint32_t)(4 * nb);   // running sum (pv.ttotal)
       const bool to_total = pv.ttotal && !last;             // this chunk only updates the TMEM sum
       const bool add_total = pv.ttotal && !first;           // the TMEM sum enters this chunk's values
+#pragma unroll 1
       for (int d = 0; d < 4; ++d) {
         // the output plane d of this tile: Y itself (a whole tile) or this piece's partial slot
         float* dst;
@@ -531,7 +553,8 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
           stride = TBM;
           valid_row = true;
         }
-        for (int cc = 0; cc < nb; cc += 32) {
+#pragma unroll 1
+        for (int cc = 32 * eh; cc < nb; cc += 32 * EPI) {
           // two TMEM loads in flight per wait (nb is a multiple of 16)
           uint32_t r0[16], r1[16], s0[16], s1[16];
           const uint32_t lane_off = ((uint32_t)(q * 32) << 16) + (uint32_t)(d * nb + cc);
@@ -574,21 +597,22 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
       }
       if (to_total) tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(&tmem_empty[b]);   // this chunk's accumulator may be overwritten
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tmem_empty[b]);   // this chunk's accumulator may be overwritten
     }
     if (sg.nseg > 1) {
       __threadfence();
-      asm volatile("bar.sync 1, 128;" ::: "memory");
+      asm volatile("bar.sync 1, %0;" ::"r"(128 * EPI) : "memory");
       if (threadIdx.x == 128) {
         const unsigned old = atomicAdd(&pv.counters[tile], 1u);
         *last_flag = (old == (unsigned)(sg.nseg - 1)) ? 1 : 0;
       }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
+      asm volatile("bar.sync 1, %0;" ::"r"(128 * EPI) : "memory");
       if (*last_flag) {
         __threadfence();
         if (grow < pv.M) {
           for (int d = 0; d < 4; ++d)
-            for (int jc0 = 0; jc0 < nb; jc0 += 16) {
+            for (int jc0 = 16 * eh; jc0 < nb; jc0 += 16 * EPI) {
               float acc[16];
 #pragma unroll
               for (int jj = 0; jj < 16; ++jj) acc[jj] = 0.f;
@@ -620,7 +644,7 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
 
 // One CTA per output tile, the whole reduction.
 template <int KIND, int AMODE, bool WIDE>
-__global__ void __launch_bounds__(TC_THREADS, 1) sketch_tc_kernel(const __grid_constant__ TcParams p) {
+__global__ void __launch_bounds__(KIND == K_BF16 ? TC_THREADS : TC_THREADS_WIDE, 1) sketch_tc_kernel(const __grid_constant__ TcParams p) {
   sketch_tile<KIND, AMODE, WIDE>(p, blockIdx.x, blockIdx.y, Seg{0, p.kiters, 0, 1, 0, 0, 0});
 }
 
@@ -637,7 +661,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) sketch_tc_kernel(const __grid_c
 // given A stage for different blocks are a tile's length apart in time and A is re-read from
 // DRAM once per block).
 template <int KIND, int AMODE, bool WIDE>
-__global__ void __launch_bounds__(TC_THREADS, 1) sketch_tc_streamk_kernel(const __grid_constant__ TcParams p) {
+__global__ void __launch_bounds__(KIND == K_BF16 ? TC_THREADS : TC_THREADS_WIDE, 1) sketch_tc_streamk_kernel(const __grid_constant__ TcParams p) {
   const int NG = (p.cgroup && p.ncb > 1) ? p.ncb : 1;             // CTAs per group step
   const int cbg = (int)(blockIdx.x % NG);                         // this CTA's block (groups)
   const int64_t K = p.kiters, W = (int64_t)p.mtiles * (p.ncb / NG) * K, G = gridDim.x / NG, c = blockIdx.x / NG;
@@ -657,8 +681,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) sketch_tc_streamk_kernel(const 
     const Seg sg{it0, it1, (int)(2 * (c * NG + cbg) + (c == c0 ? b0 : 0)), (int)(c1 - c0 + 1), (int)c0, b0, more,
                  NG, cbg};
     if (!first) __syncthreads();
-    if (NG > 1) sketch_tile<KIND, AMODE, WIDE>(p, cbg, (int)t, sg);
-    else sketch_tile<KIND, AMODE, WIDE>(p, (int)(t % p.ncb), (int)(t / p.ncb), sg);
+    const int mt = (NG > 1) ? (int)t : (int)t / p.ncb;
+    sketch_tile<KIND, AMODE, WIDE>(p, (NG > 1) ? cbg : (int)t - mt * p.ncb, mt, sg);
     first = false;
     pos += it1 - it0;
   }
@@ -1153,12 +1177,13 @@ int launch_kernel(qlr_ctx* ctx, const Plan& pl, const TcParams& prm, int kid) {
   auto kern = sketch_tc_kernel<KIND, AMODE, WIDE>;
   QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
   KTimer kt(ctx, kid);
+  const int threads = (KIND == K_TF32X3 || AMODE == A_T || prm.rn) ? TC_THREADS_WIDE : TC_THREADS;
   if (pl.grid_sk > 0) {
     auto sk = sketch_tc_streamk_kernel<KIND, AMODE, WIDE>;
     QLR_CUDA_TRY(cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
-    sk<<<pl.grid_sk, TC_THREADS, pl.smem, ctx->stream>>>(prm);
+    sk<<<pl.grid_sk, threads, pl.smem, ctx->stream>>>(prm);
   } else {
-    kern<<<dim3((unsigned)pl.ncb, (unsigned)pl.mtiles, 1u), TC_THREADS, pl.smem, ctx->stream>>>(prm);
+    kern<<<dim3((unsigned)pl.ncb, (unsigned)pl.mtiles, 1u), threads, pl.smem, ctx->stream>>>(prm);
   }
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
@@ -1615,6 +1640,8 @@ int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qm
   prm.ttotal = pl.ttotal;
   prm.rn = pl.rn ? 1 : 0;
   prm.cgroup = pl.cgroup ? 1 : 0;
+  // chunk sums read and written in global memory while the MMAs wait: twice the warps
+  prm.epi2 = (pl.kind == K_TF32X3 && pl.flush > 0 && !pl.ttotal) ? 1 : 0;
   int rc;
   const bool h = (op != QLR_OP_N);
   const int kid = (pl.kind == K_TF32X3) ? QLR_KID_SKETCH_X3 : pl.rn ? QLR_KID_SKETCH_RN : QLR_KID_SKETCH_TC;
