@@ -1001,57 +1001,85 @@ struct StageArg {
   void* out_lo;
   int fd, nb, ncb, c0;
   uint32_t neg;                   // bit c*4+d: sign(c, d) = -1
-  int nrows;                      // staged rows: 4 cols, or (4 - c0) ncb 4 nb
+  int nrows;                      // columns of the four planes: 4 cols, or 4 ncb nb with the blocks' padding
   int rn;                         // TF32: round to nearest TF32 (else the FP32 bits, truncated by the MMA)
 };
 
+// Four consecutive elements [i, i + 4) of column j of plane q of X (row r = q columns + j of the
+// unit list, columns padded to whole blocks in the fused layout) into every staged row that holds
+// them: X is read once, 16 bytes at a time where its pitch allows, and written 16 (BF16: 8) bytes
+// at a time (the earlier one-element copies read a fused column once per staged row, with one load
+// in flight per thread: 36 us at K = 10000..20000, l = 60, now 9).
 template <int MODE>
-__device__ __forceinline__ void stage_row(const StageArg& a, int r, int64_t k0, int64_t k1, int t, int nt) {
-  int q, j;
-  float sg = 1.f;
-  bool valid = true;
-  if (!a.fd) {
-    q = r / (int)a.cols;
-    j = r % (int)a.cols;
-  } else {
-    const int per = a.ncb * 4 * a.nb;
-    const int c = a.c0 + r / per, rr = r % per;
-    const int d = (rr % (4 * a.nb)) / a.nb;
-    j = (rr / (4 * a.nb)) * a.nb + rr % a.nb;
-    q = c ^ d;
-    sg = ((a.neg >> (c * 4 + d)) & 1u) ? -1.f : 1.f;
-    valid = j < a.cols;
-  }
-  const float* src = a.x[q] + (int64_t)(valid ? j : 0) * a.ldx;
-  const size_t o0 = (size_t)r * a.ldo;
-  for (int64_t i = k0 + t; i < k1; i += nt) {
-    const float v = valid ? sg * src[i] : 0.f;
-    if (MODE == K_BF16) {
-      static_cast<__nv_bfloat16*>(a.out)[o0 + i] = __float2bfloat16_rn(v);
-    } else if (MODE == K_TF32) {
-      static_cast<float*>(a.out)[o0 + i] = a.rn ? __uint_as_float(tf32_rna(__float_as_uint(v))) : v;
+__device__ __forceinline__ void stage_quad(const StageArg& a, int r, int64_t i) {
+  const int width = a.fd ? a.ncb * a.nb : (int)a.cols;
+  const int q = r / width, j = r - q * width;
+  float v[4] = {0.f, 0.f, 0.f, 0.f};
+  if (j < a.cols) {
+    const float* src = (q == 0 ? a.x[0] : q == 1 ? a.x[1] : q == 2 ? a.x[2] : a.x[3]) + (int64_t)j * a.ldx + i;
+    if (i + 4 <= a.rows && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+      const float4 f = *reinterpret_cast<const float4*>(src);
+      v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
     } else {
-      const float h = __uint_as_float(__float_as_uint(v) & 0xFFFFE000u);
-      static_cast<float*>(a.out)[o0 + i] = h;
-      static_cast<float*>(a.out_lo)[o0 + i] = v - h;
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (i + e < a.rows) v[e] = src[e];
+    }
+  }
+  // the pitch ldo is a multiple of 8 beyond the rows, so whole quads may be written
+  auto put = [&](int row, bool neg) {
+    const size_t o = (size_t)row * a.ldo + i;
+    float w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) w[e] = neg ? -v[e] : v[e];
+    if (MODE == K_BF16) {
+      __nv_bfloat162 p[2] = {__floats2bfloat162_rn(w[0], w[1]), __floats2bfloat162_rn(w[2], w[3])};
+      *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(a.out) + o) = *reinterpret_cast<uint2*>(p);
+    } else if (MODE == K_TF32) {
+      if (a.rn) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[e] = __uint_as_float(tf32_rna(__float_as_uint(w[e])));
+      }
+      *reinterpret_cast<float4*>(static_cast<float*>(a.out) + o) = make_float4(w[0], w[1], w[2], w[3]);
+    } else {
+      float h[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) h[e] = __uint_as_float(__float_as_uint(w[e]) & 0xFFFFE000u);
+      *reinterpret_cast<float4*>(static_cast<float*>(a.out) + o) = make_float4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<float4*>(static_cast<float*>(a.out_lo) + o) =
+          make_float4(w[0] - h[0], w[1] - h[1], w[2] - h[2], w[3] - h[3]);
+    }
+  };
+  if (!a.fd) {
+    put(r, false);
+  } else {
+    const int cb = j / a.nb, jj = j - cb * a.nb;
+    for (int c = a.c0; c < 4; ++c) {
+      const int d = c ^ q;
+      put(((c - a.c0) * a.ncb + cb) * 4 * a.nb + d * a.nb + jj, ((a.neg >> (c * 4 + d)) & 1u) != 0);
     }
   }
 }
 
-// Grouped: problem blockIdx.y; a warp per staged row, the rows over the grid's x blocks.
+// Grouped: problem blockIdx.y; its (column, 128 elements) units over the grid's x blocks, a warp each.
 template <int MODE>
 __global__ void __launch_bounds__(256) stage_x_grouped_kernel(const StageArg* __restrict__ args) {
   const StageArg a = args[blockIdx.y];
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  for (int r = blockIdx.x * 8 + warp; r < a.nrows; r += gridDim.x * 8) stage_row<MODE>(a, r, 0, a.rows, lane, 32);
+  const int chunks = (int)((a.rows + 127) / 128), units = a.nrows * chunks;
+  for (int u = blockIdx.x * 8 + warp; u < units; u += gridDim.x * 8) {
+    const int r = u / chunks;
+    const int64_t i = (int64_t)(u - r * chunks) * 128 + 4 * lane;
+    if (i < a.rows) stage_quad<MODE>(a, r, i);
+  }
 }
 
-// One problem: grid (reduction chunks of STAGE_ROWS, staged rows).
-constexpr int STAGE_ROWS = 2048;
+// One problem: grid (reduction chunks of STAGE_ROWS, columns of the four planes).
+constexpr int STAGE_ROWS = 1024;
 template <int MODE>
 __global__ void __launch_bounds__(256) stage_x_kernel(const StageArg a) {
-  const int64_t k0 = (int64_t)blockIdx.x * STAGE_ROWS;
-  stage_row<MODE>(a, (int)blockIdx.y, k0, min(a.rows, k0 + STAGE_ROWS), threadIdx.x, blockDim.x);
+  const int64_t i = (int64_t)blockIdx.x * STAGE_ROWS + 4 * threadIdx.x;
+  if (i < a.rows) stage_quad<MODE>(a, (int)blockIdx.y, i);
 }
 
 // Staged X bytes of one problem (hi set; the 3xTF32 lo set is as large again).
@@ -1421,8 +1449,9 @@ int sketch_tc_grouped_plan(qlr_ctx* ctx, int op, int count, const qlr_qmat* A, c
     sa.ncb = g.ncb;
     sa.c0 = 4 - apl;
     sa.neg = neg;
-    sa.nrows = fd ? apl * g.ncb * 4 * g.nb : 4 * g.l;
-    max_stage_blocks = std::max<int>(max_stage_blocks, std::min<int>((sa.nrows + 7) / 8, 64));   // 8 rows per CTA
+    sa.nrows = 4 * (fd ? g.ncb * g.nb : g.l);
+    const int64_t units = sa.nrows * ((g.K + 127) / 128);
+    max_stage_blocks = std::max<int>(max_stage_blocks, (int)std::min<int64_t>((units + 7) / 8, 64));   // 8 units per CTA and turn
     for (int mt = 0; mt < g.mtiles; ++mt)
       for (int cb = 0; cb < g.ncb; ++cb) hi.push_back(make_int4(i, mt, cb, 0));
   }
@@ -1563,9 +1592,9 @@ int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qm
     sa.ncb = pl.ncb;
     sa.c0 = 4 - pl.apl;
     sa.neg = neg_table(op);
-    sa.nrows = pl.fd ? pl.apl * pl.ncb * 4 * pl.nb : 4 * l;
+    sa.nrows = 4 * (pl.fd ? pl.ncb * pl.nb : l);
     sa.rn = pl.rn ? 1 : 0;
-    if (sa.nrows > 65535) return QLR_EUNSUPPORTED;
+    if ((pl.fd ? pl.apl * pl.ncb * 4 * pl.nb : 4 * l) > 65535) return QLR_EUNSUPPORTED;   // staged rows
     const dim3 grid((unsigned)((K + STAGE_ROWS - 1) / STAGE_ROWS), (unsigned)sa.nrows);
     KTimer kt(ctx, QLR_KID_MISC);
     if (pl.kind == K_BF16) stage_x_kernel<K_BF16><<<grid, 256, 0, ctx->stream>>>(sa);
