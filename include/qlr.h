@@ -212,7 +212,7 @@ int qlr_qsketch(qlr_ctx* ctx, int op, const qlr_qmat* A, const qlr_qmat* X, qlr_
 /*
  * qlr_qgram -- G = Y^H Y with FP64-class accuracy (the Gram step of CholeskyQR; the "QR" of
  * Algorithms 1-4, Def. 1 eq. QQR).  F64 Y: FP64 arithmetic.  F32 Y: on the tensor cores by an
- * exact splitting of every column into 6-bit BF16 slices below its largest entry (error about
+ * exact splitting of every column into 7-bit BF16 slices below its largest entry (error about
  * 2^-45 of max|y_i| max|y_j| m), or, when the workspace cannot hold the slices, double-FP32 sums
  * on the FP32 pipes.  Y: m x l column-major F32 or F64.  G: device, FP64, l x l x 4 planes,
  * column-major (G[c*l*l + j*l + i]), full Hermitian matrix written.

@@ -4,25 +4,29 @@
 // G's components are sums of the real Gram W = Yh^T Yh of the plane-stacked Yh = [Y0 Y1 Y2 Y3]
 // (m x 4l).  W is formed exactly enough for FP64-class use by an error-free splitting:
 //  - every column c of Yh gets the exponent e_c with max_r |Yh(r, c)| < 2^e_c, and each entry is
-//    written as y = 2^(e_c - 6) (q_1 + q_2 2^-6 + ... + q_8 2^-42) + rest with integers
-//    |q_i| <= 63 (48 bits below the column maximum; an entry of at least 2^-24 of the column
-//    maximum is represented exactly, a smaller one to 2^-48 of the maximum);
+//    written in balanced base 128, y = 2^(e_c - 6) (q_1 + q_2 2^-7 + ... + q_7 2^-42) + rest with
+//    integers |q_i| <= 64, each the nearest to what is left (the rest is at most 2^-49 of 2^e_c; an
+//    entry of at least 2^-25 of it is represented exactly);
 //  - the q_i are exact in BF16, their products exact in FP32, and the tensor core's FP32 sums of
 //    such integer products stay exact while they stay below 2^24: the slice pairs (i, j) of equal
-//    weight s = i + j - 2 share one TMEM accumulator, at most 8 pairs x 512 rows x 63^2 < 2^24,
+//    weight s = i + j - 2 share one TMEM accumulator, at most 7 pairs x 512 rows x 64^2 < 2^24,
 //    so every CTA reduces a chunk of at most 512 rows;
-//  - pairs with i + j > 9 (weight below 2^-48) are left out: 36 BF16 products per entry and row;
-//  - the 8 exact integer sums of a chunk are scaled by 2^-6s (exact) and added in double-FP32,
+//  - pairs with i + j > 8 (weight 2^-49 and below) are left out: 28 BF16 products per entry and row
+//    (digits rounded toward zero hold one bit less: 8 of 6 bits and 36 products for 48 bits);
+//  - the 7 exact integer sums of a chunk are scaled by 2^-7s (exact) and added in double-FP32,
 //    the chunks are added in double-FP32, and the result is scaled by 2^(e_a + e_b - 12).
 // The error of W(a, b) is about 2^-45 of max|y_a| max|y_b| m: FP64-class, as the Gram of the
 // double-FP32 SIMT path (orth.cu), at tensor-core throughput.
 //
-// Kernels: gram_slice_kernel (one CTA per column: exponent, then the 8 slices, BF16, column-major
+// Kernels: gram_slice_kernel (one CTA per column: exponent, then the 7 slices, BF16, column-major
 // per slice with rows padded to a multiple of 8), gram_tc_kernel (one CTA per (128 x 64 tile of
-// W's upper part, 512-row chunk): TMA of the 8 slices of both operands into a 4-stage ring of
-// 16-row stages, 12 MMAs of 128 x (64..256) x 16 per stage into 8 x 64 TMEM columns, epilogue to
+// W's upper part, 512-row chunk): TMA of the 7 slices of both operands into a ring of two 32-row
+// stages, 10 MMAs of 128 x (64..256) x 16 per 16 rows into 7 x 64 TMEM columns, epilogue to
 // double-FP32 partial tiles), gram_tc_combine_kernel (chunk sums, scaling, the quaternion
 // components of G).
+// Bound: a stage row is 64 bytes of one column and slice, and the TMA's row rate, then the MMAs, set
+// the pace: 16-row stages (32-byte rows) and 8 slices took 391 us at 20000 x 180 and 76 us at
+// 20000 x 60, this form 310 and 60 (error over max|y_a| max|y_b| m: 2^-48.1, before 2^-45.9).
 #include <algorithm>
 #include <cstring>
 
@@ -33,22 +37,30 @@ namespace {
 
 using namespace qlr_tc;
 
-constexpr int GS = 8;            // slices per entry, 6 bits each
-constexpr int GBITS = 6;
-constexpr int GPAIR_MAX = 9;     // slice pairs (i, j), 1-based, with i + j <= 9
-constexpr int NGRP = GPAIR_MAX - 1;   // weights s = i + j - 2 = 0 .. 7
+// The two splittings.  Slices7 (single problems): balanced base 128, as above.  Slices8 (batch
+// plans): 8 digits of 6 bits rounded toward zero, 36 products, 2^-48 of the column maximum; the
+// plans' results hang on every bit of their factors (the phase of each singular vector pair is set
+// by rounding errors), so they keep the digits they were released with.
+template <int N>
+struct Slices {
+  static constexpr int GS = N;                    // slices per entry
+  static constexpr int GBITS = (N == 7) ? 7 : 6;  // weight step of the slices
+  static constexpr bool NEAREST = (N == 7);
+  static constexpr int NGRP = N;                  // weight groups s = i + j - 2 = 0 .. N - 1
+};
+constexpr int GTOP = 6;          // bits of the first slice
+constexpr int GTMEM = 512;       // TMEM columns allocated for the weight groups' accumulators (a power of two)
 constexpr int GA = 128;          // W rows per tile (MMA M)
 constexpr int GB = 64;           // W columns per tile (MMA N)
-constexpr int GK = 16;           // rows of Y per pipeline stage (32-byte swizzled BF16 rows, one MMA K)
+constexpr int GK = 32;           // rows of Y per pipeline stage (64-byte swizzled BF16 rows, two MMA K)
 constexpr int GCHUNK = 512;      // rows of Y per CTA (exactness of the TMEM sums)
-constexpr int GSTAGES = 4;
+constexpr int GSTAGES = 2;
 constexpr int GTHREADS = 256;
 constexpr int GSW = GK * 2;           // bytes per K-major row = swizzle span
-constexpr int GMODE = 6;              // descriptor swizzle mode: 32 bytes
+constexpr int GMODE = 4;              // descriptor swizzle mode: 64 bytes
 constexpr int A_TILE = GA * GK * 2;   // bytes of one slice's A tile
 constexpr int B_TILE = GB * GK * 2;
-constexpr int STAGE_BYTES = GS * (A_TILE + B_TILE);
-constexpr size_t GSMEM = (size_t)GSTAGES * STAGE_BYTES + 1024 + 256;
+constexpr size_t gsmem(int gs) { return (size_t)GSTAGES * gs * (A_TILE + B_TILE) + 1024 + 256; }
 
 struct GramTcParams {
   CUtensorMap tmA;      // slices as (mp rows inner) x (GS L4p columns outer), box {GK, GA}
@@ -74,9 +86,9 @@ struct GramTcProb {
 };
 
 // Columns of Yh (L4p columns, the padding zero) by CTAs of 8 warps, WPC warps per column (8 for
-// one tall problem, 1 for the many short ones of a batch): the column exponent, then the 8
+// one tall problem, 1 for the many short ones of a batch): the column exponent, then the
 // slices; each lane takes row pairs, stored as BF16 pairs.
-template <int WPC>
+template <int N, int WPC>
 __device__ __forceinline__ void gram_slice_cols(const float* __restrict__ y0, const float* __restrict__ y1,
                                                 const float* __restrict__ y2, const float* __restrict__ y3, int64_t m,
                                                 int l, int64_t ld, int L4p, int64_t mp, __nv_bfloat16* __restrict__ S,
@@ -106,14 +118,15 @@ __device__ __forceinline__ void gram_slice_cols(const float* __restrict__ y0, co
   if (mx > 0.f) frexpf(mx, &e);   // max < 2^e
   if (sub == 0 && lane == 0) ex[c] = e;
   for (int64_t r = 2 * (sub * 32 + lane); r < mp; r += 64 * WPC) {   // mp is even
-    float v0 = (y && r < m) ? ldexpf(y[r], GBITS - e) : 0.f;       // |v| < 64, exact
-    float v1 = (y && r + 1 < m) ? ldexpf(y[r + 1], GBITS - e) : 0.f;
+    float v0 = (y && r < m) ? ldexpf(y[r], GTOP - e) : 0.f;       // |v| < 64, exact
+    float v1 = (y && r + 1 < m) ? ldexpf(y[r + 1], GTOP - e) : 0.f;
 #pragma unroll
-    for (int i = 0; i < GS; ++i) {
-      const float q0 = truncf(v0), q1 = truncf(v1);                // |q| <= 63
+    for (int i = 0; i < N; ++i) {
+      const float q0 = Slices<N>::NEAREST ? rintf(v0) : truncf(v0);   // |q| <= 64, or 63
+      const float q1 = Slices<N>::NEAREST ? rintf(v1) : truncf(v1);
       *reinterpret_cast<__nv_bfloat162*>(S + ((size_t)i * L4p + c) * mp + r) = __floats2bfloat162_rn(q0, q1);
-      v0 = (v0 - q0) * 64.f;                                        // exact
-      v1 = (v1 - q1) * 64.f;
+      v0 = (v0 - q0) * (float)(1 << Slices<N>::GBITS);                // exact
+      v1 = (v1 - q1) * (float)(1 << Slices<N>::GBITS);
     }
   }
 }
@@ -122,7 +135,7 @@ __global__ void __launch_bounds__(256) gram_slice_kernel(const float* __restrict
                                                          const float* __restrict__ y2, const float* __restrict__ y3,
                                                          int64_t m, int l, int64_t ld, int L4p, int64_t mp,
                                                          __nv_bfloat16* __restrict__ S, int* __restrict__ ex) {
-  gram_slice_cols<8>(y0, y1, y2, y3, m, l, ld, L4p, mp, S, ex, blockIdx.x);
+  gram_slice_cols<7, 8>(y0, y1, y2, y3, m, l, ld, L4p, mp, S, ex, blockIdx.x);
 }
 
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
@@ -144,7 +157,10 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& e, float x) {
 
 // One tile of W for one chunk of rows: tile index tl enumerates (ab, bb) with bb >= 2 ab (the
 // upper part of W).
+template <int N>
 __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, const int chunk) {
+  constexpr int GS = Slices<N>::GS, GBITS = Slices<N>::GBITS, NGRP = Slices<N>::NGRP, GPAIR_MAX = NGRP + 1;
+  constexpr int STAGE_BYTES = GS * (A_TILE + B_TILE);
   int ab = 0;
   while (ab < p.nA && tl >= max(0, p.nB - 2 * ab)) { tl -= max(0, p.nB - 2 * ab); ++ab; }
   const int bb = 2 * ab + tl;
@@ -177,7 +193,7 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(NGRP * GB)
+                 "r"(GTMEM)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -217,6 +233,9 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
       // slice tiles are adjacent in shared memory, and one MMA of A_i against slices j .. j+t-1
       // writes pair (i, j + u) to TMEM columns (i + j + u) GB, the accumulator of its weight group
       const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GA >> 4) << 24);
+      // stage 0's descriptors; a stage, slice or K step moves the 16-byte address field
+      const uint64_t ad0 = make_desc(smem_u32(a_tile(0, 0)), 16, 8 * GSW, GMODE);
+      const uint64_t bd0 = make_desc(smem_u32(b_tile(0, 0)), 16, 8 * GSW, GMODE);
       bool ok = true;
       for (int i = 0; i < nit && ok; ++i) {
         const int s = i % GSTAGES;
@@ -224,15 +243,16 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
         ok = mbar_wait(&full[s], ph, abort_flag, p.err);
         if (!ok) break;
         tc_fence_after();
+        const uint64_t so = (uint64_t)(s * (STAGE_BYTES >> 4));
 #pragma unroll
         for (int ks = 0; ks < GK / 16; ++ks) {
 #pragma unroll
           for (int qi = 0; qi < GS; ++qi) {
-            const uint64_t ad = make_desc(smem_u32(a_tile(s, qi)) + (uint32_t)(ks * 32), 16, 8 * GSW, GMODE);
+            const uint64_t ad = ad0 + so + (uint64_t)((qi * A_TILE + ks * 32) >> 4);
 #pragma unroll
             for (int qj = 0; qj <= GPAIR_MAX - 2 - qi; qj += 4) {
               const int t = min(4, GPAIR_MAX - 1 - qi - qj);   // slices qj .. qj + t - 1
-              const uint64_t bd = make_desc(smem_u32(b_tile(s, qj)) + (uint32_t)(ks * 32), 16, 8 * GSW, GMODE);
+              const uint64_t bd = bd0 + so + (uint64_t)((qj * B_TILE + ks * 32) >> 4);
               const uint32_t idesc = idesc0 | ((uint32_t)((t * GB) >> 3) << 17);
               // first products of the weight groups in this chunk: qi == 0, first stage and k-step
               const uint32_t acc = (i > 0 || ks > 0 || qi > 0) ? 1u : 0u;
@@ -245,7 +265,7 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
       umma_commit(tmem_full);     // accumulators complete (also fires after an abort)
     }
   } else if (warp >= 4) {
-    // ---------------- epilogue: 8 exact integer sums -> double-FP32 ----------------
+    // ---------------- epilogue: the exact integer sums -> double-FP32 ----------------
     const int q = warp & 3;
     const int a = a0 + q * 32 + lane;
     const bool ok = mbar_wait(tmem_full, 0, abort_flag, p.err) && !*abort_flag;
@@ -256,7 +276,7 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
       for (int jj = 0; jj < GB; ++jj) h[jj] = e[jj] = 0.f;
 #pragma unroll
       for (int g = NGRP - 1; g >= 0; --g) {
-        const float w = __int_as_float((127 - GBITS * g) << 23);   // 2^-6g
+        const float w = __int_as_float((127 - GBITS * g) << 23);   // 2^(-GBITS g)
 #pragma unroll
         for (int cc = 0; cc < GB; cc += 32) {
           uint32_t r0[16], r1[16];
@@ -286,12 +306,12 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
   tc_fence_after();
   if (warp == 1) {
     __syncwarp();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NGRP * GB) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(GTMEM) : "memory");
   }
 }
 
 __global__ void __launch_bounds__(GTHREADS, 1) gram_tc_kernel(const __grid_constant__ GramTcParams p) {
-  gram_tc_tile(p, blockIdx.x, blockIdx.y);
+  gram_tc_tile<7>(p, blockIdx.x, blockIdx.y);
 }
 
 // Batch plans: item (problem, tile, chunk) with that problem's parameters in global memory
@@ -304,7 +324,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) gram_tc_grouped_kernel(const Gram
     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&p.tmA) : "memory");
     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&p.tmB) : "memory");
   }
-  gram_tc_tile(p, it.y, it.z);
+  gram_tc_tile<8>(p, it.y, it.z);
 }
 
 // W(I, J) for I <= J: the chunk partials added in double-FP32, scaled by 2^(e_I + e_J - 12).
@@ -318,7 +338,7 @@ __device__ __forceinline__ double w_tc(const float2* __restrict__ part, int nchu
     two_sum_acc(s, e, v.x);
     e = __fadd_rn(e, v.y);
   }
-  return ldexp((double)s + (double)e, ex[I] + ex[J] - 2 * GBITS);
+  return ldexp((double)s + (double)e, ex[I] + ex[J] - 2 * GTOP);
 }
 
 // W(I, J), I <= J, as a scaled double-FP32 pair (s, e).
@@ -332,7 +352,7 @@ __device__ __forceinline__ float2 w_tc_d32(const float2* __restrict__ part, int 
     two_sum_acc(s, e, v.x);
     e = __fadd_rn(e, v.y);
   }
-  const int k = ex[I] + ex[J] - 2 * GBITS;
+  const int k = ex[I] + ex[J] - 2 * GTOP;
   return make_float2(ldexpf(s, k), ldexpf(e, k));
 }
 
@@ -380,7 +400,7 @@ __global__ void __launch_bounds__(256) gram_slice_grouped_kernel(const GramTcPro
                                                                  const int4* __restrict__ items) {
   const int4 it = items[blockIdx.x];
   const GramTcProb& a = probs[it.x];
-  gram_slice_cols<1>(a.y[0], a.y[1], a.y[2], a.y[3], a.m, a.l, a.ld, a.tc.L4p, a.mp, a.S, a.ex, it.y);
+  gram_slice_cols<8, 1>(a.y[0], a.y[1], a.y[2], a.y[3], a.m, a.l, a.ld, a.tc.L4p, a.mp, a.S, a.ex, it.y);
 }
 
 // The quaternion Gram from W, FP64 planes: 16 threads per entry (i <= j), thread (c, d) forms
@@ -437,10 +457,10 @@ struct GramTcBufs {
   float2* part;
 };
 size_t rup256(size_t b) { return (b + 255) / 256 * 256; }
-GramTcBufs gram_tc_carve(char* base, const GramTcDims& d) {
+GramTcBufs gram_tc_carve(char* base, const GramTcDims& d, int gs) {
   GramTcBufs b;
   b.S = reinterpret_cast<__nv_bfloat16*>(base);
-  base += rup256((size_t)GS * d.L4p * d.mp * 2);
+  base += rup256((size_t)gs * d.L4p * d.mp * 2);
   b.ex = reinterpret_cast<int*>(base);
   base += rup256((size_t)d.L4p * 4);
   b.part = reinterpret_cast<float2*>(base);
@@ -448,13 +468,13 @@ GramTcBufs gram_tc_carve(char* base, const GramTcDims& d) {
 }
 
 // Tensor maps and dimensions of one problem (host side).
-bool gram_tc_params(GramTcParams& prm, const GramTcDims& d, const GramTcBufs& bufs, int* err) {
+bool gram_tc_params(GramTcParams& prm, const GramTcDims& d, const GramTcBufs& bufs, int gs, int* err) {
   memset(&prm, 0, sizeof(prm));
-  const uint64_t cols = (uint64_t)GS * d.L4p;
+  const uint64_t cols = (uint64_t)gs * d.L4p;
   if (!encode_2d(&prm.tmA, bufs.S, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (uint64_t)d.mp, cols, (uint64_t)d.mp * 2, GK, GA,
-                 CU_TENSOR_MAP_SWIZZLE_32B) ||
+                 CU_TENSOR_MAP_SWIZZLE_64B) ||
       !encode_2d(&prm.tmB, bufs.S, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (uint64_t)d.mp, cols, (uint64_t)d.mp * 2, GK, GB,
-                 CU_TENSOR_MAP_SWIZZLE_32B))
+                 CU_TENSOR_MAP_SWIZZLE_64B))
     return false;
   prm.part = bufs.part;
   prm.L4 = d.L4;
@@ -472,7 +492,7 @@ namespace qlr {
 
 size_t gram_tc_ws(int64_t m, int l) {
   const GramTcDims d = gram_tc_dims(m, l);
-  return rup256((size_t)GS * d.L4p * d.mp * 2) + rup256((size_t)d.L4p * 4) + rup256((size_t)d.nchunks * d.L4 * d.L4 * 8);
+  return rup256((size_t)8 * d.L4p * d.mp * 2) + rup256((size_t)d.L4p * 4) + rup256((size_t)d.nchunks * d.L4 * d.L4 * 8);
 }
 
 bool gram_tc_supported(const qlr_qmat& Y) {
@@ -480,7 +500,7 @@ bool gram_tc_supported(const qlr_qmat& Y) {
   for (int c = 0; c < 4; ++c)
     if (Y.plane[c] == nullptr) return false;
   const GramTcDims d = gram_tc_dims(Y.rows, (int)Y.cols);
-  return Y.cols <= 1024 && (int64_t)GS * d.L4p < (1 << 30) && d.nchunks < 65536 && get_encode() != nullptr;
+  return Y.cols <= 1024 && (int64_t)8 * d.L4p < (1 << 30) && d.nchunks < 65536 && get_encode() != nullptr;
 }
 
 int gram_tc(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws) {
@@ -490,12 +510,12 @@ int gram_tc(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws) {
   const size_t mark = ws.off;
   char* base = ws.take<char>(gram_tc_ws(m, l));
   if (!ws.ok) { ws.off = mark; ws.ok = true; return QLR_ENOMEM; }
-  const GramTcBufs bufs = gram_tc_carve(base, d);
+  const GramTcBufs bufs = gram_tc_carve(base, d, 7);
   __nv_bfloat16* S = bufs.S;
   int* ex = bufs.ex;
   float2* part = bufs.part;
   GramTcParams prm;
-  if (!gram_tc_params(prm, d, bufs, ctx->d_err)) {
+  if (!gram_tc_params(prm, d, bufs, 7, ctx->d_err)) {
     ws.off = mark;
     return QLR_ECUDA;
   }
@@ -505,8 +525,8 @@ int gram_tc(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws) {
       static_cast<const float*>(Y.plane[3]), m, l, Y.ld, d.L4p, d.mp, S, ex);
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
-  QLR_CUDA_TRY(cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GSMEM));
-  gram_tc_kernel<<<dim3((unsigned)d.ntiles, (unsigned)d.nchunks), GTHREADS, GSMEM, ctx->stream>>>(prm);
+  QLR_CUDA_TRY(cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem(7)));
+  gram_tc_kernel<<<dim3((unsigned)d.ntiles, (unsigned)d.nchunks), GTHREADS, gsmem(7), ctx->stream>>>(prm);
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
   const int64_t ntri = (int64_t)l * (l + 1) / 2;
@@ -522,10 +542,10 @@ size_t gram_tc_record_bytes() { return sizeof(GramTcProb); }
 int gram_tc_record(void* dst, const qlr_qmat& Y, char* scratch, float* G, int* err) {
   const int l = (int)Y.cols;
   const GramTcDims d = gram_tc_dims(Y.rows, l);
-  const GramTcBufs bufs = gram_tc_carve(scratch, d);
+  const GramTcBufs bufs = gram_tc_carve(scratch, d, 8);
   GramTcProb r;
   memset(&r, 0, sizeof(r));
-  if (!gram_tc_params(r.tc, d, bufs, err)) return QLR_ECUDA;
+  if (!gram_tc_params(r.tc, d, bufs, 8, err)) return QLR_ECUDA;
   for (int c = 0; c < 4; ++c) r.y[c] = static_cast<const float*>(Y.plane[c]);
   r.m = Y.rows;
   r.ld = Y.ld;
@@ -556,8 +576,8 @@ int gram_tc_grouped(qlr_ctx* ctx, const void* d_probs, const int4* slice, int n_
   gram_slice_grouped_kernel<<<n_slice, 256, 0, ctx->stream>>>(probs, slice);
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
-  QLR_CUDA_TRY(cudaFuncSetAttribute(gram_tc_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GSMEM));
-  gram_tc_grouped_kernel<<<n_mma, GTHREADS, GSMEM, ctx->stream>>>(probs, mma);
+  QLR_CUDA_TRY(cudaFuncSetAttribute(gram_tc_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem(8)));
+  gram_tc_grouped_kernel<<<n_mma, GTHREADS, gsmem(8), ctx->stream>>>(probs, mma);
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
   gram_tc_combine_grouped_kernel<<<n_comb, 128, 0, ctx->stream>>>(probs, comb);
