@@ -14,9 +14,13 @@
 // each quaternion singular value of R is one of the doubled singular values of chi(R).
 //
 // The right rotations make up V_W, and R = V_W diag(sigma) U_W^H: R's left singular vectors are
-// V_W, its right ones U_W.  The sweep kernel works on W alone (in shared memory when it fits) and
-// logs every rotation (c, s, mu); a second kernel replays the log on V_W = I.  The rows of V_W
-// transform independently under right rotations, so the replay runs row-parallel on many SMs.
+// V_W, its right ones U_W.  The sweeps work on W alone (in shared memory when it fits) and log every
+// rotation (c, s, mu); other CTAs replay the log on V_W = I.  The rows of V_W transform independently
+// under right rotations, so the replay runs row-parallel on many SMs, and it runs while the sweeps
+// go on: they publish how much of the log is written (Progress), and the replaying CTAs of the same
+// launch follow a block round behind (l = 180: 615 us of a launch of its own before).
+// A sweep is the last when its rotations were all so small that they cannot have left a pair above
+// the tolerance (last_sweep_threshold): the sweep that would only confirm it is not run.
 // Both vector sets are orthonormal to the working precision.  Precision: the sweeps run in T
 // (float or double); a final FP64 step evaluates every kept singular value as the two-sided
 // Rayleigh quotient sigma = Re(u^H R v) / (|u| |v|) from the FP64 R, whose error is second order
@@ -64,12 +68,50 @@ __device__ __forceinline__ void rr_pair(int lp, int r, int i, int& p, int& q) {
   }
 }
 
+// How far the log is written, for the replaying CTAs of the same launch: `count` units published
+// (release, after a barrier behind the records' stores), `done` set after the last of them.  The
+// CTA (or cluster) that sweeps has the lowest block indices and waits for nobody; a replaying CTA's
+// wait is bounded.
+struct Progress { unsigned count, done; };
+__device__ __forceinline__ void publish(unsigned* p, unsigned v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned read_published(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// Units published beyond `have` (one thread): the new count, `have` itself once the log is complete.
+__device__ inline unsigned await_progress(const Progress* pg, unsigned have, int* err) {
+  unsigned long long t0 = 0;
+  for (int it = 0;; ++it) {
+    const unsigned d = read_published(&pg->done), c = read_published(&pg->count);
+    if (c > have || d) return c;
+    if ((it & 63) == 63) {
+      unsigned long long now;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > 1500000000ull) {
+        qlr_set_error(err, QLR_ETIMEOUT);
+        return have;
+      }
+    }
+    __nanosleep(100);
+  }
+}
+
+// A sweep whose rotations all had cosine (of the pair before it) and sine at most thr leaves every
+// cosine within l thr^2: its own pair's is zero, and each of the up to l later rotations of either
+// column mixes in at most sine times cosine.  thr^2 = tol / l makes that the tolerance.
+template <class T>
+__device__ __forceinline__ T last_sweep_threshold2(T tol, int l) { return tol / (T)l; }
+
 // Reciprocal and reciprocal square root for the rotation parameters: the hardware approximations
 // in float (a few ulp; every rotation is applied to W and V, or logged and replayed, exactly as
-// computed, so the vectors stay orthonormal to the working precision), correctly rounded in
+// computed, so the vectors stay orthonormal to the working precision), the library's (1 ulp) in
 // double.
 __device__ __forceinline__ float jrsqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double jrsqrt(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double jrsqrt(double x) { return rsqrt(x); }
 __device__ __forceinline__ float jrcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double jrcp(double x) { return 1.0 / x; }
 
@@ -79,13 +121,34 @@ __device__ __forceinline__ double jrcp(double x) { return 1.0 / x; }
 // zeta = (beta - alpha) / (2 |gamma|), c = 1 / sqrt(1 + t^2), s = c t.
 template <class T>
 __device__ __forceinline__ void jacobi_rotation(T alpha, T beta, const Quat<T>& g, T gn2, Quat<T>& mu, T& c, T& s) {
-  const T ign = jrsqrt(gn2);
-  mu = {g.w * ign, g.x * ign, g.y * ign, g.z * ign};
+  T ign;
+  if (gn2 >= (sizeof(T) == 4 ? (T)1e-30 : (T)1e-290)) {
+    ign = jrsqrt(gn2);
+    mu = {g.w * ign, g.x * ign, g.y * ign, g.z * ign};
+  } else {
+    // near the subnormals the square has lost digits, and mu would not be a unit: the columns of a
+    // numerically rank-deficient core, whose accumulated rotations must stay orthonormal all the same
+    const T up = sizeof(T) == 4 ? (T)1152921504606846976.0 : (T)3.273390607896142e150;   // 2^60, 2^500
+    const Quat<T> h = {g.w * up, g.x * up, g.y * up, g.z * up};
+    const T ih = jrsqrt(qnorm2(h));
+    mu = {h.w * ih, h.x * ih, h.y * ih, h.z * ih};
+    ign = ih * up;
+  }
   const T zeta = (beta - alpha) * ((T)0.5 * ign);
   const T az = fabs(zeta);
-  const T x = (T)1 + az * az;
-  const T den = (az < (T)1e18) ? az + x * jrsqrt(x) : (T)2 * az;
-  const T tt = (zeta >= 0 ? (T)1 : (T)-1) * jrcp(den);
+  T tt;
+  if (sizeof(T) == 8 && az < (T)1e18) {
+    // the angle in FP32, c and s = c t in FP64: the rotation is unitary to FP64 whatever t is, and
+    // the pair is left at 2^-24 of its cosine, which the next sweep (or the stopping rule) covers;
+    // an FP64 square root and division each take longer than the rest of a small pair's work
+    const float zf = (float)az, xf = 1.f + zf * zf;
+    tt = (T)__fdividef(1.f, zf + xf * rsqrtf(xf));
+  } else {
+    const T x = (T)1 + az * az;
+    const T den = (az < (T)1e18) ? az + x * jrsqrt(x) : (T)2 * az;
+    tt = jrcp(den);
+  }
+  if (zeta < 0) tt = -tt;
   c = jrsqrt((T)1 + tt * tt);
   s = c * tt;
 }
@@ -106,11 +169,12 @@ __device__ __forceinline__ S rh_elem(const S* __restrict__ R, int l, size_t ll, 
 // Cyclic (round-robin) one-sided Jacobi sweeps by one CTA of JT threads on W (l x l, planes of
 // l * l, column-major), with the same right rotations applied to Vs when it is set; otherwise
 // every rotation is logged to rlog.  Returns the number of sweeps run; *converged is set when
-// the last sweep rotated no pair.
+// the last sweep left every pair within the tolerance.
 template <class T>
 __device__ int jacobi_sweeps(T* W, T* Vs, int l, int max_sweeps, T tol, T* rlog, bool* converged_out) {
   __shared__ int s_rot;
   const int t = threadIdx.x, lane = t % 32, warp = t / 32, nwarps = JT / 32;
+  const T thr2 = last_sweep_threshold2(tol, l);
   const int lp = l + (l & 1);
   int sweep = 0;
   bool converged = (l < 2);
@@ -139,10 +203,10 @@ __device__ int jacobi_sweeps(T* W, T* Vs, int l, int max_sweeps, T tol, T* rlog,
           if (lane == 0 && lg) { lg[0] = (T)1; lg[1] = (T)0; lg[2] = (T)1; lg[3] = lg[4] = lg[5] = (T)0; }
           continue;
         }
-        if (lane == 0) s_rot = 1;
         Quat<T> mu;
         T c, s;
         jacobi_rotation(a, b, g, gn2, mu, c, s);
+        if (lane == 0 && (gn2 > (thr2 * a) * b || s * s > thr2)) s_rot = 1;
         if (lane == 0 && lg) { lg[0] = c; lg[1] = s; lg[2] = mu.w; lg[3] = mu.x; lg[4] = mu.y; lg[5] = mu.z; }
         for (int i = lane; i < l; i += 32) {
           Quat<T> wp = ldw(W, l, i, p), wq = qmulc(ldw(W, l, i, q), mu);   // w_q mu*
@@ -198,6 +262,208 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(const double* __restrict__ R
   __syncthreads();
   if (w_smem)
     for (size_t e = t; e < 4 * ll; e += JT) Wout[e] = W[e];
+}
+
+// Small cores: one CTA sweeps on W in shared memory, the others replay the log.
+// Bound by one SM's issue rate (FP64: by its FP64 pipe, under two multiply-adds a cycle) and the
+// latency of a round, so: a pair per group of 16 lanes, up to RPL rows a lane held in registers
+// between the dot products and the rotation; every pair of a round at once; quaternions as one
+// 16- or 32-byte vector.  In FP64 the six dot products are reduced in transposed form (8 additions
+// a lane instead of 24).  Measured (sweeps, replay and
+// refinement, before and now): FP32 l = 40 736 and 363 us; FP64 l = 15 1144 and 447 us.
+template <class T> struct Q4;
+template <> struct Q4<float> { using V = float4; using H = float2; };
+template <> struct Q4<double> { using V = double4; using H = double2; };
+template <class T>
+__device__ __forceinline__ Quat<T> ldq(const typename Q4<T>::V* p) {
+  const typename Q4<T>::V v = *p;
+  return {v.x, v.y, v.z, v.w};
+}
+template <class T>
+__device__ __forceinline__ void stq(typename Q4<T>::V* p, T w, T x, T y, T z) {
+  typename Q4<T>::V v;
+  v.x = w; v.y = x; v.z = y; v.w = z;
+  *p = v;
+}
+
+// Sums of six values over the 16 lanes of a group, to every lane of it.
+__device__ __forceinline__ void group_sum6(float (&v)[6]) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+    for (int e = 0; e < 6; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], o);
+}
+__device__ __forceinline__ void group_sum6(double (&v)[6]) {
+  const int lane = threadIdx.x & 15;
+  const bool b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+  double a[4], b[2], c;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {   // upper half keeps values 4, 5 (and two zeros)
+    const double lo = v[e], hi = (e < 2) ? v[4 + (e & 1)] : 0.0;
+    a[e] = (b3 ? hi : lo) + __shfl_xor_sync(0xffffffffu, b3 ? lo : hi, 8);
+  }
+#pragma unroll
+  for (int e = 0; e < 2; ++e) b[e] = (b2 ? a[2 + e] : a[e]) + __shfl_xor_sync(0xffffffffu, b2 ? a[e] : a[2 + e], 4);
+  c = (b1 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, b1 ? b[0] : b[1], 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  // value e sits in the lanes with bit 3 = e / 4, bit 2 = (e / 2) % 2, bit 1 = e % 2
+#pragma unroll
+  for (int e = 0; e < 6; ++e) v[e] = __shfl_sync(0xffffffffu, c, ((e >> 2) << 3) | (((e >> 1) & 1) << 2) | ((e & 1) << 1), 16);
+}
+
+constexpr int JS_REC = 8;      // log record: c, s, mu (4), padding
+constexpr int JS_PUBLISH = 8;                 // rounds per publication
+__host__ __device__ __forceinline__ int js_threads(int l) { return ((l + 1) / 2 * 16 + 31) / 32 * 32 + 32; }
+
+template <class T, int RPL>
+__global__ void __launch_bounds__(480) jacobi_small_kernel(const double* __restrict__ R, int l, T* __restrict__ Wout,
+                                                           T* __restrict__ Vout, int max_sweeps, T tol,
+                                                           T* __restrict__ sig_out, int* __restrict__ sweeps_out,
+                                                           T* __restrict__ rlog, Progress* __restrict__ pg, int* err) {
+  using V4 = typename Q4<T>::V;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V4* W = reinterpret_cast<V4*>(smem_raw);   // W(i, j) at W[j l + i]; a replaying CTA: a row of V per warp
+  const int t = threadIdx.x, lane = t % 32, warp = t / 32, nwarps = blockDim.x / 32;
+  const int lp = l + (l & 1), np = lp / 2, rounds = lp - 1;
+  const size_t ll = (size_t)l * l;
+  if (blockIdx.x > 0) {
+    // ---------------- replay: one warp per row of V, a lane per pair of the round ----------------
+    const int row = (blockIdx.x - 1) * nwarps + warp;
+    if (row >= l) return;
+    V4* vr = W + (size_t)warp * l;
+    for (int j = lane; j < l; j += 32) stq<T>(vr + j, j == row ? (T)1 : (T)0, 0, 0, 0);
+    __syncwarp();
+    unsigned have = 0;
+    int r = 0;
+    while (true) {
+      unsigned upto = 0;
+      if (lane == 0) upto = await_progress(pg, have, err);
+      upto = __shfl_sync(0xffffffffu, upto, 0);
+      if (upto == have) break;
+      T nx[6];
+      auto fetch = [&](unsigned u) {
+        // past L1: a line may hold later records too, read here before they are written
+        using V2 = typename Q4<T>::H;
+        const V2* rec = reinterpret_cast<const V2*>(rlog + ((size_t)u * np + min(lane, np - 1)) * JS_REC);
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          const V2 a = __ldcg(rec + e);
+          nx[2 * e] = a.x;
+          nx[2 * e + 1] = a.y;
+        }
+      };
+      fetch(have);
+      for (; have < upto; ++have) {
+        T cu[6];
+#pragma unroll
+        for (int e = 0; e < 6; ++e) cu[e] = nx[e];
+        if (have + 1 < upto) fetch(have + 1);
+        int p, q;
+        rr_pair(lp, r, min(lane, np - 1), p, q);
+        if (lane < np && p < l && q < l && cu[1] != (T)0) {
+          const T c = cu[0], s = cu[1];
+          const Quat<T> vp = ldq<T>(vr + p), vq = qmulc(ldq<T>(vr + q), Quat<T>{cu[2], cu[3], cu[4], cu[5]});
+          stq<T>(vr + p, c * vp.w - s * vq.w, c * vp.x - s * vq.x, c * vp.y - s * vq.y, c * vp.z - s * vq.z);
+          stq<T>(vr + q, s * vp.w + c * vq.w, s * vp.x + c * vq.x, s * vp.y + c * vq.y, s * vp.z + c * vq.z);
+        }
+        __syncwarp();
+        if (++r == rounds) r = 0;
+      }
+    }
+    for (int j = lane; j < l; j += 32) {
+      const Quat<T> v = ldq<T>(vr + j);
+      const size_t o = (size_t)j * l + row;
+      Vout[o] = v.w; Vout[ll + o] = v.x; Vout[2 * ll + o] = v.y; Vout[3 * ll + o] = v.z;
+    }
+    return;
+  }
+  // ---------------- sweeps ----------------
+  __shared__ int s_rot;
+  for (int e = t; e < (int)ll; e += blockDim.x) {   // W = R^H
+    const size_t i = e % l, j = e / l, src = i * l + j;
+    stq<T>(W + e, (T)R[src], (T)-R[ll + src], (T)-R[2 * ll + src], (T)-R[3 * ll + src]);
+  }
+  const T thr2 = last_sweep_threshold2(tol, l), tol2 = tol * tol;
+  const bool publisher = (warp == nwarps - 1);
+  const int pi = t / 16, sub = t % 16;
+  unsigned unit = 0;
+  int sweep = 0;
+  bool converged = (l < 2);
+  for (; sweep < max_sweeps && !converged; ++sweep) {
+    if (t == 0) s_rot = 0;
+    __syncthreads();
+    for (int r = 0; r < rounds; ++r, ++unit) {
+      if (publisher) {
+        if (lane == 0 && unit > 0 && unit % JS_PUBLISH == 0) publish(&pg->count, unit);   // the rounds before this one
+      } else {
+        int p = 0, q = 0;
+        bool valid = pi < np;
+        if (valid) {
+          rr_pair(lp, r, pi, p, q);
+          valid = p < l && q < l;
+        }
+        V4* Wp = W + (size_t)p * l + sub;
+        V4* Wq = W + (size_t)q * l + sub;
+        Quat<T> wp[RPL], wq[RPL];
+        T v[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll
+        for (int u = 0; u < RPL; ++u) {
+          wp[u] = wq[u] = {0, 0, 0, 0};
+          if (valid && sub + 16 * u < l) {
+            wp[u] = ldq<T>(Wp + 16 * u);
+            wq[u] = ldq<T>(Wq + 16 * u);
+            v[0] += qnorm2(wp[u]);
+            v[1] += qnorm2(wq[u]);
+            const Quat<T> pr = qcmul(wp[u], wq[u]);
+            v[2] += pr.w; v[3] += pr.x; v[4] += pr.y; v[5] += pr.z;
+          }
+        }
+        group_sum6(v);
+        const Quat<T> g = {v[2], v[3], v[4], v[5]};
+        const T gn2 = qnorm2(g);
+        const bool rot = valid && gn2 > (tol2 * v[0]) * v[1];
+        T c = 1, s = 0;
+        Quat<T> mu = {1, 0, 0, 0};
+        if (rot) {
+          jacobi_rotation(v[0], v[1], g, gn2, mu, c, s);
+          if (sub == 0 && (gn2 > (thr2 * v[0]) * v[1] || s * s > thr2)) s_rot = 1;
+#pragma unroll
+          for (int u = 0; u < RPL; ++u) {
+            if (sub + 16 * u < l) {
+              const Quat<T> z = qmulc(wq[u], mu);   // w_q mu*
+              stq<T>(Wp + 16 * u, c * wp[u].w - s * z.w, c * wp[u].x - s * z.x, c * wp[u].y - s * z.y, c * wp[u].z - s * z.z);
+              stq<T>(Wq + 16 * u, s * wp[u].w + c * z.w, s * wp[u].x + c * z.x, s * wp[u].y + c * z.y, s * wp[u].z + c * z.z);
+            }
+          }
+        }
+        if (sub == 0 && pi < np) {
+          V4* rec = reinterpret_cast<V4*>(rlog + ((size_t)unit * np + pi) * JS_REC);
+          stq<T>(rec, c, s, mu.w, mu.x);
+          stq<T>(rec + 1, mu.y, mu.z, 0, 0);
+        }
+      }
+      __syncthreads();
+    }
+    converged = (s_rot == 0);
+    __syncthreads();
+  }
+  if (publisher && lane == 0) {
+    publish(&pg->count, unit);
+    publish(&pg->done, 1u);
+    *sweeps_out = sweep;
+    if (!converged) qlr_set_error(err, QLR_ENOCONV);
+  }
+  for (int j = warp; j < l; j += nwarps) {   // column norms -> sigma, columns normalised
+    T a = 0;
+    for (int i = lane; i < l; i += 32) a += qnorm2(ldq<T>(W + (size_t)j * l + i));
+    a = sqrt(warp_sum(a));
+    if (lane == 0) sig_out[j] = a;
+    const T inv = a > (T)0 ? (T)1 / a : (T)0;
+    for (int i = lane; i < l; i += 32) {
+      const Quat<T> w = ldq<T>(W + (size_t)j * l + i);
+      stw(Wout, l, i, j, {w.w * inv, w.x * inv, w.y * inv, w.z * inv});
+    }
+  }
 }
 
 template <class T>
@@ -425,26 +691,35 @@ __host__ __device__ __forceinline__ int jb_stages_per_sweep(int bw, int jp) { re
 __host__ __device__ __forceinline__ int jb_stage(int br, int lr, int bw) { return br == 0 ? lr : (2 * bw - 1) + (br - 1) * bw + lr; }
 
 
+template <class T>
+__device__ void jacobi_block_replay(int l, int bw, int jp, int cta, const T* __restrict__ rlog, const Progress* pg,
+                                    T* __restrict__ Vout, unsigned char* smem, int* err);
+
 // Rows per lane RPL: the two columns of a pair stay in registers between the dot products and
-// the rotation (l <= 32 RPL).
+// the rotation (l <= 32 RPL).  The first cluster of jp CTAs sweeps, the others replay.
 template <class T, int RPL, int NT>
-__global__ void __launch_bounds__(NT, 1) jacobi_block_kernel(const double* __restrict__ R, int l, int bw,
-                                                                   T* __restrict__ W, int max_sweeps, T tol,
+__global__ void __launch_bounds__(NT, 1) jacobi_block_kernel(const double* __restrict__ R, int l, int bw, int jp,
+                                                                   T* __restrict__ W, T* __restrict__ Vout,
+                                                                   int max_sweeps, T tol,
                                                                    T* __restrict__ rlog, int* __restrict__ flags,
                                                                    int* __restrict__ sweeps_out, T* __restrict__ sig_out,
-                                                                   int* err) {
+                                                                   Progress* __restrict__ pg, int* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if ((int)blockIdx.x >= jp) {   // whole clusters: no cluster barrier is left waiting
+    jacobi_block_replay<T>(l, bw, jp, (int)blockIdx.x - jp, rlog, pg, Vout, smem_raw, err);
+    return;
+  }
   T* S = reinterpret_cast<T*>(smem_raw);          // [4][2 bw][l]: plane, local column, row
   cg::cluster_group cluster = cg::this_cluster();
   const int p = (int)cluster.block_rank();
   const int t = threadIdx.x, lane = t % 32, warp = t / 32, nwarps = NT / 32;
   const size_t ll = (size_t)l * l;
-  const int JPR = (int)gridDim.x;                 // cluster size: one cluster of JPR CTAs
+  const int JPR = jp;                             // cluster size
   const int NB = 2 * JPR;
   const int U = 2 * bw;
   const int sps = jb_stages_per_sweep(bw, JPR);
   const int stage_cap = JPR * bw;
-  const T tol2 = tol * tol;
+  const T tol2 = tol * tol, thr2 = last_sweep_threshold2(tol, l);
   for (size_t e = (size_t)p * NT + t; e < 4 * ll; e += (size_t)JPR * NT) W[e] = (T)rh_elem(R, l, ll, e);
   if (p == 0)
     for (int i = t; i < max_sweeps; i += NT) flags[i] = 0;
@@ -524,10 +799,10 @@ __global__ void __launch_bounds__(NT, 1) jacobi_block_kernel(const double* __res
               if (!(gn2 > (tol2 * aa) * bb2)) {
                 if (lane == 0) { lg[0] = (T)ga; lg[1] = (T)gb; lg[2] = (T)1; lg[3] = (T)0; }
               } else {
-                if (lane == 0) s_rot = 1;
                 Quat<T> mu;
                 T c, sn;
                 jacobi_rotation(aa, bb2, g, gn2, mu, c, sn);
+                if (lane == 0 && (gn2 > (thr2 * aa) * bb2 || sn * sn > thr2)) s_rot = 1;
                 if (lane == 0) {
                   lg[0] = (T)ga; lg[1] = (T)gb; lg[2] = c; lg[3] = sn;
                   lg[4] = mu.w; lg[5] = mu.x; lg[6] = mu.y; lg[7] = mu.z;
@@ -598,10 +873,10 @@ __global__ void __launch_bounds__(NT, 1) jacobi_block_kernel(const double* __res
             if (lane == 0) { lg[0] = (T)ga; lg[1] = (T)gb; lg[2] = (T)1; lg[3] = (T)0; }
             continue;
           }
-          if (lane == 0) s_rot = 1;
           Quat<T> mu;
           T c, sn;
           jacobi_rotation(aa, bb2, g, gn2, mu, c, sn);
+          if (lane == 0 && (gn2 > (thr2 * aa) * bb2 || sn * sn > thr2)) s_rot = 1;
           if (lane == 0) {
             lg[0] = (T)ga; lg[1] = (T)gb; lg[2] = c; lg[3] = sn;
             lg[4] = mu.w; lg[5] = mu.x; lg[6] = mu.y; lg[7] = mu.z;
@@ -632,13 +907,16 @@ __global__ void __launch_bounds__(NT, 1) jacobi_block_kernel(const double* __res
           }
       }
       cluster.sync();   // arrive.release / wait.acquire at cluster scope: W's columns visible to all CTAs
+      // the block round's records are complete (one of the warps that the cross rounds need least)
+      if (p == JPR - 1 && t == NT - 32) publish(&pg->count, (unsigned)(sweep * sps + jb_stage(br + 1, 0, bw)));
     }
     if (t == 0 && s_rot) atomicOr(&flags[sweep], 1);
     cluster.sync();
     converged = (*(volatile int*)&flags[sweep] == 0);
     cluster.sync();
   }
-  if (p == 0 && t == 0) {
+  if (p == JPR - 1 && t == NT - 32) {
+    publish(&pg->done, 1u);
     *sweeps_out = sweep;
     if (!converged) qlr_set_error(err, QLR_ENOCONV);
   }
@@ -656,7 +934,7 @@ __global__ void __launch_bounds__(NT, 1) jacobi_block_kernel(const double* __res
 }
 
 // Replay of the staged rotation log on V = I, one warp per row of V.  The log is read in chunks
-// of RCH stages that the CTA's four warps share: each chunk is copied to shared memory with
+// of RCH stages that the CTA's warps share: each chunk is copied to shared memory with
 // cp.async while the previous one is applied.
 constexpr int RCH = 8;
 
@@ -679,87 +957,95 @@ __device__ __forceinline__ void ld_rec<float>(const float* r, float (&v)[REC]) {
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 
-size_t jb_replay_smem(int l, int bw, int jp, size_t esz) {
-  return (size_t)2 * RCH * jp * bw * REC * esz + (size_t)4 * 4 * l * esz;
+size_t jb_replay_smem(int l, int bw, int jp, size_t esz, int nwarps) {
+  return (size_t)2 * RCH * jp * bw * REC * esz + (size_t)nwarps * 4 * l * esz;
 }
 
 template <class T>
-__global__ void __launch_bounds__(128) jacobi_block_replay_kernel(int l, int bw, int jp, const T* __restrict__ rlog,
-                                                                   const int* __restrict__ nsweeps, T* __restrict__ Vout) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+__device__ void jacobi_block_replay(int l, int bw, int jp, int cta, const T* __restrict__ rlog, const Progress* pg,
+                                    T* __restrict__ Vout, unsigned char* smem, int* err) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, nwarps = blockDim.x / 32;
+  const int row = cta * nwarps + warp;
+  if (cta * nwarps >= l) return;                                  // a CTA without rows
   const int cap = jp * bw;
   const size_t stage_elems = (size_t)cap * REC;
-  T* logbuf = reinterpret_cast<T*>(smem_raw);                    // [2][RCH][cap][REC]
+  T* logbuf = reinterpret_cast<T*>(smem);                         // [2][RCH][cap][REC]
   T* vr = logbuf + 2 * RCH * stage_elems + (size_t)warp * 4 * l;  // this warp's row of V, 4 planes
-  const int row = blockIdx.x * 4 + warp;
   const bool active = row < l;
   if (active)
     for (int j = lane; j < l; j += 32) {
       vr[j] = (j == row) ? (T)1 : (T)0;
       vr[l + j] = vr[2 * l + j] = vr[3 * l + j] = (T)0;
     }
-  const size_t nst = (size_t)(*nsweeps) * jb_stages_per_sweep(bw, jp);
-  const size_t nchunks = (nst + RCH - 1) / RCH;
-  auto stage_chunk = [&](size_t ch) {
-    const size_t s0 = ch * RCH;
-    const size_t ns = (nst - s0 < (size_t)RCH) ? nst - s0 : (size_t)RCH;
-    const size_t bytes = ns * stage_elems * sizeof(T);
-    const char* src = reinterpret_cast<const char*>(rlog + s0 * stage_elems);
-    char* dst = reinterpret_cast<char*>(logbuf + (ch & 1) * RCH * stage_elems);
-    for (size_t o = (size_t)threadIdx.x * 16; o < bytes; o += (size_t)blockDim.x * 16) cp_async16(dst + o, src + o);
-    cp_async_commit();
-  };
-  if (nchunks > 0) stage_chunk(0);
-  for (size_t ch = 0; ch < nchunks; ++ch) {
-    if (ch + 1 < nchunks) {
-      stage_chunk(ch + 1);     // fills the other buffer, released by the barrier that ended chunk ch - 1
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
-    }
+  __shared__ unsigned s_upto;
+  unsigned have = 0;
+  while (true) {
+    if (threadIdx.x == 0) s_upto = await_progress(pg, have, err);
     __syncthreads();
-    const T* lb = logbuf + (ch & 1) * RCH * stage_elems;
-    const int ns = (int)((nst - ch * RCH < (size_t)RCH) ? nst - ch * RCH : (size_t)RCH);
-    if (active) {
-      for (int st = 0; st < ns; ++st) {
-        // two records per lane and iteration, loaded and applied side by side (a stage's pairs are
-        // disjoint, so the two rotations touch different entries of the row)
-        for (int k0 = 0; k0 < cap; k0 += 64) {
-          T r[2][REC];
-          int pp[2], qq[2];
-          bool on[2];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int k = k0 + 32 * h + lane;
-            if (k < cap) ld_rec(lb + ((size_t)st * cap + k) * REC, r[h]);
-            else r[h][3] = (T)0;
-            on[h] = (r[h][3] != (T)0);
-            pp[h] = on[h] ? (int)r[h][0] : 0;
-            qq[h] = on[h] ? (int)r[h][1] : 0;
-          }
-          Quat<T> vp[2], vq[2];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            vp[h] = {vr[pp[h]], vr[l + pp[h]], vr[2 * l + pp[h]], vr[3 * l + pp[h]]};
-            vq[h] = {vr[qq[h]], vr[l + qq[h]], vr[2 * l + qq[h]], vr[3 * l + qq[h]]};
-          }
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            if (!on[h]) continue;
-            const T c = r[h][2], sn = r[h][3];
-            const Quat<T> q = qmulc(vq[h], Quat<T>{r[h][4], r[h][5], r[h][6], r[h][7]});
-            const int a = pp[h], b = qq[h];
-            vr[a] = c * vp[h].w - sn * q.w; vr[l + a] = c * vp[h].x - sn * q.x; vr[2 * l + a] = c * vp[h].y - sn * q.y;
-            vr[3 * l + a] = c * vp[h].z - sn * q.z;
-            vr[b] = sn * vp[h].w + c * q.w; vr[l + b] = sn * vp[h].x + c * q.x; vr[2 * l + b] = sn * vp[h].y + c * q.y;
-            vr[3 * l + b] = sn * vp[h].z + c * q.z;
-          }
-        }
-        __syncwarp();
+    const unsigned upto = s_upto;
+    if (upto == have) break;
+    const int nchunks = (int)((upto - have + RCH - 1) / RCH);
+    auto stage_chunk = [&](int ch) {
+      const size_t s0 = have + (size_t)ch * RCH;
+      const size_t ns = (upto - s0 < (size_t)RCH) ? upto - s0 : (size_t)RCH;
+      const size_t bytes = ns * stage_elems * sizeof(T);
+      const char* src = reinterpret_cast<const char*>(rlog + s0 * stage_elems);
+      char* dst = reinterpret_cast<char*>(logbuf + (ch & 1) * RCH * stage_elems);
+      for (size_t o = (size_t)threadIdx.x * 16; o < bytes; o += (size_t)blockDim.x * 16) cp_async16(dst + o, src + o);
+      cp_async_commit();
+    };
+    stage_chunk(0);
+    for (int ch = 0; ch < nchunks; ++ch) {
+      if (ch + 1 < nchunks) {
+        stage_chunk(ch + 1);     // fills the other buffer, released by the barrier that ended chunk ch - 1
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
       }
+      __syncthreads();
+      const T* lb = logbuf + (ch & 1) * RCH * stage_elems;
+      const int ns = (int)min((unsigned)RCH, upto - have - (unsigned)(ch * RCH));
+      if (active) {
+        for (int st = 0; st < ns; ++st) {
+          // two records per lane and iteration, loaded and applied side by side (a stage's pairs are
+          // disjoint, so the two rotations touch different entries of the row)
+          for (int k0 = 0; k0 < cap; k0 += 64) {
+            T r[2][REC];
+            int pp[2], qq[2];
+            bool on[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int k = k0 + 32 * h + lane;
+              if (k < cap) ld_rec(lb + ((size_t)st * cap + k) * REC, r[h]);
+              else r[h][3] = (T)0;
+              on[h] = (r[h][3] != (T)0);
+              pp[h] = on[h] ? (int)r[h][0] : 0;
+              qq[h] = on[h] ? (int)r[h][1] : 0;
+            }
+            Quat<T> vp[2], vq[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              vp[h] = {vr[pp[h]], vr[l + pp[h]], vr[2 * l + pp[h]], vr[3 * l + pp[h]]};
+              vq[h] = {vr[qq[h]], vr[l + qq[h]], vr[2 * l + qq[h]], vr[3 * l + qq[h]]};
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              if (!on[h]) continue;
+              const T c = r[h][2], sn = r[h][3];
+              const Quat<T> q = qmulc(vq[h], Quat<T>{r[h][4], r[h][5], r[h][6], r[h][7]});
+              const int a = pp[h], b = qq[h];
+              vr[a] = c * vp[h].w - sn * q.w; vr[l + a] = c * vp[h].x - sn * q.x; vr[2 * l + a] = c * vp[h].y - sn * q.y;
+              vr[3 * l + a] = c * vp[h].z - sn * q.z;
+              vr[b] = sn * vp[h].w + c * q.w; vr[l + b] = sn * vp[h].x + c * q.x; vr[2 * l + b] = sn * vp[h].y + c * q.y;
+              vr[3 * l + b] = sn * vp[h].z + c * q.z;
+            }
+          }
+          __syncwarp();
+        }
+      }
+      __syncthreads();
     }
-    __syncthreads();
+    have = upto;
   }
   if (!active) return;
   const size_t ll = (size_t)l * l;
@@ -837,13 +1123,16 @@ __global__ void __launch_bounds__(256) refine_kernel(const double* __restrict__ 
 namespace qlr {
 
 constexpr int JMAX_SWEEPS = 30;
-constexpr int JBLOCK_MIN_L = 48;     // from this size on, the cluster block Jacobi is used
+// From this size on, the cluster block Jacobi is used; below it one CTA sweeps (jacobi_small_kernel).
+// Sweeps, replay and refinement, one CTA against the cluster: FP32 l = 48: 465 / 730 us, 56: 686 /
+// 760, 60: 750 / 773, 64: 824 / 790; FP64 l = 20: 1250 / 1372, 24: 1545 / 1518, 30: 2660 / 1610.
+constexpr int jblock_min_l(size_t esz) { return esz == 4 ? 57 : 25; }
 
 // The cluster block Jacobi holds two column blocks per CTA in shared memory and gives each replay
 // lane at most four records per stage; larger cores run the single-CTA sweep.
 static bool use_block_jacobi(int l, size_t esz) {
   const int bw = (l + 2 * JP - 1) / (2 * JP);
-  return l >= JBLOCK_MIN_L && l <= 256 && (size_t)4 * l * 2 * bw * esz <= 220 * 1024 && JP * bw <= 128;
+  return l >= jblock_min_l(esz) && l <= 256 && (size_t)4 * l * 2 * bw * esz <= 220 * 1024 && JP * bw <= 128;
 }
 
 size_t jacobi_log_floats(int l) {
@@ -853,8 +1142,25 @@ size_t jacobi_log_floats(int l) {
     blk = std::max(blk, (size_t)JMAX_SWEEPS * jb_stages_per_sweep(bw, jp) * jp * bw * REC + REC);
   }
   const int lp = l + (l & 1);
-  const size_t one = (size_t)JMAX_SWEEPS * (lp - 1) * (lp / 2) * 6 + 6;
+  const size_t one = (size_t)JMAX_SWEEPS * (lp - 1) * (lp / 2) * JS_REC + JS_REC;
   return blk > one ? blk : one;
+}
+
+// The instantiation for this l (rows per lane) and thread count, and its shared memory: the sweeping
+// CTAs' two column blocks, or the replaying CTAs' log chunks and rows.
+template <class T>
+static auto block_jacobi_kernel(int l, bool wide) {
+  if constexpr (sizeof(T) == 4)
+    if (wide)
+      return l <= 128 ? jacobi_block_kernel<T, 4, JB_THREADS_WIDE>
+             : l <= 192 ? jacobi_block_kernel<T, 6, JB_THREADS_WIDE> : jacobi_block_kernel<T, 8, JB_THREADS_WIDE>;
+  if constexpr (sizeof(T) == 8)
+    if (l <= 64) return l <= 32 ? jacobi_block_kernel<T, 1, JB_THREADS> : jacobi_block_kernel<T, 2, JB_THREADS>;
+  return l <= 128 ? jacobi_block_kernel<T, 4, JB_THREADS>
+         : l <= 192 ? jacobi_block_kernel<T, 6, JB_THREADS> : jacobi_block_kernel<T, 8, JB_THREADS>;
+}
+static size_t block_jacobi_smem(int l, int bw, int jp, size_t esz, int threads) {
+  return std::max((size_t)4 * l * 2 * bw * esz, jb_replay_smem(l, bw, jp, esz, threads / 32));
 }
 
 // Cluster size of the block Jacobi for this l: 16 when the device allows the non-portable size
@@ -869,8 +1175,8 @@ static int block_jacobi_cluster(int device, int l) {
     if (e.first == key) return e.second;
   int pick = JP;
   const int bw = (l + 2 * JP_MAX - 1) / (2 * JP_MAX);
-  auto kern = (l <= 128) ? jacobi_block_kernel<T, 4, JB_THREADS> : jacobi_block_kernel<T, 8, JB_THREADS>;
-  const size_t smem = (size_t)4 * l * 2 * bw * sizeof(T);
+  auto kern = block_jacobi_kernel<T>(l, false);
+  const size_t smem = block_jacobi_smem(l, bw, JP_MAX, sizeof(T), JB_THREADS);
   if (bw <= JB_THREADS / 32 &&
       cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
@@ -903,6 +1209,7 @@ static int core_tsvd_t(qlr_ctx* ctx, int l, const double* R, int k, double* L, d
   int* order = ws.take<int>(l);
   int* sweeps = ws.take<int>(1);
   int* flags = ws.take<int>(JMAX_SWEEPS);
+  Progress* pg = ws.take<Progress>(1);
   if (!ws.ok) return QLR_ENOMEM;
   const T eps = (sizeof(T) == 4) ? (T)5.9604645e-08 : (T)1.1102230246251565e-16;
   const T tol = (T)8 * eps * (T)sqrt((double)l);   // above the rounding noise of the dot products
@@ -910,22 +1217,21 @@ static int core_tsvd_t(qlr_ctx* ctx, int l, const double* R, int k, double* L, d
   if (blockj) {
     // FP32 sweeps spread over a 16-CTA cluster where the GPU can co-schedule one (the sweeps are
     // bound by the FMA issue of the cluster's SMs), else over 8 CTAs
-    const int jp = (sizeof(T) == 4) ? block_jacobi_cluster<T>(ctx->device, l) : JP;
+    const int jp = block_jacobi_cluster<T>(ctx->device, l);
     const int bw = (l + 2 * jp - 1) / (2 * jp);
-    const size_t smem = (size_t)4 * l * 2 * bw * sizeof(T);
     // FP32 sweeps with more than 8 pairs per local round: a warp for every pair (up to 12), so a
     // local round is one pair rotation deep (the register budget of 384 threads still holds the
     // kernel's working set without spilling)
     const bool wide = sizeof(T) == 4 && bw > JB_THREADS / 32;
-    auto kern = (l <= 128) ? jacobi_block_kernel<T, 4, JB_THREADS> : jacobi_block_kernel<T, 8, JB_THREADS>;
-    if constexpr (sizeof(T) == 4) {
-      if (wide) kern = (l <= 128) ? jacobi_block_kernel<T, 4, JB_THREADS_WIDE> : jacobi_block_kernel<T, 8, JB_THREADS_WIDE>;
-    }
+    auto kern = block_jacobi_kernel<T>(l, wide);
+    const int threads = wide ? JB_THREADS_WIDE : JB_THREADS;
+    const size_t smem = block_jacobi_smem(l, bw, jp, sizeof(T), threads);
+    const int replay = (l + threads / 32 - 1) / (threads / 32);   // CTAs with rows of V
     QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     cudaLaunchConfig_t cfg = {};
     if (jp > JP) QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    cfg.gridDim = dim3(jp, 1, 1);
-    cfg.blockDim = dim3(wide ? JB_THREADS_WIDE : JB_THREADS, 1, 1);
+    cfg.gridDim = dim3(jp * (1 + (replay + jp - 1) / jp), 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = ctx->stream;
     cudaLaunchAttribute attr[1];
@@ -937,19 +1243,23 @@ static int core_tsvd_t(qlr_ctx* ctx, int l, const double* R, int k, double* L, d
     cfg.numAttrs = 1;
     {
       KTimer kt(ctx, QLR_KID_JACOBI);
-      QLR_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, R, l, bw, W, (int)JMAX_SWEEPS, tol, rlog, flags, sweeps, sig,
+      QLR_CUDA_TRY(cudaMemsetAsync(pg, 0, sizeof(Progress), ctx->stream));
+      QLR_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, R, l, bw, jp, W, V, (int)JMAX_SWEEPS, tol, rlog, flags, sweeps, sig, pg,
                                       ctx->d_err));
       qlr_count_launch();
     }
-    {
-      KTimer kt(ctx, QLR_KID_JACOBI);
-      const size_t rs = jb_replay_smem(l, bw, jp, sizeof(T));
-      // static shared memory comes on top of the dynamic size: always opt in
-      QLR_CUDA_TRY(cudaFuncSetAttribute(jacobi_block_replay_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs));
-      jacobi_block_replay_kernel<T><<<(l + 3) / 4, 128, rs, ctx->stream>>>(l, bw, jp, rlog, sweeps, V);
-      qlr_count_launch();
-      QLR_CUDA_TRY(cudaGetLastError());
-    }
+  } else if (l < jblock_min_l(sizeof(T))) {
+    const int threads = js_threads(l), nwarps = threads / 32;
+    const size_t smem = (size_t)4 * sizeof(T) * l * std::max(l, nwarps);
+    auto kern = l <= 16 ? jacobi_small_kernel<T, 1> : l <= 32 ? jacobi_small_kernel<T, 2>
+                : l <= 48 ? jacobi_small_kernel<T, 3> : jacobi_small_kernel<T, 4>;
+    QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    KTimer kt(ctx, QLR_KID_JACOBI);
+    QLR_CUDA_TRY(cudaMemsetAsync(pg, 0, sizeof(Progress), ctx->stream));
+    kern<<<1 + (l + nwarps - 1) / nwarps, threads, smem, ctx->stream>>>(R, l, W, V, JMAX_SWEEPS, tol, sig, sweeps, rlog, pg,
+                                                                       ctx->d_err);
+    qlr_count_launch();
+    QLR_CUDA_TRY(cudaGetLastError());
   } else {
     const size_t one = ll4 * sizeof(T);
     const bool w_smem = one <= 220 * 1024;
@@ -1007,7 +1317,7 @@ int jacobi_grouped(qlr_ctx* ctx, const JacobiGroupArgs* d_args, int count, int l
 }
 
 size_t core_tsvd_ws(int l) {
-  return (size_t)2 * 4 * l * l * 8 + jacobi_log_floats(l) * 8 + (size_t)16 * l + JMAX_SWEEPS * 4 + 8 * 256;
+  return (size_t)2 * 4 * l * l * 8 + jacobi_log_floats(l) * 8 + (size_t)16 * l + JMAX_SWEEPS * 4 + 9 * 256;
 }
 
 int core_tsvd(qlr_ctx* ctx, int l, const double* R, int k, double* L, double* S, double* Rt, int prec, WsArena& ws) {
