@@ -25,7 +25,7 @@ size_t cholqr_ws_bound(int64_t rows, int64_t l, size_t esz) {
   // + the double-FP32 copies of R and the diagonal-block inverses (FP32 sketches); the Gram's
   // slices and the tall product's splits take turns
   const size_t tall = (esz == 4 && l < (1 << 20) && tall_gemm_wanted(rows, l, (int)l)) ? tall_gemm_ws(rows, l, (int)l) : 0;
-  return (size_t)12 * 32 * l * l + (size_t)8 * l * l + (size_t)4 * (rows + 4) * l * esz + (size_t)16 * l * l +
+  return (size_t)13 * 32 * l * l + (size_t)8 * l * l + (size_t)4 * (rows + 4) * l * esz + (size_t)16 * l * l +
          std::max(gram_ws_bound(rows, l), tall) + (size_t)32 * l * l + (size_t)8 * 1024 * ((l + 15) / 16) + 17 * 256;
 }
 

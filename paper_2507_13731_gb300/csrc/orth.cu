@@ -1108,10 +1108,15 @@ __global__ void __launch_bounds__(256) tri_inv_blocked_kernel(const double* __re
 // F = Phi(E - F^H F), Phi(X) = strict upper part of X plus half its (real) diagonal, a fixed point
 // reached by iterating from F = Phi(E) (the error shrinks like |E|^(n+1)).  The inverse is
 // (I + F)^{-1} = I + D with D = -F - F D (the Neumann series I - F + F^2 - ...), iterated from
-// D = 0.  Each step is a triangular product spread over all SMs -- no serial pivots.  Both
-// iterations contract with rate of order |E|, so a step whose predecessor changed no entry by
-// more than SERIES_TOL (far below the FP64 resolution of I + F) only copies its input forward.
-// The init kernel raises `use_chol` when l * max|E_ij| exceeds SERIES_MAX; the blocked Cholesky
+// D = -F.  Each step is a triangular product spread over all SMs -- no serial pivots.  Both
+// iterations contract with a rate of at most 4 l max|E|, and stop when the next step could change no
+// entry by more than SERIES_TOL (far below the FP64 resolution of I + F).
+// One cooperative launch runs everything, a barrier over its CTAs between two steps: as 16 launches
+// (most of them finding their iteration converged) the series took 206 us at l = 180 and 49 us at
+// l = 60 plus the gaps between them, now 88 and 31 (l = 40: 40 and 14).  The factors that a step multiplies are kept as
+// quaternion vectors in the accumulation type, F in both orders, so every lane reads consecutive
+// 16-byte (FP64: 32-byte) entries.
+// When l * max|E_ij| exceeds SERIES_MAX the kernel raises `use_chol` and leaves; the blocked Cholesky
 // kernels then run instead (they are predicated on that flag, so no host synchronisation is
 // needed).
 //
@@ -1122,121 +1127,223 @@ __global__ void __launch_bounds__(256) tri_inv_blocked_kernel(const double* __re
 // sketches accumulate in FP64.
 constexpr double SERIES_MAX = 5e-3;
 constexpr double SERIES_TOL = 1e-18;
-constexpr int SERIES_ITERS = 6, NEUMANN_ITERS = 7;
+constexpr int SERIES_ITERS = 6, NEUMANN_ITERS = 7;   // the first Neumann step is D = -F
 constexpr int SPLIT = 16;   // lanes per entry: sums as short per-lane chains plus a shuffle tree
 
-__global__ void series_init_kernel(const double* __restrict__ G, double* __restrict__ E, double* __restrict__ F, int l,
-                                   unsigned long long* __restrict__ emax_bits) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)l * l) return;
-  const int i = (int)(idx % l), j = (int)(idx / l);
-  Quat<double> e = ld_small(G, l, i, j);
-  if (i == j) e.w -= 1.0;
-  st_small(E, l, i, j, e);
-  Quat<double> f = {0, 0, 0, 0};
-  if (i < j) f = e;
-  else if (i == j) f.w = 0.5 * e.w;
-  st_small(F, l, i, j, f);
-  const double mx = fmax(fmax(fabs(e.w), fabs(e.x)), fmax(fabs(e.y), fabs(e.z)));
-  atomicMax(emax_bits, (unsigned long long)__double_as_longlong(mx));
-}
+struct SeriesArgs {
+  const double* G;
+  // quaternion vectors of TA, l x l each: E, the sums F^H F and F D (their entry's owner only), F by
+  // columns (two, taking turns) and by rows, D by columns
+  void *e, *s1, *s2, *fc[2], *fr, *dc[2];
+  double *R2, *R2inv;
+  unsigned* mx;                  // FP32 bits: [0] max|E|, [1 ..] each step's largest change (zeroed)
+  unsigned* arrived;             // the barrier's count (zeroed)
+  int* use_chol;
+  int* err;
+  int l;
+};
+template <class TA> struct SeriesVec;
+template <> struct SeriesVec<float> { using V = float4; };
+template <> struct SeriesVec<double> { using V = double4; };
 
-__global__ void series_decide_kernel(const unsigned long long* __restrict__ emax_bits, int l, int* use_chol) {
-  const double emax = __longlong_as_double((long long)*emax_bits);
-  *use_chol = (!(emax * l <= SERIES_MAX)) ? 1 : 0;
-}
-
-template <class TA>
-__device__ __forceinline__ Quat<TA> ld_small_as(const double* M, int l, int i, int j) {
-  const Quat<double> q = ld_small(M, l, i, j);
-  return {(TA)q.w, (TA)q.x, (TA)q.y, (TA)q.z};
-}
-
-// out(i, j) for i <= j with SPLIT threads per entry:
-//   mode 0 (series):  Phi(E - F^H F)(i, j),  (F^H F)_ij = sum_{t <= i} conj(F_ti) F_tj
-//   mode 1 (Neumann): (-F - F D)_ij,          (F D)_ij  = sum_{i <= t <= j} F_it D_tj
-// The largest change against the step's
-// input (F in mode 0, D in mode 1) goes to *delta; when the previous step's change *prev_delta is
-// at most SERIES_TOL the input is copied unchanged.  `add_identity` stores I + out (the last
-// Neumann step writes R2^{-1} = I + D).
-template <class TA>
-__global__ void __launch_bounds__(128) series_step_kernel(const double* __restrict__ E, const double* __restrict__ F,
-                                                           const double* __restrict__ D, double* __restrict__ out, int l,
-                                                           int mode, int nentries, int add_identity,
-                                                           const unsigned long long* __restrict__ prev_delta,
-                                                           unsigned long long* __restrict__ delta) {
-  const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t ent = gt / SPLIT;
-  const int part = (int)(gt % SPLIT);
-  const bool valid = ent < nentries;
-  const double* in = (mode == 0) ? F : D;
-  int i = 0, j = 0;
-  if (valid) {
-    const int2 ij = upper_tri_entry((int)ent);
-    i = ij.x;
-    j = ij.y;
-  }
-  if (prev_delta && __longlong_as_double((long long)*prev_delta) <= SERIES_TOL) {
-    if (valid && part == 0) {
-      Quat<double> o = ld_small(in, l, i, j);
-      if (add_identity && i == j) o.w += 1.0;
-      st_small(out, l, i, j, o);
-    }
-    return;
-  }
-  Quat<TA> acc = {0, 0, 0, 0};
-  if (valid) {
-    if (mode == 0) {
-#pragma unroll 4
-      for (int t = part; t <= i; t += SPLIT) {
-        Quat<TA> pr = qcmul(ld_small_as<TA>(F, l, t, i), ld_small_as<TA>(F, l, t, j));
-        acc.w += pr.w; acc.x += pr.x; acc.y += pr.y; acc.z += pr.z;
-      }
-    } else {
-#pragma unroll 4
-      for (int t = i + part; t <= j; t += SPLIT) {
-        Quat<TA> pr = qmul(ld_small_as<TA>(F, l, i, t), ld_small_as<TA>(D, l, t, j));
-        acc.w += pr.w; acc.x += pr.x; acc.y += pr.y; acc.z += pr.z;
+// Barrier number k over the grid (its CTAs are co-resident: a cooperative launch); false when the
+// bounded wait gave up.
+__device__ inline bool series_barrier(const SeriesArgs& a, unsigned k) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ok = 1;
+    __threadfence();
+    atomicAdd(a.arrived, 1u);
+    const unsigned want = (k + 1) * gridDim.x;
+    unsigned long long t0 = 0;
+    for (int it = 0;; ++it) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.arrived) : "memory");
+      if (v >= want) break;
+      if ((it & 255) == 255) {
+        unsigned long long now;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+        if (t0 == 0) t0 = now;
+        else if (now - t0 > 1500000000ull) {
+          qlr_set_error(a.err, QLR_ETIMEOUT);
+          ok = 0;
+          break;
+        }
       }
     }
+    __threadfence();
   }
-#pragma unroll
-  for (int o = SPLIT / 2; o > 0; o >>= 1) {
-    acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
-    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-    acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
-  }
-  double ch = 0.0;
-  if (valid && part == 0) {
-    Quat<double> r;
-    if (mode == 0) {
-      const Quat<double> e = ld_small(E, l, i, j);
-      if (i < j) r = {e.w - (double)acc.w, e.x - (double)acc.x, e.y - (double)acc.y, e.z - (double)acc.z};
-      else r = {0.5 * (e.w - (double)acc.w), 0.0, 0.0, 0.0};
-    } else {
-      const Quat<double> f = ld_small(F, l, i, j);
-      r = {-f.w - (double)acc.w, -f.x - (double)acc.x, -f.y - (double)acc.y, -f.z - (double)acc.z};
-    }
-    const Quat<double> o = ld_small(in, l, i, j);
-    ch = fmax(fmax(fabs(r.w - o.w), fabs(r.x - o.x)), fmax(fabs(r.y - o.y), fabs(r.z - o.z)));
-    if (add_identity && i == j) r.w += 1.0;
-    st_small(out, l, i, j, r);
-  }
-  // warp maximum, one atomic per warp (non-negative doubles order like their bit patterns)
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) ch = fmax(ch, __shfl_xor_sync(0xffffffffu, ch, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(delta, (unsigned long long)__double_as_longlong(ch));
+  __syncthreads();
+  return ok != 0;
 }
 
-// R2 = I + F (full matrix written; lower part zero)
-__global__ void series_form_kernel(const double* __restrict__ F, double* __restrict__ R2, int l) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)l * l) return;
-  const int i = (int)(idx % l), j = (int)(idx / l);
-  Quat<double> f = (i <= j) ? ld_small(F, l, i, j) : Quat<double>{0, 0, 0, 0};
-  if (i == j) f.w += 1.0;
-  st_small(R2, l, i, j, f);
+// CTAs of 256 threads for small l (few arrivals a barrier), of 1024 where that leaves an SM more than
+// two entries a group (l = 180: 128 us with 256).
+constexpr int SERIES_THREADS = 1024;
+template <class TA>
+__global__ void __launch_bounds__(SERIES_THREADS) series_kernel(const SeriesArgs a) {
+  using V = typename SeriesVec<TA>::V;
+  const int l = a.l, nent = l * (l + 1) / 2;
+  const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+  const int part = threadIdx.x % SPLIT;
+  V* ev = static_cast<V*>(a.e);
+  V* s1 = static_cast<V*>(a.s1);
+  V* s2 = static_cast<V*>(a.s2);
+  V* fr = static_cast<V*>(a.fr);
+  unsigned bar = 0;
+  auto raise = [&](unsigned* m, float v) {   // the warp's largest value, one atomic
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(m, __float_as_uint(v));
+  };
+  auto largest = [&](const unsigned* m) { return __uint_as_float(__ldcg(m)); };
+  auto vec = [](TA w, TA x, TA y, TA z) {
+    V v;
+    v.x = w; v.y = x; v.z = y; v.w = z;
+    return v;
+  };
+  auto ldc = [](const V* p) {   // written by other CTAs of this launch: past L1
+    Quat<TA> q;
+    if constexpr (sizeof(TA) == 4) {
+      const float4 v = __ldcg(p);
+      q = {v.x, v.y, v.z, v.w};
+    } else {
+      const double2 u = __ldcg(reinterpret_cast<const double2*>(p)), w = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+      q = {u.x, u.y, w.x, w.y};
+    }
+    return q;
+  };
+  // E and F = Phi(E); an entry belongs to the first lane of its group of SPLIT
+  float mx = 0.f;
+  for (int64_t x = gt / SPLIT; x < nent; x += nt / SPLIT) {
+    if (part != 0) continue;
+    const int2 ij = upper_tri_entry((int)x);
+    const size_t o = (size_t)ij.y * l + ij.x;
+    Quat<double> e = ld_small(a.G, l, ij.x, ij.y);
+    if (ij.x == ij.y) e.w -= 1.0;
+    const V v = vec((TA)e.w, (TA)e.x, (TA)e.y, (TA)e.z);
+    ev[o] = v;
+    s1[o] = s2[o] = vec(0, 0, 0, 0);
+    static_cast<V*>(a.fc[0])[o] = (ij.x == ij.y) ? vec((TA)0.5 * v.x, 0, 0, 0) : v;
+    const float m4 = fmaxf(fmaxf(fabsf((float)v.x), fabsf((float)v.y)), fmaxf(fabsf((float)v.z), fabsf((float)v.w)));
+    mx = (m4 <= mx) ? mx : m4;   // a NaN stays
+  }
+  raise(a.mx, isnan(mx) ? INFINITY : mx);
+  if (!series_barrier(a, bar++)) return;
+  const float emax = largest(a.mx);
+  const bool chol = !((double)emax * l <= SERIES_MAX);
+  if (gt == 0) *a.use_chol = chol ? 1 : 0;
+  if (chol) return;
+  // a step's change times this bounds the next one's
+  const float rate = 4.f * (float)l * emax;
+  // One step: sum(i, j) by the entry's lanes, kept in `prev` by its owner, who writes next(i, j, sum);
+  // the largest change of a sum goes to m.
+  auto step = [&](unsigned* m, V* prev, auto sum, auto next) {
+    float ch = 0.f;
+    for (int64_t x = gt / SPLIT; x < (int64_t)(nent + 1) / 2 * 2; x += nt / SPLIT) {   // whole warps: two entries each
+      const bool valid = x < nent;
+      const int2 ij = upper_tri_entry(valid ? (int)x : 0);
+      Quat<TA> acc = {0, 0, 0, 0};
+      if (valid) acc = sum(ij.x, ij.y);
+#pragma unroll
+      for (int o = SPLIT / 2; o > 0; o >>= 1) {
+        acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
+      }
+      if (valid && part == 0) {
+        V* p = prev + (size_t)ij.y * l + ij.x;
+        const V old = *p;
+        *p = vec(acc.w, acc.x, acc.y, acc.z);
+        ch = fmaxf(ch, fmaxf(fmaxf((float)fabs(acc.w - old.x), (float)fabs(acc.x - old.y)),
+                             fmaxf((float)fabs(acc.y - old.z), (float)fabs(acc.z - old.w))));
+        next(ij.x, ij.y, acc);
+      }
+    }
+    raise(m, ch);
+  };
+  auto phi = [&](int i, int j, const Quat<TA>& s) {   // Phi(E - s)(i, j)
+    const V e = ev[(size_t)j * l + i];
+    return (i == j) ? vec((TA)0.5 * (e.x - s.w), 0, 0, 0) : vec(e.x - s.w, e.y - s.x, e.z - s.y, e.w - s.z);
+  };
+  // F <- Phi(E - F^H F), (F^H F)_ij = sum_{t <= i} conj(F_ti) F_tj
+  int cur = 0;
+  unsigned* m = a.mx + 1;
+  for (int it = 0; it < SERIES_ITERS; ++it, ++m) {
+    const V* F = static_cast<V*>(cur ? a.fc[1] : a.fc[0]);
+    V* Fn = static_cast<V*>(cur ? a.fc[0] : a.fc[1]);
+    step(m, s1,
+         [&](int i, int j) {
+           Quat<TA> acc = {0, 0, 0, 0};
+#pragma unroll 4
+           for (int t = part; t <= i; t += SPLIT) {
+             const Quat<TA> pr = qcmul(ldc(F + (size_t)i * l + t), ldc(F + (size_t)j * l + t));
+             acc.w += pr.w; acc.x += pr.x; acc.y += pr.y; acc.z += pr.z;
+           }
+           return acc;
+         },
+         [&](int i, int j, const Quat<TA>& s) { Fn[(size_t)j * l + i] = phi(i, j, s); });
+    cur ^= 1;
+    if (!series_barrier(a, bar++)) return;
+    if ((double)largest(m) * rate <= SERIES_TOL) break;
+  }
+  // D = -F, F by rows; then D <- -F - F D, (F D)_ij = sum_{i <= t <= j} F_it D_tj
+  const V* Ff = static_cast<V*>(cur ? a.fc[1] : a.fc[0]);
+  for (int64_t x = gt / SPLIT; x < nent; x += nt / SPLIT) {
+    if (part != 0) continue;
+    const int2 ij = upper_tri_entry((int)x);
+    const size_t o = (size_t)ij.y * l + ij.x;
+    const V f = Ff[o];
+    fr[(size_t)ij.x * l + ij.y] = f;
+    static_cast<V*>(a.dc[0])[o] = vec(-f.x, -f.y, -f.z, -f.w);
+  }
+  if (!series_barrier(a, bar++)) return;
+  cur = 0;
+  m = a.mx + 1 + SERIES_ITERS;
+  for (int it = 1; it < NEUMANN_ITERS; ++it, ++m) {
+    const V* Dv = static_cast<V*>(cur ? a.dc[1] : a.dc[0]);
+    V* Dn = static_cast<V*>(cur ? a.dc[0] : a.dc[1]);
+    step(m, s2,
+         [&](int i, int j) {
+           Quat<TA> acc = {0, 0, 0, 0};
+#pragma unroll 4
+           for (int t = i + part; t <= j; t += SPLIT) {
+             const Quat<TA> pr = qmul(ldc(fr + (size_t)i * l + t), ldc(Dv + (size_t)j * l + t));
+             acc.w += pr.w; acc.x += pr.x; acc.y += pr.y; acc.z += pr.z;
+           }
+           return acc;
+         },
+         [&](int i, int j, const Quat<TA>& s) {
+           const V f = Ff[(size_t)j * l + i];
+           Dn[(size_t)j * l + i] = vec(-f.x - s.w, -f.y - s.x, -f.z - s.y, -f.w - s.z);
+         });
+    cur ^= 1;
+    if (!series_barrier(a, bar++)) return;
+    if ((double)largest(m) * rate <= SERIES_TOL) break;
+  }
+  // R2 = I + F and R2^{-1} = I + D in FP64 from E and the sums, by their entries' owners (16 lanes
+  // take the four components of R2, R2inv and their zero mirror images)
+  for (int64_t x = gt / SPLIT; x < nent; x += nt / SPLIT) {
+    const int2 ij = upper_tri_entry((int)x);
+    const int i = ij.x, j = ij.y, c = part & 3;
+    const size_t o = (size_t)j * l + i, ll = (size_t)l * l;
+    if (part >= 8) {
+      if (i != j) (part < 12 ? a.R2 : a.R2inv)[c * ll + (size_t)i * l + j] = 0.0;
+      continue;
+    }
+    // written by lane 0 of this group before the last barrier
+    const TA* q1 = reinterpret_cast<const TA*>(s1 + o);
+    const TA* q2 = reinterpret_cast<const TA*>(s2 + o);
+    double e = a.G[c * ll + o];
+    if (i == j && c == 0) e -= 1.0;
+    double f = e - (double)__ldcg(q1 + c);
+    if (i == j) f = (c == 0) ? 0.5 * f : 0.0;
+    const double one = (i == j && c == 0) ? 1.0 : 0.0;
+    if (part < 4) a.R2[c * ll + o] = f + one;
+    else a.R2inv[c * ll + o] = one - f - (double)__ldcg(q2 + c);
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1956,50 +2063,31 @@ static int apply_rinv(qlr_ctx* ctx, const qlr_qmat& Y, const double* Rinv, qlr_q
 // f32acc: accumulate the small products in FP32 (Grams of FP32 sketches).
 static int series_factor(qlr_ctx* ctx, int l, const double* G, double* R2, double* R2inv, WsArena& ws,
                          int** use_chol_out, bool f32acc) {
-  const size_t ll4 = (size_t)4 * l * l;
-  double* E = ws.take<double>(ll4);
-  double* Fa = ws.take<double>(ll4);
-  double* Fb = ws.take<double>(ll4);
-  double* Xa = ws.take<double>(ll4);
-  double* Xb = ws.take<double>(ll4);
-  unsigned long long* emax = ws.take<unsigned long long>(1 + SERIES_ITERS + NEUMANN_ITERS);
-  unsigned long long* deltas = emax + 1;
-  int* use_chol = ws.take<int>(1);
-  const int nent = l * (l + 1) / 2;
+  const size_t ll = (size_t)l * l, vsz = f32acc ? 16 : 32;
+  constexpr int NMAX = 1 + SERIES_ITERS + NEUMANN_ITERS;
+  SeriesArgs a{};
+  a.G = G;
+  for (void** v : {&a.e, &a.s1, &a.s2, &a.fc[0], &a.fc[1], &a.fr, &a.dc[0], &a.dc[1]}) *v = ws.take<char>(ll * vsz);
+  a.mx = ws.take<unsigned>(NMAX + 1);
+  a.arrived = a.mx + NMAX;
+  a.use_chol = ws.take<int>(1);
   if (!ws.ok) return QLR_ENOMEM;
-  QLR_CUDA_TRY(cudaMemsetAsync(emax, 0, (1 + SERIES_ITERS + NEUMANN_ITERS) * sizeof(unsigned long long), ctx->stream));
+  a.R2 = R2;
+  a.R2inv = R2inv;
+  a.err = ctx->d_err;
+  a.l = l;
+  QLR_CUDA_TRY(cudaMemsetAsync(a.mx, 0, (NMAX + 1) * sizeof(unsigned), ctx->stream));
   KTimer kt(ctx, QLR_KID_SERIES);
-  const int64_t tot = (int64_t)l * l;
-  const unsigned gsq = (unsigned)((tot + 127) / 128);
-  const unsigned gst = (unsigned)(((int64_t)nent * SPLIT + 127) / 128);
-  series_init_kernel<<<gsq, 128, 0, ctx->stream>>>(G, E, Fa, l, emax);
+  const int64_t lanes = (int64_t)l * (l + 1) / 2 * SPLIT;
+  const int sms = ctx->num_sms > 0 ? ctx->num_sms : 148;
+  const int threads = lanes > (int64_t)sms * 512 ? SERIES_THREADS : 256;
+  const unsigned grid = (unsigned)std::min<int64_t>(sms, (lanes + threads - 1) / threads);
+  void* args[] = {&a};
+  const void* kern = f32acc ? (const void*)series_kernel<float> : (const void*)series_kernel<double>;
+  QLR_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, 0, ctx->stream));
   qlr_count_launch();
-  series_decide_kernel<<<1, 1, 0, ctx->stream>>>(emax, l, use_chol);
-  qlr_count_launch();
-  auto step = f32acc ? series_step_kernel<float> : series_step_kernel<double>;
-  double* Fc = Fa;
-  double* Fn = Fb;
-  for (int it = 0; it < SERIES_ITERS; ++it) {
-    step<<<gst, 128, 0, ctx->stream>>>(E, Fc, nullptr, Fn, l, 0, nent, 0, it ? deltas + it - 1 : nullptr, deltas + it);
-    qlr_count_launch();
-    std::swap(Fc, Fn);
-  }
-  series_form_kernel<<<gsq, 128, 0, ctx->stream>>>(Fc, R2, l);
-  qlr_count_launch();
-  // the Neumann iteration runs on D = X - I from D = 0; its last step writes I + D
-  QLR_CUDA_TRY(cudaMemsetAsync(Xa, 0, ll4 * sizeof(double), ctx->stream));
-  double* Xc = Xa;
-  double* Xn = Xb;
-  unsigned long long* nd = deltas + SERIES_ITERS;
-  for (int it = 0; it < NEUMANN_ITERS; ++it) {
-    const bool last = (it == NEUMANN_ITERS - 1);
-    step<<<gst, 128, 0, ctx->stream>>>(nullptr, Fc, Xc, last ? R2inv : Xn, l, 1, nent, last ? 1 : 0,
-                                       it ? nd + it - 1 : nullptr, nd + it);
-    qlr_count_launch();
-    std::swap(Xc, Xn);
-  }
   QLR_CUDA_TRY(cudaGetLastError());
-  *use_chol_out = use_chol;
+  *use_chol_out = a.use_chol;
   return QLR_OK;
 }
 
@@ -2055,7 +2143,7 @@ int cholqr(qlr_ctx* ctx, const qlr_qmat& Y, qlr_qmat& Q, double* R, int orth, Ws
       QLR_TRY(tri_inv(ctx, l, Rcur, Rinv, Dinv_all, nullptr, d32buf));
     }
     QLR_TRY(apply_rinv(ctx, src, Rinv, dst, ws));
-    if (s > 0) {   // R_total <- R_s * R_total
+    if (s > 0 && R) {   // R_total <- R_s * R_total
       QLR_TRY(small_matmul(ctx, l, Rs, Rprod, Rnext));
       double* sw = Rprod; Rprod = Rnext; Rnext = sw;
     }
