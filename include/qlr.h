@@ -430,7 +430,7 @@ int qlr_selftest_wait_timeout(qlr_ctx* ctx);
  * of it (the kept address would be stale).  The stream-K schedule uses as many CTAs as the array's
  * partial-tile space allows (up to one per SM).
  * The array is shared by all calls on a device and keeps the previous call's contents; each call
- * clears the parts that must start at zero.  Calls that overlap on the GPU (other streams or
+ * writes what it reads.  Calls that overlap on the GPU (other streams or
  * threads) race on the array: serialise them.  `err` (device int, may be NULL) receives
  * QLR_ETIMEOUT if a bounded device wait gives up.
  * Degenerate sizes as qlr_qsketch: an empty Y launches nothing; an empty inner dimension writes Y = 0.

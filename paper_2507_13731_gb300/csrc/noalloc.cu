@@ -7,9 +7,8 @@
 // product Y = A X / Y = A^H X of qlr_qsketch with every scratch byte taken from one fixed
 // file-scope device array that the CUDA module carries, so the call itself allocates nothing.
 //
-// The scratch array is shared by every call on a device and keeps the last call's contents; the
-// parts that must start at zero (the stream-K arrival counters) are cleared on the stream by each
-// call.  Calls that overlap on the GPU (different streams, or another thread's call in flight)
+// The scratch array is shared by every call on a device and keeps the last call's contents; a call
+// writes every part that it reads.  Calls that overlap on the GPU (different streams, or another thread's call in flight)
 // race on the array.
 #include <mutex>
 

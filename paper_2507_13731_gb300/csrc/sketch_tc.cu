@@ -20,7 +20,7 @@
 // it into hi / lo on the way for 3xTF32).
 // Warp roles: 0 = TMA producer, 1 = MMA issuer (owns TMEM), 2-3 = a pair of workers (hi/lo split,
 // rounding and/or transpose of A), 4-7 = epilogue (TMEM -> registers -> global, or a stream-K
-// partial + the last piece's reduction); with 384 threads, 8-11 = two more worker pairs or four more
+// partial); with 384 threads, 8-11 = two more worker pairs or four more
 // epilogue warps.
 // The MMA issuer is one thread, and what it does between two stages' MMAs leaves the tensor pipe
 // idle: its ring and chunk positions are counters (the integer divisions they replace took 300 of a
@@ -67,7 +67,6 @@ struct TcParams {
   float* y[4];
   int64_t ldy;
   float* part;              // stream-K partial tiles (two slots per CTA)
-  unsigned* counters;       // one arrival counter per output tile
   int64_t M;                // output rows
   int l;                    // valid output columns
   int nb;                   // output columns per CTA block
@@ -97,7 +96,6 @@ struct TcScalars {
   float *y0, *y1, *y2, *y3;                // output planes (selected without an indexed array)
   int64_t ldy;
   float* part;
-  unsigned* counters;
   int64_t M;
   int l, nb, ncb, kiters, c_first, stages;
   uint32_t neg_mask, idesc_base, tmem_cols;
@@ -108,7 +106,7 @@ struct TcScalars {
 __device__ __forceinline__ TcScalars tc_scalars(const TcParams& p) {
   TcScalars v;
   v.y0 = p.y[0]; v.y1 = p.y[1]; v.y2 = p.y[2]; v.y3 = p.y[3];
-  v.ldy = p.ldy; v.part = p.part; v.counters = p.counters; v.M = p.M; v.l = p.l; v.nb = p.nb; v.ncb = p.ncb;
+  v.ldy = p.ldy; v.part = p.part; v.M = p.M; v.l = p.l; v.nb = p.nb; v.ncb = p.ncb;
   v.kiters = p.kiters; v.c_first = p.c_first; v.stages = p.stages;
   v.neg_mask = p.neg_mask; v.idesc_base = p.idesc_base; v.tmem_cols = p.tmem_cols; v.err = p.err;
   v.flush = p.flush; v.nbuf = p.nbuf < 1 ? 1 : p.nbuf; v.ttotal = p.ttotal; v.apl = p.apl == 3 ? 3 : 4; v.fd = p.fd;
@@ -266,8 +264,8 @@ __device__ __forceinline__ void issue_stage(const StageDescs& D, int s, uint32_t
 // A contiguous piece of one output tile's reduction: stages [it0, it1).  A tile reduced in
 // nseg > 1 pieces (stream-K) has them from CTAs c0 .. c0 + nseg - 1 of its group; piece o writes
 // its partial to slot 2 ((c0 + o) cs + coff) + (o == 0 ? b0 : 0) (b0 = 1 when the tile starts
-// inside CTA c0's range, as that CTA's second piece), and the last piece to arrive adds the
-// partials in slot order.  A group is every CTA (cs = 1, coff = 0), or, with column-block groups,
+// inside CTA c0's range, as that CTA's second piece), and sketch_reduce_kernel adds the partials in
+// slot order.  A group is every CTA (cs = 1, coff = 0), or, with column-block groups,
 // the CTAs coff, coff + cs, coff + 2 cs, ... of one column block (cs = the number of blocks).
 struct Seg {
   int it0, it1, slot, nseg, c0, b0;
@@ -312,7 +310,6 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
   uint64_t* tmem_empty = bars + 3 * MAX_STAGES + 2;   // [2] a chunk accumulator has been drained
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * MAX_STAGES + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* last_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
   // Accumulation chunks: the tensor cores' FP32 accumulation does not round to nearest, and on
   // data of one sign its error grows with the number of MMAs added into one accumulator (~1 ulp
   // each).  With pv.flush > 0 the piece is reduced in chunks of pv.flush stages, each started from
@@ -350,7 +347,6 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
       mbar_init(&tmem_empty[b], 4 * EPI);           // one arrival per epilogue warp
     }
     *abort_flag = 0;
-    *last_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -522,7 +518,6 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
     const int q = warp & 3;                 // TMEM lane quarter of this warp
     const int row = q * 32 + lane;
     const int64_t grow = m0 + row;
-    const int tile = mt * pv.ncb + cb;
     const size_t tile_elems = (size_t)4 * TBM * nb;
     const int nchunks = (nit > 0) ? (nit + F - 1) / F : 1;
     const int nb_log = NBUF - 1, eh = warp >= 8 ? 1 : 0;   // NBUF is 1 or 2; this warp's half of the columns
@@ -600,38 +595,6 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
       __syncwarp();
       if (lane == 0) mbar_arrive(&tmem_empty[b]);   // this chunk's accumulator may be overwritten
     }
-    if (sg.nseg > 1) {
-      __threadfence();
-      asm volatile("bar.sync 1, %0;" ::"r"(128 * EPI) : "memory");
-      if (threadIdx.x == 128) {
-        const unsigned old = atomicAdd(&pv.counters[tile], 1u);
-        *last_flag = (old == (unsigned)(sg.nseg - 1)) ? 1 : 0;
-      }
-      asm volatile("bar.sync 1, %0;" ::"r"(128 * EPI) : "memory");
-      if (*last_flag) {
-        __threadfence();
-        if (grow < pv.M) {
-          for (int d = 0; d < 4; ++d)
-            for (int jc0 = 16 * eh; jc0 < nb; jc0 += 16 * EPI) {
-              float acc[16];
-#pragma unroll
-              for (int jj = 0; jj < 16; ++jj) acc[jj] = 0.f;
-              for (int o = 0; o < sg.nseg; ++o) {
-                const int slot = 2 * ((sg.c0 + o) * sg.cs + sg.coff) + (o == 0 ? sg.b0 : 0);
-                const float* P = pv.part + (size_t)slot * tile_elems + (size_t)d * TBM * nb + (size_t)jc0 * TBM + row;
-#pragma unroll
-                for (int jj = 0; jj < 16; ++jj) acc[jj] += __ldcg(P + (size_t)jj * TBM);   // 16 loads in flight
-              }
-#pragma unroll
-              for (int jj = 0; jj < 16; ++jj) {
-                const int j = j0 + jc0 + jj;
-                if (jc0 + jj < nb && j < pv.l) pv.y(d)[grow + (int64_t)j * pv.ldy] = acc[jj];
-              }
-            }
-        }
-        if (threadIdx.x == 128) pv.counters[tile] = 0u;
-      }
-    }
   }
   tc_fence_before();
   __syncthreads();
@@ -651,8 +614,8 @@ __global__ void __launch_bounds__(KIND == K_BF16 ? TC_THREADS : TC_THREADS_WIDE,
 // Stream-K: the reduction stages of all tiles, taken in tile order, are cut into gridDim.x equal
 // ranges, one per CTA.  A range may start inside one tile (its tail piece), run through whole
 // tiles, and end inside another (its head piece); each piece is reduced as in sketch_tile, a
-// whole tile writes its output directly, and the pieces of a split tile are added by the last one
-// to finish.  A CTA writes at most two partial tiles: slot 2c for its tail piece, slot 2c + 1 for a
+// whole tile writes its output directly, and the pieces of a split tile are added by
+// sketch_reduce_kernel.  A CTA writes at most two partial tiles: slot 2c for its tail piece, slot 2c + 1 for a
 // head piece that is not its first piece.
 // Column-block groups (p.cgroup, gridDim.x a multiple of ncb): CTA c works on column block
 // c mod ncb only, and the CTAs of each block split that block's row tiles' stages the same way,
@@ -660,23 +623,27 @@ __global__ void __launch_bounds__(KIND == K_BF16 ? TC_THREADS : TC_THREADS_WIDE,
 // DRAM once and from L2 for the other blocks (with one list over all blocks, the CTAs reading a
 // given A stage for different blocks are a tile's length apart in time and A is re-read from
 // DRAM once per block).
+struct StreamK {
+  int64_t K, W, G;   // stages per tile, stages in all, CTAs (of a column-block group where p.cgroup)
+  __device__ __forceinline__ int64_t start(int64_t cc) const { return cc * W / G; }
+  // the CTA whose range holds stage x: the largest cc with start(cc) <= x
+  __device__ __forceinline__ int64_t owner(int64_t x) const { return ((x + 1) * G + W - 1) / W - 1; }
+};
 template <int KIND, int AMODE, bool WIDE>
 __global__ void __launch_bounds__(KIND == K_BF16 ? TC_THREADS : TC_THREADS_WIDE, 1) sketch_tc_streamk_kernel(const __grid_constant__ TcParams p) {
   const int NG = (p.cgroup && p.ncb > 1) ? p.ncb : 1;             // CTAs per group step
   const int cbg = (int)(blockIdx.x % NG);                         // this CTA's block (groups)
-  const int64_t K = p.kiters, W = (int64_t)p.mtiles * (p.ncb / NG) * K, G = gridDim.x / NG, c = blockIdx.x / NG;
-  auto start = [&](int64_t cc) { return cc * W / G; };
-  // the CTA whose range holds stage x: the largest cc with start(cc) <= x
-  auto owner = [&](int64_t x) { return ((x + 1) * G + W - 1) / W - 1; };
-  int64_t pos = start(c);
-  const int64_t end = start(c + 1);
+  const StreamK sk{p.kiters, (int64_t)p.mtiles * (p.ncb / NG) * p.kiters, gridDim.x / NG};
+  const int64_t K = p.kiters, c = blockIdx.x / NG;
+  int64_t pos = sk.start(c);
+  const int64_t end = sk.start(c + 1);
   bool first = true;
   while (pos < end) {
     const int64_t t = pos / K;
     const int it0 = (int)(pos - t * K);
     const int it1 = (int)min(K, (int64_t)it0 + (end - pos));
-    const int64_t c0 = owner(t * K), c1 = owner((t + 1) * K - 1);
-    const int b0 = (start(c0) < t * K) ? 1 : 0;
+    const int64_t c0 = sk.owner(t * K), c1 = sk.owner((t + 1) * K - 1);
+    const int b0 = (sk.start(c0) < t * K) ? 1 : 0;
     const int more = (pos + (it1 - it0) < end) ? 1 : 0;
     const Seg sg{it0, it1, (int)(2 * (c * NG + cbg) + (c == c0 ? b0 : 0)), (int)(c1 - c0 + 1), (int)c0, b0, more,
                  NG, cbg};
@@ -686,6 +653,56 @@ __global__ void __launch_bounds__(KIND == K_BF16 ? TC_THREADS : TC_THREADS_WIDE,
     first = false;
     pos += it1 - it0;
   }
+}
+
+// The output tiles that stream-K reduced in pieces: Y = the sum of the pieces' partials in slot order.
+// blockIdx.x is the tile, blockIdx.y four of its 4 nb columns; a thread per row, up to 32 loads in
+// flight.  (The last CTA of a tile to finish did this before, 16 columns at a time while the others had
+// left: 80 of 85 us at 1500 x 600 x 100, 12 tiles of 12 pieces.)
+constexpr int RED_COLS = 4, RED_AHEAD = 8;
+struct ReduceArgs {
+  const float* part;
+  float* y[4];
+  int64_t ldy, M;
+  int l, nb, ncb, kiters, mtiles, cgroup, grid;
+};
+__global__ void __launch_bounds__(TBM) sketch_reduce_kernel(const ReduceArgs a) {
+  const int NG = (a.cgroup && a.ncb > 1) ? a.ncb : 1;
+  const StreamK sk{a.kiters, (int64_t)a.mtiles * (a.ncb / NG) * a.kiters, a.grid / NG};
+  // tile t of the list (of its column block's list in groups)
+  const int coff = NG > 1 ? (int)blockIdx.x % NG : 0;
+  const int64_t t = (int64_t)blockIdx.x / NG, K = a.kiters;
+  const int cb = NG > 1 ? coff : (int)(t % a.ncb), mt = (int)(NG > 1 ? t : t / a.ncb);
+  const int64_t c0 = sk.owner(t * K), c1 = sk.owner((t + 1) * K - 1);
+  const int nseg = (int)(c1 - c0 + 1);
+  if (nseg == 1) return;                       // written by its CTA
+  const int b0 = (sk.start(c0) < t * K) ? 1 : 0;
+  const int per = (a.nb + RED_COLS - 1) / RED_COLS, d = (int)blockIdx.y / per, jc = ((int)blockIdx.y % per) * RED_COLS;
+  const int64_t row = (int64_t)mt * TBM + threadIdx.x;
+  const int j0 = cb * a.nb + jc;
+  if (row >= a.M || j0 >= a.l) return;
+  const size_t tile_elems = (size_t)4 * TBM * a.nb, off = ((size_t)d * a.nb + jc) * TBM + threadIdx.x;
+  auto piece = [&](int o) { return a.part + (size_t)(2 * ((c0 + o) * NG + coff) + (o == 0 ? b0 : 0)) * tile_elems + off; };
+  float acc[RED_COLS] = {};
+  for (int o0 = 0; o0 < nseg; o0 += RED_AHEAD) {
+    float v[RED_AHEAD][RED_COLS];
+#pragma unroll
+    for (int u = 0; u < RED_AHEAD; ++u)
+      if (o0 + u < nseg) {
+        const float* P = piece(o0 + u);
+#pragma unroll
+        for (int e = 0; e < RED_COLS; ++e) v[u][e] = __ldcg(P + e * TBM);
+      }
+#pragma unroll
+    for (int u = 0; u < RED_AHEAD; ++u)
+      if (o0 + u < nseg)
+#pragma unroll
+        for (int e = 0; e < RED_COLS; ++e) acc[e] += v[u][e];
+  }
+  float* y = (d == 0 ? a.y[0] : d == 1 ? a.y[1] : d == 2 ? a.y[2] : a.y[3]) + row + (int64_t)j0 * a.ldy;
+#pragma unroll
+  for (int e = 0; e < RED_COLS; ++e)
+    if (j0 + e < a.l) y[e * a.ldy] = acc[e];   // nb is a multiple of RED_COLS
 }
 
 // Grouped launch over many problems: CTA b computes the tile items[b] = (problem, row tile,
@@ -1210,6 +1227,15 @@ int launch_kernel(qlr_ctx* ctx, const Plan& pl, const TcParams& prm, int kid) {
     auto sk = sketch_tc_streamk_kernel<KIND, AMODE, WIDE>;
     QLR_CUDA_TRY(cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
     sk<<<pl.grid_sk, threads, pl.smem, ctx->stream>>>(prm);
+    qlr_count_launch();
+    QLR_CUDA_TRY(cudaGetLastError());
+    ReduceArgs ra{};
+    ra.part = prm.part;
+    for (int c = 0; c < 4; ++c) ra.y[c] = prm.y[c];
+    ra.ldy = prm.ldy; ra.M = prm.M; ra.l = prm.l; ra.nb = prm.nb; ra.ncb = prm.ncb; ra.kiters = prm.kiters;
+    ra.mtiles = prm.mtiles; ra.cgroup = prm.cgroup; ra.grid = pl.grid_sk;
+    sketch_reduce_kernel<<<dim3((unsigned)(pl.mtiles * pl.ncb), (unsigned)(4 * ((pl.nb + RED_COLS - 1) / RED_COLS))), TBM, 0,
+                           ctx->stream>>>(ra);
   } else {
     kern<<<dim3((unsigned)pl.ncb, (unsigned)pl.mtiles, 1u), threads, pl.smem, ctx->stream>>>(prm);
   }
@@ -1547,7 +1573,7 @@ size_t sketch_tc_need(int op, int64_t M, int64_t K, int l, int compute, int num_
   size_t b = align256(xb);
   if (pl.kind == K_TF32X3) b += align256(xb);
   if (pl.grid_sk > 0) b += align256((size_t)2 * pl.grid_sk * 4 * TBM * pl.nb * sizeof(float));
-  return b + align256((size_t)pl.mtiles * pl.ncb * sizeof(unsigned));
+  return b;
 }
 
 int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qmat& Y, int compute, WsArena& ws) {
@@ -1571,7 +1597,6 @@ int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qm
   void* xlo = (pl.kind == K_TF32X3) ? ws.take<char>(xb) : nullptr;
   const size_t tile_elems = (size_t)4 * TBM * pl.nb;
   float* part = pl.grid_sk > 0 ? ws.take<float>((size_t)2 * pl.grid_sk * tile_elems) : nullptr;
-  unsigned* counters = ws.take<unsigned>((size_t)pl.mtiles * pl.ncb);
   if (!ws.ok) return QLR_ENOMEM;
   if (X.dtype == QLR_BF16) {
     qlr_qmat dst = X;
@@ -1603,7 +1628,6 @@ int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qm
     qlr_count_launch();
     QLR_CUDA_TRY(cudaGetLastError());
   }
-  QLR_CUDA_TRY(cudaMemsetAsync(counters, 0, (size_t)pl.mtiles * pl.ncb * sizeof(unsigned), ctx->stream));
 
   TcParams prm;
   memset(&prm, 0, sizeof(prm));
@@ -1649,7 +1673,6 @@ int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qm
   for (int c = 0; c < 4; ++c) prm.y[c] = static_cast<float*>(Y.plane[c]);
   prm.ldy = Y.ld;
   prm.part = part;
-  prm.counters = counters;
   prm.M = M;
   prm.l = l;
   prm.nb = pl.nb;
