@@ -17,7 +17,7 @@ namespace qlr {
 size_t gram_ws_bound(int64_t rows, int64_t l) {
   size_t per = (size_t)32 * l * l;
   size_t cap = std::max<size_t>(per, (size_t)64 << 20);
-  const size_t tc = (l <= 1024) ? gram_tc_ws(rows, (int)l) : 0;
+  const size_t tc = (l <= 1024) ? gram_tc_ws(rows, (int)l, true) : 0;
   return std::max(cap, tc) + (size_t)8 * ((l + 31) / 32) * ((l + 31) / 32) + 4096;
 }
 

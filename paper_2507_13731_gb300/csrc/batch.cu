@@ -276,7 +276,7 @@ size_t layout(qlr_batch* b, const qlr_qmat* A, const int* k, const int* p, const
     P.Z = thin_at(cur, n, P.l);
     P.Q2 = thin_at(cur, n, P.l);
     P.T = thin_at(cur, std::max(m, n), P.l);
-    P.gsc = take<char>(cur, gram_tc_ws(std::max(m, n), P.l));
+    P.gsc = take<char>(cur, gram_tc_ws(std::max(m, n), P.l, false));
     P.G = take<float>(cur, (size_t)8 * P.l * P.l);
     P.Rinv = take<float>(cur, (size_t)4 * P.l * P.l);
     P.Rp[0] = take<float>(cur, (size_t)4 * P.l * P.l);

@@ -19,14 +19,14 @@
 // double-FP32 SIMT path (orth.cu), at tensor-core throughput.
 //
 // Kernels: gram_slice_kernel (one CTA per column: exponent, then the 7 slices, BF16, column-major
-// per slice with rows padded to a multiple of 8), gram_tc_kernel (one CTA per (128 x 64 tile of
-// W's upper part, 512-row chunk): TMA of the 7 slices of both operands into a ring of two 32-row
+// per slice with rows padded to a multiple of 8), gram_tc_kernel (persistent CTAs over the (128 x 64
+// tile of W's upper part, 512-row chunk) items: TMA of the 7 slices of both operands into a ring of two 32-row
 // stages, 10 MMAs of 128 x (64..256) x 16 per 16 rows into 7 x 64 TMEM columns, epilogue to
 // double-FP32 partial tiles), gram_tc_combine_kernel (chunk sums, scaling, the quaternion
 // components of G).
 // Bound: a stage row is 64 bytes of one column and slice, and the TMA's row rate, then the MMAs, set
 // the pace: 16-row stages (32-byte rows) and 8 slices took 391 us at 20000 x 180 and 76 us at
-// 20000 x 60, this form 310 and 60 (error over max|y_a| max|y_b| m: 2^-48.1, before 2^-45.9).
+// 20000 x 60, this form 251 and 43 (error over max|y_a| max|y_b| m: 2^-48.1, before 2^-45.9).
 #include <algorithm>
 #include <cstring>
 
@@ -53,9 +53,10 @@ constexpr int GTMEM = 512;       // TMEM columns allocated for the weight groups
 constexpr int GA = 128;          // W rows per tile (MMA M)
 constexpr int GB = 64;           // W columns per tile (MMA N)
 constexpr int GK = 32;           // rows of Y per pipeline stage (64-byte swizzled BF16 rows, two MMA K)
-constexpr int GCHUNK = 512;      // rows of Y per CTA (exactness of the TMEM sums)
+constexpr int GCHUNK = 512;      // rows of Y per item at most (exactness of the TMEM sums)
 constexpr int GSTAGES = 2;
-constexpr int GTHREADS = 256;
+constexpr int GEPI = 8;                // epilogue warps: a lane quarter and half the columns each
+constexpr int GTHREADS = 64 + 32 * GEPI;
 constexpr int GSW = GK * 2;           // bytes per K-major row = swizzle span
 constexpr int GMODE = 4;              // descriptor swizzle mode: 64 bytes
 constexpr int A_TILE = GA * GK * 2;   // bytes of one slice's A tile
@@ -70,6 +71,7 @@ struct GramTcParams {
   int L4p;              // columns per slice (L4 rounded up to GB; an A tile may run into the
                         // next slice: those W rows a >= L4 are never stored)
   int kiters;           // GK-row stages over all m rows
+  int cstages;          // stages per chunk
   int* err;
 };
 
@@ -87,7 +89,7 @@ struct GramTcProb {
 
 // Columns of Yh (L4p columns, the padding zero) by CTAs of 8 warps, WPC warps per column (8 for
 // one tall problem, 1 for the many short ones of a batch): the column exponent, then the
-// slices; each lane takes row pairs, stored as BF16 pairs.
+// slices (two rows a lane and 4-byte stores took 60 us at 20000 x 180, now 51).
 template <int N, int WPC>
 __device__ __forceinline__ void gram_slice_cols(const float* __restrict__ y0, const float* __restrict__ y1,
                                                 const float* __restrict__ y2, const float* __restrict__ y3, int64_t m,
@@ -102,9 +104,26 @@ __device__ __forceinline__ void gram_slice_cols(const float* __restrict__ y0, co
     const int pl = c / l, j = c % l;
     y = (pl == 0 ? y0 : pl == 1 ? y1 : pl == 2 ? y2 : y3) + (int64_t)j * ld;
   }
+  // eight rows a lane and turn: two 16-byte loads where the column allows, one 16-byte store a slice
+  const bool vec = (reinterpret_cast<uintptr_t>(y) & 15u) == 0;
+  auto load8 = [&](int64_t r, float (&v)[8]) {
+    if (vec && r + 8 <= m) {
+      const float4 a = *reinterpret_cast<const float4*>(y + r), b = *reinterpret_cast<const float4*>(y + r + 4);
+      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = (r + u < m) ? y[r + u] : 0.f;
+    }
+  };
   float mx = 0.f;
   if (y)
-    for (int64_t r = sub * 32 + lane; r < m; r += 32 * WPC) mx = fmaxf(mx, fabsf(y[r]));
+#pragma unroll 2
+    for (int64_t r = 8 * (sub * 32 + lane); r < m; r += 256 * WPC) {
+      float v[8];
+      load8(r, v);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) mx = fmaxf(mx, fabsf(v[u]));
+    }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if (WPC > 1) {
@@ -117,16 +136,26 @@ __device__ __forceinline__ void gram_slice_cols(const float* __restrict__ y0, co
   int e = 0;
   if (mx > 0.f) frexpf(mx, &e);   // max < 2^e
   if (sub == 0 && lane == 0) ex[c] = e;
-  for (int64_t r = 2 * (sub * 32 + lane); r < mp; r += 64 * WPC) {   // mp is even
-    float v0 = (y && r < m) ? ldexpf(y[r], GTOP - e) : 0.f;       // |v| < 64, exact
-    float v1 = (y && r + 1 < m) ? ldexpf(y[r + 1], GTOP - e) : 0.f;
+  // 2^(GTOP - e) as two factors (its exponent may exceed FP32's)
+  const int k = GTOP - e, k1 = k / 2;
+  const float f1 = __int_as_float((127 + k1) << 23), f2 = __int_as_float((127 + k - k1) << 23);
+  for (int64_t r = 8 * (sub * 32 + lane); r < mp; r += 256 * WPC) {   // mp is a multiple of 8
+    float v[8] = {};
+    if (y && r < m) load8(r, v);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = (v[u] * f1) * f2;               // |v| < 64, exact
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const float q0 = Slices<N>::NEAREST ? rintf(v0) : truncf(v0);   // |q| <= 64, or 63
-      const float q1 = Slices<N>::NEAREST ? rintf(v1) : truncf(v1);
-      *reinterpret_cast<__nv_bfloat162*>(S + ((size_t)i * L4p + c) * mp + r) = __floats2bfloat162_rn(q0, q1);
-      v0 = (v0 - q0) * (float)(1 << Slices<N>::GBITS);                // exact
-      v1 = (v1 - q1) * (float)(1 << Slices<N>::GBITS);
+      __nv_bfloat162 p[4];
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        const float q0 = Slices<N>::NEAREST ? rintf(v[u]) : truncf(v[u]);   // |q| <= 64, or 63
+        const float q1 = Slices<N>::NEAREST ? rintf(v[u + 1]) : truncf(v[u + 1]);
+        p[u / 2] = __floats2bfloat162_rn(q0, q1);
+        v[u] = (v[u] - q0) * (float)(1 << Slices<N>::GBITS);                // exact
+        v[u + 1] = (v[u + 1] - q1) * (float)(1 << Slices<N>::GBITS);
+      }
+      *reinterpret_cast<uint4*>(S + ((size_t)i * L4p + c) * mp + r) = *reinterpret_cast<const uint4*>(p);
     }
   }
 }
@@ -155,27 +184,34 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& e, float x) {
   e = __fadd_rn(e, err);
 }
 
-// One tile of W for one chunk of rows: tile index tl enumerates (ab, bb) with bb >= 2 ab (the
-// upper part of W).
-template <int N>
-__device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, const int chunk) {
-  constexpr int GS = Slices<N>::GS, GBITS = Slices<N>::GBITS, NGRP = Slices<N>::NGRP, GPAIR_MAX = NGRP + 1;
-  constexpr int STAGE_BYTES = GS * (A_TILE + B_TILE);
+// A tile of W for one chunk of rows: tile index tl enumerates (ab, bb) with bb >= 2 ab (the upper part
+// of W).
+struct GramTile {
+  int a0, b0, it0, nit, chunk;
+};
+__device__ __forceinline__ GramTile gram_tile(const GramTcParams& p, int tl, int chunk) {
   int ab = 0;
   while (ab < p.nA && tl >= max(0, p.nB - 2 * ab)) { tl -= max(0, p.nB - 2 * ab); ++ab; }
-  const int bb = 2 * ab + tl;
-  const int a0 = ab * GA, b0 = bb * GB;
-  const int it0 = chunk * (GCHUNK / GK);
-  const int it1 = min(p.kiters, it0 + GCHUNK / GK);
-  const int nit = it1 - it0;
+  const int it0 = chunk * p.cstages;
+  return {ab * GA, (2 * ab + tl) * GB, it0, min(p.kiters, it0 + p.cstages) - it0, chunk};
+}
 
+// Persistent CTAs: CTA b takes items b, b + gridDim.x, ...  `item(i)` gives the parameters and the tile.
+// The accumulators fill the TMEM, so an item's MMAs wait for the one before to be read out; its
+// first stages are loaded meanwhile, and eight warps read (one CTA per item with four epilogue
+// warps spent 21 of 50 thousand cycles outside the MMAs).
+template <int N, class Item>
+__device__ __forceinline__ void gram_tc_items(const int nitems, Item item, int* err) {
+  constexpr int GS = Slices<N>::GS, GBITS = Slices<N>::GBITS, NGRP = Slices<N>::NGRP, GPAIR_MAX = NGRP + 1;
+  constexpr int STAGE_BYTES = GS * (A_TILE + B_TILE);
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + GSTAGES * STAGE_BYTES);
   uint64_t* full = bars;
   uint64_t* empty = bars + GSTAGES;
   uint64_t* tmem_full = bars + 2 * GSTAGES;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * GSTAGES + 1);
+  uint64_t* tmem_empty = tmem_full + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_empty + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   auto a_tile = [&](int s, int i) { return smem + s * STAGE_BYTES + i * A_TILE; };
   auto b_tile = [&](int s, int j) { return smem + s * STAGE_BYTES + GS * A_TILE + j * B_TILE; };
@@ -187,11 +223,12 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
       mbar_init(&empty[s], 1);
     }
     mbar_init(tmem_full, 1);
+    mbar_init(tmem_empty, GEPI);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  if (warp == 1) {
+  if (warp == GEPI + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(GTMEM)
                  : "memory");
@@ -202,31 +239,35 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0) {
+  if (warp == GEPI) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      int issued = 0;
-      for (int i = 0; i < nit; ++i) {
-        const int s = i % GSTAGES;
-        const uint32_t ph = (uint32_t)(i / GSTAGES) & 1u;
-        if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, p.err)) break;
-        mbar_expect_tx(&full[s], (uint32_t)STAGE_BYTES);
-        const int k0 = (it0 + i) * GK;
-        for (int q = 0; q < GS; ++q) {
-          tma_load_2d(smem_u32(a_tile(s, q)), &p.tmA, k0, q * p.L4p + a0, &full[s]);
-          tma_load_2d(smem_u32(b_tile(s, q)), &p.tmB, k0, q * p.L4p + b0, &full[s]);
+      int issued = 0, s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int x = blockIdx.x; x < nitems && ok; x += gridDim.x) {
+        const GramTcParams* pp;
+        const GramTile g = item(x, pp, true);
+        for (int i = 0; i < g.nit; ++i) {
+          ok = mbar_wait(&empty[s], ph ^ 1u, abort_flag, err);
+          if (!ok) break;
+          mbar_expect_tx(&full[s], (uint32_t)STAGE_BYTES);
+          const int k0 = (g.it0 + i) * GK;
+          for (int q = 0; q < GS; ++q) {
+            tma_load_2d(smem_u32(a_tile(s, q)), &pp->tmA, k0, q * pp->L4p + g.a0, &full[s]);
+            tma_load_2d(smem_u32(b_tile(s, q)), &pp->tmB, k0, q * pp->L4p + g.b0, &full[s]);
+          }
+          ++issued;
+          if (++s == GSTAGES) { s = 0; ph ^= 1u; }
         }
-        ++issued;
       }
       // drain: every issued stage must have landed before the CTA may exit
       for (int i = max(0, issued - GSTAGES); i < issued; ++i) {
-        const int s = i % GSTAGES;
-        const uint32_t ph = (uint32_t)(i / GSTAGES) & 1u;
         const uint64_t t0 = now_ns();
-        while (!mbar_try_wait(&full[s], ph) && now_ns() - t0 < WAIT_NS) __nanosleep(64);
+        while (!mbar_try_wait(&full[i % GSTAGES], (uint32_t)(i / GSTAGES) & 1u) && now_ns() - t0 < WAIT_NS) __nanosleep(64);
       }
     }
-  } else if (warp == 1) {
+  } else if (warp == GEPI + 1) {
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
       // BF16 A and B, FP32 D, both K-major, M = GA; N = t GB for t consecutive B slices: the B
@@ -237,66 +278,74 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
       const uint64_t ad0 = make_desc(smem_u32(a_tile(0, 0)), 16, 8 * GSW, GMODE);
       const uint64_t bd0 = make_desc(smem_u32(b_tile(0, 0)), 16, 8 * GSW, GMODE);
       bool ok = true;
-      for (int i = 0; i < nit && ok; ++i) {
-        const int s = i % GSTAGES;
-        const uint32_t ph = (uint32_t)(i / GSTAGES) & 1u;
-        ok = mbar_wait(&full[s], ph, abort_flag, p.err);
-        if (!ok) break;
+      int s = 0;
+      uint32_t ph = 0, done = 0;                 // done: items handed to the epilogue
+      for (int x = blockIdx.x; x < nitems && ok; x += gridDim.x, ++done) {
+        const GramTcParams* pp;
+        const GramTile g = item(x, pp, false);
+        if (done > 0) {
+          ok = mbar_wait(tmem_empty, (done - 1) & 1u, abort_flag, err);
+          if (!ok) break;
+        }
         tc_fence_after();
-        const uint64_t so = (uint64_t)(s * (STAGE_BYTES >> 4));
+        for (int i = 0; i < g.nit; ++i) {
+          ok = mbar_wait(&full[s], ph, abort_flag, err);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t so = (uint64_t)(s * (STAGE_BYTES >> 4));
 #pragma unroll
-        for (int ks = 0; ks < GK / 16; ++ks) {
+          for (int ks = 0; ks < GK / 16; ++ks) {
 #pragma unroll
-          for (int qi = 0; qi < GS; ++qi) {
-            const uint64_t ad = ad0 + so + (uint64_t)((qi * A_TILE + ks * 32) >> 4);
+            for (int qi = 0; qi < GS; ++qi) {
+              const uint64_t ad = ad0 + so + (uint64_t)((qi * A_TILE + ks * 32) >> 4);
 #pragma unroll
-            for (int qj = 0; qj <= GPAIR_MAX - 2 - qi; qj += 4) {
-              const int t = min(4, GPAIR_MAX - 1 - qi - qj);   // slices qj .. qj + t - 1
-              const uint64_t bd = bd0 + so + (uint64_t)((qj * B_TILE + ks * 32) >> 4);
-              const uint32_t idesc = idesc0 | ((uint32_t)((t * GB) >> 3) << 17);
-              // first products of the weight groups in this chunk: qi == 0, first stage and k-step
-              const uint32_t acc = (i > 0 || ks > 0 || qi > 0) ? 1u : 0u;
-              umma_bf16(tmem + (uint32_t)((qi + qj) * GB), ad, bd, idesc, acc);
+              for (int qj = 0; qj <= GPAIR_MAX - 2 - qi; qj += 4) {
+                const int t = min(4, GPAIR_MAX - 1 - qi - qj);   // slices qj .. qj + t - 1
+                const uint64_t bd = bd0 + so + (uint64_t)((qj * B_TILE + ks * 32) >> 4);
+                const uint32_t idesc = idesc0 | ((uint32_t)((t * GB) >> 3) << 17);
+                // first products of the weight groups in this chunk: qi == 0, first stage and k-step
+                const uint32_t acc = (i > 0 || ks > 0 || qi > 0) ? 1u : 0u;
+                umma_bf16(tmem + (uint32_t)((qi + qj) * GB), ad, bd, idesc, acc);
+              }
             }
           }
+          umma_commit(&empty[s]);   // frees the stage once these MMAs have read it
+          if (++s == GSTAGES) { s = 0; ph ^= 1u; }
         }
-        umma_commit(&empty[s]);   // frees the stage once these MMAs have read it
+        umma_commit(tmem_full);     // accumulators complete (also fires after an abort)
       }
-      umma_commit(tmem_full);     // accumulators complete (also fires after an abort)
     }
-  } else if (warp >= 4) {
+  } else {
     // ---------------- epilogue: the exact integer sums -> double-FP32 ----------------
-    const int q = warp & 3;
-    const int a = a0 + q * 32 + lane;
-    const bool ok = mbar_wait(tmem_full, 0, abort_flag, p.err) && !*abort_flag;
-    tc_fence_after();
-    if (ok && nit > 0) {
-      float h[GB], e[GB];
+    const int q = warp & 3, c0 = (warp >> 2) * (GB / 2);
+    uint32_t done = 0;
+    for (int x = blockIdx.x; x < nitems; x += gridDim.x, ++done) {
+      const GramTcParams* pp;
+      const GramTile g = item(x, pp, false);
+      if (!mbar_wait(tmem_full, done & 1u, abort_flag, err) || *abort_flag) break;
+      tc_fence_after();
+      float h[GB / 2], e[GB / 2];
 #pragma unroll
-      for (int jj = 0; jj < GB; ++jj) h[jj] = e[jj] = 0.f;
+      for (int jj = 0; jj < GB / 2; ++jj) h[jj] = e[jj] = 0.f;
 #pragma unroll
-      for (int g = NGRP - 1; g >= 0; --g) {
-        const float w = __int_as_float((127 - GBITS * g) << 23);   // 2^(-GBITS g)
+      for (int gr = NGRP - 1; gr >= 0; --gr) {
+        const float w = __int_as_float((127 - GBITS * gr) << 23);   // 2^(-GBITS gr)
+        uint32_t r[32];
+        tmem_ld32_issue(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(gr * GB + c0), r);
+        tmem_wait_ld();
 #pragma unroll
-        for (int cc = 0; cc < GB; cc += 32) {
-          uint32_t r0[16], r1[16];
-          const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * GB + cc);
-          tmem_ld16_issue(ta, r0);
-          tmem_ld16_issue(ta + 16, r1);
-          tmem_wait_ld();
-#pragma unroll
-          for (int jj = 0; jj < 16; ++jj) {
-            two_sum_acc(h[cc + jj], e[cc + jj], __uint_as_float(r0[jj]) * w);
-            two_sum_acc(h[cc + 16 + jj], e[cc + 16 + jj], __uint_as_float(r1[jj]) * w);
-          }
-        }
+        for (int jj = 0; jj < GB / 2; ++jj) two_sum_acc(h[jj], e[jj], __uint_as_float(r[jj]) * w);
       }
-      if (a < p.L4) {
-        float2* P = p.part + (size_t)chunk * p.L4 * p.L4;
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tmem_empty);
+      const int a = g.a0 + q * 32 + lane, L4 = pp->L4;
+      if (a < L4) {
+        float2* P = pp->part + (size_t)g.chunk * L4 * L4;
 #pragma unroll
-        for (int jj = 0; jj < GB; ++jj) {
-          const int b = b0 + jj;
-          if (b < p.L4) P[(size_t)b * p.L4 + a] = make_float2(h[jj], e[jj]);
+        for (int jj = 0; jj < GB / 2; ++jj) {
+          const int b = g.b0 + c0 + jj;
+          if (b < L4) P[(size_t)b * L4 + a] = make_float2(h[jj], e[jj]);
         }
       }
     }
@@ -304,27 +353,38 @@ __device__ __forceinline__ void gram_tc_tile(const GramTcParams& p, int tl, cons
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) {
+  if (warp == GEPI + 1) {
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(GTMEM) : "memory");
   }
 }
 
-__global__ void __launch_bounds__(GTHREADS, 1) gram_tc_kernel(const __grid_constant__ GramTcParams p) {
-  gram_tc_tile<7>(p, blockIdx.x, blockIdx.y);
+__global__ void __launch_bounds__(GTHREADS, 1) gram_tc_kernel(const __grid_constant__ GramTcParams p, int ntiles, int nitems) {
+  gram_tc_items<7>(
+      nitems,
+      [&](int x, const GramTcParams*& pp, bool) {
+        pp = &p;
+        return gram_tile(p, x % ntiles, x / ntiles);
+      },
+      p.err);
 }
 
 // Batch plans: item (problem, tile, chunk) with that problem's parameters in global memory
 // (tensor maps 64-byte aligned, written before the launch).
 __global__ void __launch_bounds__(GTHREADS, 1) gram_tc_grouped_kernel(const GramTcProb* __restrict__ probs,
-                                                                      const int4* __restrict__ items) {
-  const int4 it = items[blockIdx.x];
-  const GramTcParams& p = probs[it.x].tc;
-  if (threadIdx.x == 0) {   // the TMA-issuing thread
-    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&p.tmA) : "memory");
-    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&p.tmB) : "memory");
-  }
-  gram_tc_tile<8>(p, it.y, it.z);
+                                                                      const int4* __restrict__ items, int nitems, int* err) {
+  gram_tc_items<8>(
+      nitems,
+      [&](int x, const GramTcParams*& pp, bool tma) {
+        const int4 it = items[x];
+        pp = &probs[it.x].tc;
+        if (tma) {   // the TMA-issuing thread
+          asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&pp->tmA) : "memory");
+          asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&pp->tmB) : "memory");
+        }
+        return gram_tile(*pp, it.y, it.z);
+      },
+      err);
 }
 
 // W(I, J) for I <= J: the chunk partials added in double-FP32, scaled by 2^(e_I + e_J - 12).
@@ -434,10 +494,13 @@ __global__ void __launch_bounds__(128) gram_tc_combine_kernel(const float2* __re
 }
 
 struct GramTcDims {
-  int L4, L4p, nA, nB, ntiles, nchunks, kiters;
+  int L4, L4p, nA, nB, ntiles, nchunks, kiters, chunk;
   int64_t mp;
 };
-GramTcDims gram_tc_dims(int64_t m, int l) {
+// `single`: rows per chunk such that the items fill whole waves of the SMs, an item's time outside its
+// MMAs counted as 100 rows (4096 x 40: 32 items of 512 rows took 25 us, 128 of 128 rows 12; 20000 x 60: 49 and
+// 43 us); from four waves on, and in batch plans, 512.
+GramTcDims gram_tc_dims(int64_t m, int l, bool single) {
   GramTcDims d{};
   d.L4 = 4 * l;
   d.L4p = (d.L4 + GB - 1) / GB * GB;
@@ -447,7 +510,16 @@ GramTcDims gram_tc_dims(int64_t m, int l) {
   for (int ab = 0; ab < d.nA; ++ab) d.ntiles += std::max(0, d.nB - 2 * ab);
   d.mp = std::max<int64_t>(GK, (m + 7) / 8 * 8);   // at least one TMA box of rows
   d.kiters = (int)((m + GK - 1) / GK);
-  d.nchunks = (int)((m + GCHUNK - 1) / GCHUNK);
+  d.chunk = GCHUNK;
+  constexpr int64_t SMS = 152;
+  if (single && d.ntiles * ((m + GCHUNK - 1) / GCHUNK) < 4 * SMS) {
+    int64_t best = INT64_MAX;
+    for (int c = GCHUNK; c >= 128; c -= GK) {
+      const int64_t items = d.ntiles * ((m + c - 1) / c), cost = (items + SMS - 1) / SMS * (std::min<int64_t>(c, m) + 100);
+      if (cost < best) { best = cost; d.chunk = c; }
+    }
+  }
+  d.nchunks = (int)((m + d.chunk - 1) / d.chunk);
   return d;
 }
 
@@ -482,6 +554,7 @@ bool gram_tc_params(GramTcParams& prm, const GramTcDims& d, const GramTcBufs& bu
   prm.nB = d.nB;
   prm.L4p = d.L4p;
   prm.kiters = d.kiters;
+  prm.cstages = d.chunk / GK;
   prm.err = err;
   return true;
 }
@@ -490,8 +563,8 @@ bool gram_tc_params(GramTcParams& prm, const GramTcDims& d, const GramTcBufs& bu
 
 namespace qlr {
 
-size_t gram_tc_ws(int64_t m, int l) {
-  const GramTcDims d = gram_tc_dims(m, l);
+size_t gram_tc_ws(int64_t m, int l, bool single) {
+  const GramTcDims d = gram_tc_dims(m, l, single);
   return rup256((size_t)8 * d.L4p * d.mp * 2) + rup256((size_t)d.L4p * 4) + rup256((size_t)d.nchunks * d.L4 * d.L4 * 8);
 }
 
@@ -499,16 +572,16 @@ bool gram_tc_supported(const qlr_qmat& Y) {
   if (Y.dtype != QLR_F32 || Y.layout != QLR_COL_MAJOR || Y.rows <= 0 || Y.cols <= 0) return false;
   for (int c = 0; c < 4; ++c)
     if (Y.plane[c] == nullptr) return false;
-  const GramTcDims d = gram_tc_dims(Y.rows, (int)Y.cols);
+  const GramTcDims d = gram_tc_dims(Y.rows, (int)Y.cols, false);
   return Y.cols <= 1024 && (int64_t)8 * d.L4p < (1 << 30) && d.nchunks < 65536 && get_encode() != nullptr;
 }
 
 int gram_tc(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws) {
   const int64_t m = Y.rows;
   const int l = (int)Y.cols;
-  const GramTcDims d = gram_tc_dims(m, l);
+  const GramTcDims d = gram_tc_dims(m, l, true);
   const size_t mark = ws.off;
-  char* base = ws.take<char>(gram_tc_ws(m, l));
+  char* base = ws.take<char>(gram_tc_ws(m, l, true));
   if (!ws.ok) { ws.off = mark; ws.ok = true; return QLR_ENOMEM; }
   const GramTcBufs bufs = gram_tc_carve(base, d, 7);
   __nv_bfloat16* S = bufs.S;
@@ -526,7 +599,8 @@ int gram_tc(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws) {
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
   QLR_CUDA_TRY(cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem(7)));
-  gram_tc_kernel<<<dim3((unsigned)d.ntiles, (unsigned)d.nchunks), GTHREADS, gsmem(7), ctx->stream>>>(prm);
+  const int nitems = d.ntiles * d.nchunks, sms = ctx->num_sms > 0 ? ctx->num_sms : 148;
+  gram_tc_kernel<<<(unsigned)std::min(nitems, sms), GTHREADS, gsmem(7), ctx->stream>>>(prm, d.ntiles, nitems);
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
   const int64_t ntri = (int64_t)l * (l + 1) / 2;
@@ -541,7 +615,7 @@ size_t gram_tc_record_bytes() { return sizeof(GramTcProb); }
 
 int gram_tc_record(void* dst, const qlr_qmat& Y, char* scratch, float* G, int* err) {
   const int l = (int)Y.cols;
-  const GramTcDims d = gram_tc_dims(Y.rows, l);
+  const GramTcDims d = gram_tc_dims(Y.rows, l, false);
   const GramTcBufs bufs = gram_tc_carve(scratch, d, 8);
   GramTcProb r;
   memset(&r, 0, sizeof(r));
@@ -561,7 +635,7 @@ int gram_tc_record(void* dst, const qlr_qmat& Y, char* scratch, float* G, int* e
 
 void gram_tc_grouped_items(int64_t m, int l, int prob, std::vector<int4>& slice, std::vector<int4>& mma,
                            std::vector<int4>& comb) {
-  const GramTcDims d = gram_tc_dims(m, l);
+  const GramTcDims d = gram_tc_dims(m, l, false);
   for (int g = 0; g < (d.L4p + 7) / 8; ++g) slice.push_back(make_int4(prob, g, 0, 0));
   for (int ch = 0; ch < d.nchunks; ++ch)
     for (int t = 0; t < d.ntiles; ++t) mma.push_back(make_int4(prob, t, ch, 0));
@@ -577,7 +651,8 @@ int gram_tc_grouped(qlr_ctx* ctx, const void* d_probs, const int4* slice, int n_
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
   QLR_CUDA_TRY(cudaFuncSetAttribute(gram_tc_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem(8)));
-  gram_tc_grouped_kernel<<<n_mma, GTHREADS, gsmem(8), ctx->stream>>>(probs, mma);
+  gram_tc_grouped_kernel<<<std::min(n_mma, ctx->num_sms > 0 ? ctx->num_sms : 148), GTHREADS, gsmem(8), ctx->stream>>>(
+      probs, mma, n_mma, ctx->d_err);
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
   gram_tc_combine_grouped_kernel<<<n_comb, 128, 0, ctx->stream>>>(probs, comb);

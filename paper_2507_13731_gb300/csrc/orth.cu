@@ -1877,7 +1877,7 @@ static int gram_df32(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws) {
 int gram(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws) {
   if (Y.dtype == QLR_F32 && Y.cols > 0 && Y.rows > 0) {
     // tensor cores when the workspace holds the slices, else the double-FP32 SIMT Gram
-    if (gram_tc_supported(Y) && ws.cap - ws.off >= gram_tc_ws(Y.rows, (int)Y.cols)) return gram_tc(ctx, Y, G, ws);
+    if (gram_tc_supported(Y) && ws.cap - ws.off >= gram_tc_ws(Y.rows, (int)Y.cols, true)) return gram_tc(ctx, Y, G, ws);
     return gram_df32(ctx, Y, G, ws);
   }
   const int l = (int)Y.cols;

@@ -207,7 +207,7 @@ int sketch_tc_grouped_run(qlr_ctx* ctx, const GroupedSketch& gs);
 // orthonormalisation pieces (orth.cu)
 int gram(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws);
 // FP64-class Gram of FP32 Y on the tensor cores by exact BF16 slicing (gram_tc.cu); G FP64 planes.
-size_t gram_tc_ws(int64_t m, int l);
+size_t gram_tc_ws(int64_t m, int l, bool single);   // single: gram_tc's, else a batch plan's problem
 bool gram_tc_supported(const qlr_qmat& Y);
 int gram_tc(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws);
 // Batch plans (grouped launches): a per-problem record of gram_tc_record_bytes() bytes (64-byte
