@@ -1185,13 +1185,25 @@ Plan make_plan(int compute, int op, int64_t M, int64_t K, int l, int num_sms, bo
   pl.bk = pl.sw / pl.esz;
   pl.mtiles = (int)((M + TBM - 1) / TBM);
   pl.kiters = (int)((K + pl.bk - 1) / pl.bk);
-  // Stream-K over every SM (each CTA at least 8 stages) when the tiles do not fill whole waves:
+  // Stream-K over every SM (each CTA at least 8 stages; shorter pieces below) when the tiles do not fill whole waves:
   // fewer tiles than SMs, or a last wave that would leave SMs idle (e.g. 157 row tiles on 152
   // SMs would take two full tile times).  A CTA's range then holds at most two partial pieces
   // (the tail of one tile and the head of another) around any number of whole tiles.
   const int64_t tiles = (int64_t)pl.mtiles * pl.ncb;
   const int64_t g = std::min<int64_t>(num_sms, tiles * pl.kiters / 8);
-  if (g > tiles) pl.grid_sk = (int)g;
+  // FP32-accurate sketches of few tiles with a short reduction: every tile in the same number of
+  // pieces, as many as the SMs take, down to one stage each.  Their stages are long (three products,
+  // or staged operands rounded on the way), while a CTA whose range crosses a tile boundary pays two
+  // accumulator read-outs; cuts at the boundaries keep it at one.  Over 8 to 170 columns of nine
+  // sizes from 100 x 100 to 3000 x 3000, against ranges of at least 8 stages: 1.32x (geometric mean),
+  // 2.5x for 517 x 389 x 60 rounded (48 -> 19 us), none below 0.99x.  Equal pieces leave up to
+  // num_sms mod tiles SMs idle, which costs 2 % where a piece is longer than 24 stages
+  // (700 x 2500 x 170): such reductions keep one range per SM.  TF32 and BF16 keep their cuts too:
+  // their accumulators truncate, so other cuts give other results.
+  int64_t cuts = 0;
+  if (pl.kind == K_TF32X3 || pl.rn) cuts = std::min<int64_t>(num_sms / tiles, pl.kiters);
+  if (cuts > 1 && pl.kiters < 24 * cuts) pl.grid_sk = (int)(tiles * cuts);
+  else if (g > tiles) pl.grid_sk = (int)g;
   else if (tiles > num_sms && tiles % num_sms != 0 && g == num_sms) pl.grid_sk = num_sms;
   else pl.grid_sk = 0;
   // several column blocks: the stream-K CTAs in groups of one CTA per block (a whole number of
