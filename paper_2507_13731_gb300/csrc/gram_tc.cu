@@ -167,14 +167,6 @@ __global__ void __launch_bounds__(256) gram_slice_kernel(const float* __restrict
   gram_slice_cols<7, 8>(y0, y1, y2, y3, m, l, ld, L4p, mp, S, ex, blockIdx.x);
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-      : "memory");
-}
-
 // (s, e) += x exactly into a two-float sum (Knuth's two-sum, the rounding error kept in e).
 __device__ __forceinline__ void two_sum_acc(float& s, float& e, float x) {
   const float t = __fadd_rn(s, x);
@@ -216,7 +208,7 @@ __device__ __forceinline__ void gram_tc_items(const int nitems, Item item, int* 
   auto a_tile = [&](int s, int i) { return smem + s * STAGE_BYTES + i * A_TILE; };
   auto b_tile = [&](int s, int j) { return smem + s * STAGE_BYTES + GS * A_TILE + j * B_TILE; };
 
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   if (threadIdx.x == 0) {
     for (int s = 0; s < GSTAGES; ++s) {
       mbar_init(&full[s], 1);
@@ -269,7 +261,8 @@ __device__ __forceinline__ void gram_tc_items(const int nitems, Item item, int* 
     }
   } else if (warp == GEPI + 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    {   // the whole warp, MMAs by one elected lane
+      const uint32_t lead = elect_one();
       // BF16 A and B, FP32 D, both K-major, M = GA; N = t GB for t consecutive B slices: the B
       // slice tiles are adjacent in shared memory, and one MMA of A_i against slices j .. j+t-1
       // writes pair (i, j + u) to TMEM columns (i + j + u) GB, the accumulator of its weight group
@@ -284,12 +277,12 @@ __device__ __forceinline__ void gram_tc_items(const int nitems, Item item, int* 
         const GramTcParams* pp;
         const GramTile g = item(x, pp, false);
         if (done > 0) {
-          ok = mbar_wait(tmem_empty, (done - 1) & 1u, abort_flag, err);
+          ok = mbar_wait_warp(tmem_empty, (done - 1) & 1u, abort_flag, err);
           if (!ok) break;
         }
         tc_fence_after();
         for (int i = 0; i < g.nit; ++i) {
-          ok = mbar_wait(&full[s], ph, abort_flag, err);
+          ok = mbar_wait_warp(&full[s], ph, abort_flag, err);
           if (!ok) break;
           tc_fence_after();
           const uint64_t so = (uint64_t)(s * (STAGE_BYTES >> 4));
@@ -305,14 +298,14 @@ __device__ __forceinline__ void gram_tc_items(const int nitems, Item item, int* 
                 const uint32_t idesc = idesc0 | ((uint32_t)((t * GB) >> 3) << 17);
                 // first products of the weight groups in this chunk: qi == 0, first stage and k-step
                 const uint32_t acc = (i > 0 || ks > 0 || qi > 0) ? 1u : 0u;
-                umma_bf16(tmem + (uint32_t)((qi + qj) * GB), ad, bd, idesc, acc);
+                umma_bf16(lead, tmem + (uint32_t)((qi + qj) * GB), ad, bd, idesc, acc);
               }
             }
           }
-          umma_commit(&empty[s]);   // frees the stage once these MMAs have read it
+          umma_commit(lead, &empty[s]);   // frees the stage once these MMAs have read it
           if (++s == GSTAGES) { s = 0; ph ^= 1u; }
         }
-        umma_commit(tmem_full);     // accumulators complete (also fires after an abort)
+        umma_commit(lead, tmem_full);     // accumulators complete (also fires after an abort)
       }
     }
   } else {

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(128, 1) mma_peak_kernel(int64_t rounds, int* e
               : "memory");
       }
     }
-    umma_commit(done);
+    umma_commit(1u, done);
   }
   __syncwarp();
   // every thread waits (bounded) for the last MMA, then warp 0 reads one accumulator row

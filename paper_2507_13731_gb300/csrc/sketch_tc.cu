@@ -128,20 +128,10 @@ __device__ __forceinline__ uint4 tf32_rna4(uint4 v) {
 
 // ---------------------------------------------------------------------------------------
 template <int KIND>
-__device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
-  if (KIND == K_BF16) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-        : "memory");
-  } else {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-        : "memory");
-  }
+__device__ __forceinline__ void umma(uint32_t lead, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                     uint32_t accum) {
+  if (KIND == K_BF16) umma_bf16(lead, d_tmem, adesc, bdesc, idesc, accum);
+  else umma_tf32(lead, d_tmem, adesc, bdesc, idesc, accum);
 }
 // Stage geometry.  WIDE (K-major A, column blocks of at most 64): 128-byte rows per stage (128 B
 // swizzle), so every TMA row fetch of A moves 128 contiguous bytes; otherwise 64-byte rows.
@@ -164,41 +154,43 @@ template <> struct Cfg<K_TF32X3, false> {   // 4-byte operands, 32 B swizzle, 8 
 template <> struct Cfg<K_TF32X3, true> : Cfg<K_TF32X3, false> {};
 
 // ---------------------------------------------------------------------------------------
-// MMA issue.  The shared-memory descriptors of stage 0's operand tiles are built once; stage s
-// and K step ks only move the start address, whose field holds (address >> 4) in the low 14 bits
-// of the descriptor, so they are plain 64-bit additions.  A stage is then issued as a fully
-// unrolled run of tcgen05.mma with no per-MMA address arithmetic: with 64-column blocks an MMA
-// takes ~32 tensor-pipe cycles, so the issuing thread must spend only a few instructions on each.
+// MMA issue.  Every operand tile of a stage lies at a fixed distance from the ring's first, and a
+// shared-memory descriptor holds (address >> 4) in its low bits, so a tile's descriptor is the low
+// word of the ring's first tile plus offsets known at compile time (A planes, K steps) or kept in
+// one register (stage, X tile, lo set) beside a constant high word.  A stage is then issued as a
+// fully unrolled run of tcgen05.mma with two or three 32-bit additions each.  The issue rate, not the
+// tensor pipe, bounded the plain form while one lane ran the loop from per-tile descriptors in local
+// memory; issued by a whole warp (umma_bf16), at 15000 x 6000: 455 -> 301 us (TF32 A^H, 33 columns),
+// 1147 -> 853 us (3xTF32, 33), 488 -> 395 us (BF16, 170), 1.05 to 1.24x over each mode's sizes.
 struct StageDescs {
-  uint64_t a[4], alo[4], x[4], xlo[4];
-  uint64_t sstep;                 // one stage, in descriptor address units (16 bytes)
+  uint32_t a, x;                  // low words of plane 0 of A, X tile 0 of stage 0
+  uint32_t ahi, xhi;              // high words
+  uint32_t alo, xlo, xstep;       // to the lo set of A and of X, from one X tile to the next
+  uint32_t sstep;                 // one stage
 };
 
+// Plane c of A at slot c - (4 - apl), X tile c of the fused set at slot c - x0: a_off and x_off are
+// the sets' offsets less the absent planes, in plain integers (a start below the ring is brought back
+// by the first plane's offset).
 template <int KIND, int AMODE, bool WIDE = false>
-__device__ __forceinline__ StageDescs make_stage_descs(uint32_t sbase, int stage_bytes, int hi_off, int a_bytes,
-                                                       int a_set, int x_bytes, int apl, int nxp) {
+__device__ __forceinline__ StageDescs make_stage_descs(uint32_t sbase, int stage_bytes, int a_off, int x_off,
+                                                       int a_bytes, int x_bytes, int apl, int nxp) {
   using C = Cfg<KIND, WIDE>;
+  // MN-major: LBO = stride between MN atoms, SBO = stride between 8-row K groups
+  const uint64_t ad = make_desc(0, (AMODE == A_MN) ? C::BK * C::SW : 16, 8 * C::SW, C::MODE);
+  const uint64_t xd = make_desc(0, 16, 8 * C::SW, C::MODE);
   StageDescs D;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    // plane c of the hi (and lo) set at slot c - (4 - apl): hi_off is the set's offset minus
-    // (4 - apl) planes; the slots of absent planes are never used
-    const uint32_t ah = sbase + (uint32_t)(hi_off + c * a_bytes), al = ah + (uint32_t)(apl * a_bytes);
-    if (AMODE == A_MN) {   // MN-major: LBO = stride between MN atoms, SBO = stride between 8-row K groups
-      D.a[c] = make_desc(ah, C::BK * C::SW, 8 * C::SW, C::MODE);
-      D.alo[c] = make_desc(al, C::BK * C::SW, 8 * C::SW, C::MODE);
-    } else {
-      D.a[c] = make_desc(ah, 16, 8 * C::SW, C::MODE);
-      D.alo[c] = make_desc(al, 16, 8 * C::SW, C::MODE);
-    }
-    // X tile c of the hi (and lo) set: nxp tiles of x_bytes each
-    const uint32_t xh = sbase + (uint32_t)(a_set + c * x_bytes), xl = xh + (uint32_t)(nxp * x_bytes);
-    D.x[c] = make_desc(xh, 16, 8 * C::SW, C::MODE);
-    D.xlo[c] = make_desc(xl, 16, 8 * C::SW, C::MODE);
-  }
-  D.sstep = (uint64_t)(stage_bytes >> 4);
+  D.a = (uint32_t)ad + (uint32_t)(((int)sbase + a_off) >> 4);
+  D.x = (uint32_t)xd + (uint32_t)(((int)sbase + x_off) >> 4);
+  D.ahi = (uint32_t)(ad >> 32);
+  D.xhi = (uint32_t)(xd >> 32);
+  D.alo = (uint32_t)(apl * a_bytes) >> 4;
+  D.xlo = (uint32_t)(nxp * x_bytes) >> 4;
+  D.xstep = (uint32_t)x_bytes >> 4;
+  D.sstep = (uint32_t)stage_bytes >> 4;
   return D;
 }
+__device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
 
 // All MMAs of stage s into the accumulator at TMEM column abase (output plane d at abase + d nb).
 // Plain form: per K step and input plane c, one MMA per output plane d of A_c against X_{c xor d}
@@ -210,50 +202,44 @@ __device__ __forceinline__ StageDescs make_stage_descs(uint32_t sbase, int stage
 // of the MMAs at four times the width.  `fresh`: the first stage of an accumulation chunk (its
 // first MMA overwrites the accumulator).
 template <int KIND, int AMODE, bool WIDE = false>
-__device__ __forceinline__ void issue_stage(const StageDescs& D, int s, uint32_t abase, int nb, int c_first,
-                                            uint32_t idesc_base, uint32_t neg_mask, bool fresh, int fd, int c0) {
+__device__ __forceinline__ void issue_stage(uint32_t lead, const StageDescs& D, int s, uint32_t abase, int nb, int c_first,
+                                            uint32_t idesc_base, uint32_t neg_mask, bool fresh, int fd) {
   using C = Cfg<KIND, WIDE>;
   constexpr bool X3 = (KIND == K_TF32X3);
   constexpr int KSTEPS = C::BK / C::MMA_K;
-  constexpr uint64_t KA = (AMODE == A_MN) ? (uint64_t)((C::MMA_K * C::SW) >> 4) : (uint64_t)((C::MMA_K * C::ESZ) >> 4);
-  constexpr uint64_t KB = (uint64_t)((C::MMA_K * C::ESZ) >> 4);
-  const uint64_t so = (uint64_t)s * D.sstep;
-  if (fd) {
-#pragma unroll
-    for (int ks = 0; ks < KSTEPS; ++ks) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        if (c < c_first) continue;
-        const uint64_t ad = D.a[c] + so + ks * KA;
-        const uint64_t bd = D.x[c - c0] + so + ks * KB;
-        const uint32_t acc = (!fresh || ks > 0 || c > c_first) ? 1u : 0u;
-        umma<KIND>(abase, ad, bd, idesc_base, acc);
-        if (X3) {
-          umma<KIND>(abase, D.alo[c] + so + ks * KA, bd, idesc_base, 1u);
-          umma<KIND>(abase, ad, D.xlo[c - c0] + so + ks * KB, idesc_base, 1u);
-        }
-      }
-    }
-    return;
-  }
+  constexpr uint32_t KA = (uint32_t)((AMODE == A_MN ? C::MMA_K * C::SW : C::MMA_K * C::ESZ) >> 4);
+  constexpr uint32_t KB = (uint32_t)((C::MMA_K * C::ESZ) >> 4);
+  constexpr uint32_t PA = (uint32_t)((TBM * C::SW) >> 4);   // one A plane
+  const uint32_t as = D.a + (uint32_t)s * D.sstep, xs = D.x + (uint32_t)s * D.sstep;
 #pragma unroll
   for (int ks = 0; ks < KSTEPS; ++ks) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       if (c < c_first) continue;
-      const uint64_t ad = D.a[c] + so + ks * KA;
-      const uint64_t adlo = D.alo[c] + so + ks * KA;
+      const uint32_t al = as + c * PA + ks * KA;
+      const uint64_t ad = desc64(al, D.ahi), adlo = desc64(al + D.alo, D.ahi);
+      const uint32_t acc = (!fresh || ks > 0 || c > c_first) ? 1u : 0u;
+      if (fd) {
+        const uint32_t xl = xs + c * D.xstep + ks * KB;
+        const uint64_t bd = desc64(xl, D.xhi);
+        umma<KIND>(lead, abase, ad, bd, idesc_base, acc);
+        if (X3) {
+          umma<KIND>(lead, abase, adlo, bd, idesc_base, 1u);
+          umma<KIND>(lead, abase, ad, desc64(xl + D.xlo, D.xhi), idesc_base, 1u);
+        }
+        continue;
+      }
 #pragma unroll
       for (int d = 0; d < 4; ++d) {
         const int q = c ^ d;
-        const uint64_t bd = D.x[q] + so + ks * KB;
+        const uint32_t xl = xs + q * D.xstep + ks * KB;
+        const uint64_t bd = desc64(xl, D.xhi);
         const uint32_t idesc = idesc_base | (((neg_mask >> (c * 4 + d)) & 1u) << 14);
         const uint32_t dt = abase + (uint32_t)(d * nb);
-        const uint32_t acc = (!fresh || ks > 0 || c > c_first) ? 1u : 0u;
-        umma<KIND>(dt, ad, bd, idesc, acc);
+        umma<KIND>(lead, dt, ad, bd, idesc, acc);
         if (X3) {
-          umma<KIND>(dt, adlo, bd, idesc, 1u);
-          umma<KIND>(dt, ad, D.xlo[q] + so + ks * KB, idesc, 1u);
+          umma<KIND>(lead, dt, adlo, bd, idesc, 1u);
+          umma<KIND>(lead, dt, ad, desc64(xl + D.xlo, D.xhi), idesc, 1u);
         }
       }
     }
@@ -319,7 +305,7 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
   const int F = pv.flush > 0 ? pv.flush : (1 << 30);
   const int NBUF = pv.nbuf;
 
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const int EPI = pv.epi2 ? 2 : 1;                     // epilogue warps per lane quarter
   // worker pairs: warps 2-3, then those from warp 8 on that are not epilogue warps
   const int NPAIR = WORKERS ? 1 + ((int)blockDim.x - TC_THREADS - (pv.epi2 ? 128 : 0)) / 64 : 0;
@@ -415,36 +401,37 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    {   // the whole warp, MMAs by one elected lane
+      const uint32_t lead = elect_one();
       bool ok = true;
       int chunk = 0, buf = 0, ic = 0, s = 0;       // chunk, its buffer, stage within it, ring slot
       uint32_t ph = 0;
       const int nb_log = NBUF - 1;                 // NBUF is 1 or 2
       const StageDescs D = make_stage_descs<KIND, AMODE, WIDE>(smem_u32(smem), stage_bytes, HI_OFF - C0 * A_BYTES,
-                                                               A_BYTES, A_SET, X_BYTES, APL, NXP);
+                                                               A_SET - (FD ? C0 * X_BYTES : 0), A_BYTES, X_BYTES, APL, NXP);
 #pragma unroll 1
       for (int i = 0; i < nit; ++i) {
         if (ic == F) {                             // chunk boundary: hand the finished chunk over
-          umma_commit(&tmem_full[buf]);
+          umma_commit(lead, &tmem_full[buf]);
           ++chunk;
           buf = chunk & nb_log;
           ic = 0;
           if (chunk >= NBUF) {                     // its buffer must have been drained first
-            ok = mbar_wait(&tmem_empty[buf], (uint32_t)((chunk >> nb_log) - 1) & 1u, abort_flag, pv.err);
+            ok = mbar_wait_warp(&tmem_empty[buf], (uint32_t)((chunk >> nb_log) - 1) & 1u, abort_flag, pv.err);
             if (!ok) break;
             tc_fence_after();
           }
         }
         const uint32_t abase = tmem + (uint32_t)(buf * 4 * nb);
-        ok = mbar_wait(WORKERS ? &ready[s] : &full[s], ph, abort_flag, pv.err);
+        ok = mbar_wait_warp(WORKERS ? &ready[s] : &full[s], ph, abort_flag, pv.err);
         if (!ok) break;
         tc_fence_after();
-        issue_stage<KIND, AMODE, WIDE>(D, s, abase, nb, pv.c_first, pv.idesc_base, pv.neg_mask, ic == 0, pv.fd, C0);
-        umma_commit(&empty[s]);   // frees the stage once these MMAs have read it
+        issue_stage<KIND, AMODE, WIDE>(lead, D, s, abase, nb, pv.c_first, pv.idesc_base, pv.neg_mask, ic == 0, pv.fd);
+        umma_commit(lead, &empty[s]);   // frees the stage once these MMAs have read it
         ++ic;
         if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
-      umma_commit(&tmem_full[buf]);   // last chunk complete (also fires after an abort)
+      umma_commit(lead, &tmem_full[buf]);   // last chunk complete (also fires after an abort)
     }
   } else if (warp < 4 || warp >= (pv.epi2 ? 12 : 8)) {
     // ---------------- workers: hi/lo split (3xTF32) and/or transpose of A ----------------
@@ -766,7 +753,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * PMAX_STAGES + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const int my_items = (nitems - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
   const int HI_OFF = 0;
   auto raw_plane = [&](int s, int c) { return smem + s * stage_bytes + (c - c0) * A_BYTES; };   // = a_plane
@@ -859,11 +846,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    {   // the whole warp, MMAs by one elected lane
+      const uint32_t lead = elect_one();
       int g = 0;
       bool ok = true;
       const StageDescs D = make_stage_descs<KIND, AMODE, WIDE>(smem_u32(smem), stage_bytes, HI_OFF - c0 * A_BYTES,
-                                                               A_BYTES, A_SET, X_BYTES, apl, NXP);
+                                                               A_SET - (fd ? c0 * X_BYTES : 0), A_BYTES, X_BYTES, apl, NXP);
       int prev_nb = 0;
       for (int t = 0; t < my_items && ok; ++t) {
         const int4 it = items[blockIdx.x + t * gridDim.x];
@@ -871,11 +859,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const TcScalars pv = tc_scalars(p);
         const int a = t & 1;
         if (t >= 2) {   // item t - 2 (same end of TMEM) drained
-          ok = mbar_wait(&acc_empty[a], (uint32_t)((t >> 1) - 1) & 1u, abort_flag, err);
+          ok = mbar_wait_warp(&acc_empty[a], (uint32_t)((t >> 1) - 1) & 1u, abort_flag, err);
           if (!ok) break;
         }
         if (t >= 1 && 4 * (pv.nb + prev_nb) > (int)tmem_cols) {   // overlaps item t - 1: wait for its drain
-          ok = mbar_wait(&acc_empty[a ^ 1], (uint32_t)((t - 1) >> 1) & 1u, abort_flag, err);
+          ok = mbar_wait_warp(&acc_empty[a ^ 1], (uint32_t)((t - 1) >> 1) & 1u, abort_flag, err);
           if (!ok) break;
         }
         if (t >= 1) tc_fence_after();
@@ -884,13 +872,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         for (int i = 0; i < pv.kiters; ++i, ++g) {
           const int s = g % STAGES;
           const uint32_t ph = (uint32_t)(g / STAGES) & 1u;
-          ok = mbar_wait(WORKERS ? &ready[s] : &full[s], ph, abort_flag, err);
+          ok = mbar_wait_warp(WORKERS ? &ready[s] : &full[s], ph, abort_flag, err);
           if (!ok) break;
           tc_fence_after();
-          issue_stage<KIND, AMODE, WIDE>(D, s, acc_base, pv.nb, pv.c_first, pv.idesc_base, pv.neg_mask, i == 0, fd, c0);
-          umma_commit(&empty[s]);
+          issue_stage<KIND, AMODE, WIDE>(lead, D, s, acc_base, pv.nb, pv.c_first, pv.idesc_base, pv.neg_mask, i == 0, fd);
+          umma_commit(lead, &empty[s]);
         }
-        umma_commit(&acc_full[a]);   // accumulator of item t complete (also after an abort)
+        umma_commit(lead, &acc_full[a]);   // accumulator of item t complete (also after an abort)
       }
     }
   } else if (warp < 4) {

@@ -73,13 +73,6 @@ struct TallArgs {
   int* err;
 };
 
-__device__ __forceinline__ void umma_bf16_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-
 // x = s0 + s1 + s2.  A value that rounds beyond BF16's range is truncated instead; a non-finite
 // value is kept whole in s0.
 __device__ __forceinline__ void split3(float x, __nv_bfloat16 (&s)[3]) {
@@ -186,7 +179,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
   uint64_t* acc_empty = acc_full + TL_ACC;       // [TL_ACC]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + TL_ACC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const int64_t tiles = (int64_t)p.mtiles * p.ntiles;
   const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
   auto ksteps_of = [&](int nt) {
@@ -261,7 +254,8 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
     }
   } else if (warp > TL_EPI) {
     // ---------------- MMA issuers: stages in turn ----------------
-    if (lane == 0) {
+    {   // the whole warp, MMAs by one elected lane
+      const uint32_t lead = elect_one();
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(TL_N >> 3) << 17) |
                              ((uint32_t)(TL_M >> 4) << 24);
       // descriptors of the first stage (later ones move the 16-byte address field): the tall operand
@@ -276,7 +270,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
       for (int left = (int)(t1 - t0); left > 0 && ok; --left) {
         const bool fresh = (mt != cur);             // new rows: their resident operand is on its way
         if (fresh) {
-          if (res && cur >= 0) umma_commit(adone);   // the old one may be overwritten once these MMAs have read it
+          if (res && cur >= 0) umma_commit(lead, adone);   // the old one may be overwritten once these MMAs have read it
           ++nm;
         }
         cur = mt;
@@ -292,10 +286,10 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
           }
           turn = TL_ISSUERS - 1;
           if (res && nm != seen) {                   // new rows: wait for their operand
-            for (int c2 = 0; c2 < nchunks && ok; ++c2) ok = mbar_wait(&afull[c2], (uint32_t)(nm - 1) & 1u, abort_flag, p.err);
+            for (int c2 = 0; c2 < nchunks && ok; ++c2) ok = mbar_wait_warp(&afull[c2], (uint32_t)(nm - 1) & 1u, abort_flag, p.err);
             seen = nm;
           }
-          ok = ok && mbar_wait(&full[s], sph, abort_flag, p.err);
+          ok = ok && mbar_wait_warp(&full[s], sph, abort_flag, p.err);
           if (!ok) break;
           const uint64_t ad = adesc0 + (uint64_t)(uint32_t)((res ? ch * TL_OP : s * stage_bytes) >> 4);
           const uint64_t bd = bdesc0 + (uint64_t)(uint32_t)((s * stage_bytes) >> 4);
@@ -303,22 +297,22 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
           // one accumulation chunk: the corrections of its steps [h0, h1), then x0 y0
           auto chunk = [&](auto H0, auto H1) {
             constexpr int h0 = decltype(H0)::value, h1 = decltype(H1)::value;
-            ok = mbar_wait(&acc_empty[b], bph ^ 1u, abort_flag, p.err);
+            ok = mbar_wait_warp(&acc_empty[b], bph ^ 1u, abort_flag, p.err);
             if (!ok) return;
             tc_fence_after();
             const uint32_t acc = tmem + (uint32_t)(b * TL_N);
 #pragma unroll
             for (int h = h0; h < h1; ++h) {
               const uint64_t x = ad + h * KA, y = bd + h * KB;
-              umma_bf16_ss(acc, x, y + 2 * SP, idesc, h > h0);
-              umma_bf16_ss(acc, x + 2 * SP, y, idesc, 1u);
-              umma_bf16_ss(acc, x + SP, y + SP, idesc, 1u);
-              umma_bf16_ss(acc, x, y + SP, idesc, 1u);
-              umma_bf16_ss(acc, x + SP, y, idesc, 1u);
+              umma_bf16(lead, acc, x, y + 2 * SP, idesc, h > h0);
+              umma_bf16(lead, acc, x + 2 * SP, y, idesc, 1u);
+              umma_bf16(lead, acc, x + SP, y + SP, idesc, 1u);
+              umma_bf16(lead, acc, x, y + SP, idesc, 1u);
+              umma_bf16(lead, acc, x + SP, y, idesc, 1u);
             }
 #pragma unroll
-            for (int h = h0; h < h1; ++h) umma_bf16_ss(acc, ad + h * KA, bd + h * KB, idesc, 1u);
-            umma_commit(&acc_full[b]);
+            for (int h = h0; h < h1; ++h) umma_bf16(lead, acc, ad + h * KA, bd + h * KB, idesc, 1u);
+            umma_commit(lead, &acc_full[b]);
             if (++b == TL_ACC) { b = 0; bph ^= 1u; }
           };
           using I0 = std::integral_constant<int, 0>;
@@ -331,7 +325,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
             if (ok && 2 * ch + 1 < ks_n) chunk(I1{}, I2{});
           }
           if (!ok) break;
-          umma_commit(&empty[s]);
+          umma_commit(lead, &empty[s]);
           if (++s == stages) { s = 0; sph ^= 1u; }
         }
         if (++nt == p.ntiles) { nt = 0; ++mt; }
