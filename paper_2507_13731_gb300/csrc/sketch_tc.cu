@@ -1145,33 +1145,45 @@ Plan make_plan(int compute, int op, int64_t M, int64_t K, int l, int num_sms, bo
   const int max_nb = (pl.kind == K_TF32X3) ? X3_MAX_NB : 128;
   pl.ncb = (lp + max_nb - 1) / max_nb;
   pl.nb = ((lp + pl.ncb - 1) / pl.ncb + 15) / 16 * 16;
-  // fused output planes when one MMA of N = 4 nb fits (nb <= 64): a quarter of the MMAs, but a
-  // fused X set (4 - c0) times larger; kept only while the ring still holds 3 stages (with two, the
-  // transposed-A form lost more to exposed loads than it gained: 1.16 against 0.87 ms at
-  // 20000 x 10000 x 60, TF32 op H)
+  // Fused output planes (one MMA of N = 4 nb, nb <= 64): a quarter of the MMAs, but a staged operand
+  // (4 - c0) times larger, read by every row tile through L2; only while the ring still holds 3 stages
+  // (with two, the transposed-A form lost more to exposed loads than it gained: 1.16 against 0.87 ms
+  // at 20000 x 10000 x 60, TF32 op H).
+  //  - Blocks of at most 32 columns: fused (15 columns of a pure 15000 x 6000, fused against plain: 183
+  //    and 214 us TF32 N, 471 and 632 us 3xTF32 N, 98 and 116 us BF16 N).
+  //  - Wider blocks: plain, which reads a third of the operand (60 columns of the same: 168 to 151 us
+  //    BF16 N, 228 to 175 us BF16 H, 280 to 267 us TF32 H), except 3xTF32 (656 against 720 us), whose
+  //    operand is split in two either way, and TF32 of A itself: its plain form runs best in 128-byte
+  //    rows, whose other cuts of the reduction give a truncating accumulator other results.
   const bool x3 = pl.kind == K_TF32X3;
-  const bool chunked = x3 || pl.rn;   // accumulation in chunks (FP32-accurate modes)
   const size_t budget = (size_t)227 * 1024 - 1024 - 256;
   const int sw0 = x3 ? 32 : 64;
   const size_t aset = (size_t)apl * TBM * sw0 * (x3 ? 2 : 1);
-  pl.fd = allow_fd && pl.nb <= 64 && budget / (aset + (size_t)apl * 4 * pl.nb * sw0 * (x3 ? 2 : 1)) >= 3;
-  if (allow_fd && !pl.fd && chunked && pl.ncb >= 2) {
-    // 3xTF32 (or rounded TF32) over several column blocks anyway: fused planes in blocks of <= 64
-    // (one more read of A, but a quarter of the MMAs and the chunk sums kept in TMEM): 5.27
-    // against 6.02 ms at 20000 x 10000 x 180, 3xTF32 op N
+  const bool fits = allow_fd && pl.nb <= 64 && budget / (aset + (size_t)apl * 4 * pl.nb * sw0 * (x3 ? 2 : 1)) >= 3;
+  pl.fd = fits && (pl.nb <= 32 || x3 || (pl.kind == K_TF32 && pl.amode == A_K));
+  if (allow_fd && !fits && pl.rn && pl.ncb >= 2) {
+    // rounded TF32 over several column blocks anyway: blocks of <= 64 (one more read of A, the chunk
+    // sums kept in TMEM).  Pure 15000 x 6000 x 170: 857 us fused in such blocks against 944 plain and
+    // 1021 in two blocks of 96 for A itself; 833 plain against 1090 fused and 953 for A^H.  (3xTF32
+    // stays with the fewest blocks: 2081 against 2115 us, 2064 against 2333.)
     const int ncb = (lp + 63) / 64, nb = ((lp + ncb - 1) / ncb + 15) / 16 * 16;
-    if (budget / (aset + (size_t)apl * 4 * nb * sw0 * (x3 ? 2 : 1)) >= 3) {
+    if (budget / (aset + (size_t)apl * 4 * nb * sw0) >= 3) {
       pl.ncb = ncb;
       pl.nb = nb;
-      pl.fd = true;
+      pl.fd = pl.amode == A_K;
     }
   }
+  pl.mtiles = (int)((M + TBM - 1) / TBM);
+  // 128-byte rows double the stage: with 2+ stages of the fused operand where that would fit (the
+  // choice, and with it the cuts of the reduction, does not depend on the form).  Rounded TF32, whose
+  // workers sit between the load and the MMAs, wants 3+ where tiles are many: 395 -> 340 and 411 ->
+  // 369 us for 46 and 60 columns of 15000 x 6000, 49 -> 46 us at 9000 x 700, but 58 -> 60 us at
+  // 3000 x 3000 and 20 -> 22 us at 1500 x 600.
   pl.wide = allow_wide && (pl.amode == A_K) && (pl.kind != K_TF32X3) && (pl.nb <= 64);
-  if (pl.wide && pl.fd)   // 128-byte rows double the stage: only with 2+ stages
-    pl.wide = budget / (2 * (aset + (size_t)apl * 4 * pl.nb * sw0)) >= 2;
+  if (pl.wide && (fits || pl.fd)) pl.wide = budget / (2 * (aset + (size_t)apl * 4 * pl.nb * sw0)) >= 2;
+  if (pl.wide && pl.rn && !pl.fd && pl.mtiles >= 48) pl.wide = budget / (2 * (aset + (size_t)4 * pl.nb * sw0)) >= 3;
   pl.sw = pl.kind == K_TF32X3 ? 32 : (pl.wide ? 128 : 64);
   pl.bk = pl.sw / pl.esz;
-  pl.mtiles = (int)((M + TBM - 1) / TBM);
   pl.kiters = (int)((K + pl.bk - 1) / pl.bk);
   // Stream-K over every SM (each CTA at least 8 stages; shorter pieces below) when the tiles do not fill whole waves:
   // fewer tiles than SMs, or a last wave that would leave SMs idle (e.g. 157 row tiles on 152
