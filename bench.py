@@ -578,10 +578,11 @@ def completion_leg(dev, golden, steps=5):
     flops = 32.0 * m * n * k
     obs = float(P.extra["mask"].mean())
     nbytes = m * n * (1 + 16 + 12 * obs)           # mask, C written, M read at observed entries
-    peak, unit, _, note = peak_for("F32")
+    peak, unit, _, note = peak_for("BF16")         # six BF16 slice products per flop on the tensor cores
     ach = flops / (up_ms / 1e3) / 1e12
-    out["update_kernel"] = {"ms": round(up_ms, 4), "bound": "alu", "achieved": round(ach, 3), "peak": round(peak, 3),
+    out["update_kernel"] = {"ms": round(up_ms, 4), "bound": "tensor", "achieved": round(ach, 3), "peak": round(peak, 3),
                             "unit": "TFLOP/s", "frac": round(ach / peak, 4), "peak_source": note,
+                            "products_per_flop": 6, "frac_of_own_ceiling": round(6.0 * ach / peak, 4),
                             "algorithmic_flops_per_launch": flops, "algorithmic_bytes_per_launch": nbytes,
                             "hbm_gbs": round(nbytes / (up_ms / 1e3) / 1e9, 1)}
     out["device_error"] = rc
