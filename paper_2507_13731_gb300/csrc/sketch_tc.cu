@@ -20,13 +20,14 @@
 // it into hi / lo on the way for 3xTF32).
 // Warp roles: 0 = TMA producer, 1 = MMA issuer (owns TMEM), 2-3 = a pair of workers (hi/lo split,
 // rounding and/or transpose of A), 4-7 = epilogue (TMEM -> registers -> global, or a stream-K
-// partial); with 384 threads, 8-11 = two more worker pairs or four more
-// epilogue warps.
-// The MMA issuer is one thread, and what it does between two stages' MMAs leaves the tensor pipe
-// idle: its ring and chunk positions are counters (the integer divisions they replace took 300 of a
-// stage's 1700 cycles in plain TF32).  Measured (Y = A X and Z = A^H W together, with the staging):
-// 3xTF32 4096 x 4096 x 110 761 -> 630 us, BF16 16384 x 8192 x 220 1638 -> 1522 us, TF32 pure
-// 20000 x 10000 x 60 1431 -> 1348 us, rounded TF32 x 180 5021 -> 4736 us.
+// partial); with 384 threads, 8-11 = two more worker pairs or four more epilogue warps.
+// What the MMA issuer does between two stages' MMAs leaves the tensor pipe idle: its ring and chunk
+// positions are counters (the integer divisions they replace took 300 of a stage's 1700 cycles in
+// plain TF32), and the whole warp runs its loop with one elected lane issuing (see umma_bf16).
+// Measured (Y = A X and Z = A^H W together, with the staging; one lane with divisions, with counters,
+// and now with the choice of form below): 3xTF32 4096 x 4096 x 110 761, 630, 525 us, BF16 16384 x
+// 8192 x 220 1638, 1522, 1277 us, TF32 pure 20000 x 10000 x 60 1431, 1348, 1201 us, rounded TF32
+// x 180 5021, 4736, 3796 us.
 //
 // Precision modes: BF16 (kind::f16, A stored BF16, X rounded to BF16), TF32 (kind::tf32, one
 // product on FP32 data, which the tensor cores truncate to TF32), rounded TF32 (one product, A and
@@ -1185,9 +1186,9 @@ Plan make_plan(int compute, int op, int64_t M, int64_t K, int l, int num_sms, bo
   pl.sw = pl.kind == K_TF32X3 ? 32 : (pl.wide ? 128 : 64);
   pl.bk = pl.sw / pl.esz;
   pl.kiters = (int)((K + pl.bk - 1) / pl.bk);
-  // Stream-K over every SM (each CTA at least 8 stages; shorter pieces below) when the tiles do not fill whole waves:
-  // fewer tiles than SMs, or a last wave that would leave SMs idle (e.g. 157 row tiles on 152
-  // SMs would take two full tile times).  A CTA's range then holds at most two partial pieces
+  // Stream-K over every SM (each CTA at least 8 stages; shorter pieces below) when the tiles do not
+  // fill whole waves: fewer tiles than SMs, or a last wave that would leave SMs idle (e.g. 157 row
+  // tiles on 152 SMs would take two full tile times).  A CTA's range then holds at most two partial pieces
   // (the tail of one tile and the head of another) around any number of whole tiles.
   const int64_t tiles = (int64_t)pl.mtiles * pl.ncb;
   const int64_t g = std::min<int64_t>(num_sms, tiles * pl.kiters / 8);
