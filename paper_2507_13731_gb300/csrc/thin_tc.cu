@@ -263,14 +263,23 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
       // factor K-major, 64-byte rows
       const uint64_t adesc0 = make_desc(smem_u32(res ? smem : ring), TL_SPLIT / 2, 1024, 2);
       const uint64_t bdesc0 = make_desc(smem_u32(res ? ring : ring + TL_OP), 16, 512, 4);
-      int cur = -1, nm = 0, s = 0, b = 0, turn = warp - TL_EPI - 1, seen = 0;
-      uint32_t sph = 0, bph = 0;                // phases of the ring and of the accumulators
+      int cur = -1, nm = 0, s = 0, b = 0, turn = warp - TL_EPI - 1;
+      // Phases of the ring and of the accumulators.  An issuer skips the other's stages without waiting, and
+      // yet none of its waits by parity is two phases behind: the ring holds an even number of stages
+      // (TL_MAX_STAGES), so a slot is always the same issuer's; of the accumulators between two uses of one,
+      // at most two belong to a stage of the other issuer, so this one has waited for the drain of a
+      // later one than the use before the last, and they are drained in order.
+      uint32_t sph = 0, bph = 0;
       bool ok = true;
       int mt = (int)(t0 / p.ntiles), nt = (int)(t0 % p.ntiles);
       for (int left = (int)(t1 - t0); left > 0 && ok; --left) {
-        const bool fresh = (mt != cur);             // new rows: their resident operand is on its way
-        if (fresh) {
-          if (res && cur >= 0) umma_commit(lead, adone);   // the old one may be overwritten once these MMAs have read it
+        if (res && mt != cur) {   // new rows: their resident operand is on its way
+          if (cur >= 0) umma_commit(lead, adone);   // the old one may be overwritten once these MMAs have read it
+          // Both issuers wait for every phase of afull, also one whose rows have no stage for them (a range
+          // that begins on the last column tile of its rows): a wait by parity would take a phase not yet
+          // begun for one that is over.
+          for (int c2 = 0; c2 < nchunks && ok; ++c2) ok = mbar_wait_warp(&afull[c2], (uint32_t)nm & 1u, abort_flag, p.err);
+          if (!ok) break;
           ++nm;
         }
         cur = mt;
@@ -285,11 +294,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
             continue;
           }
           turn = TL_ISSUERS - 1;
-          if (res && nm != seen) {                   // new rows: wait for their operand
-            for (int c2 = 0; c2 < nchunks && ok; ++c2) ok = mbar_wait_warp(&afull[c2], (uint32_t)(nm - 1) & 1u, abort_flag, p.err);
-            seen = nm;
-          }
-          ok = ok && mbar_wait_warp(&full[s], sph, abort_flag, p.err);
+          ok = mbar_wait_warp(&full[s], sph, abort_flag, p.err);
           if (!ok) break;
           const uint64_t ad = adesc0 + (uint64_t)(uint32_t)((res ? ch * TL_OP : s * stage_bytes) >> 4);
           const uint64_t bd = bdesc0 + (uint64_t)(uint32_t)((s * stage_bytes) >> 4);
@@ -462,7 +467,7 @@ int run_gemm(qlr_ctx* ctx, TallArgs& p, const __nv_bfloat16* A, const __nv_bfloa
   p.resident = (p.Kq <= TL_RES_CHUNKS * TL_BK && p.ntiles > 1) ? 1 : 0;
   const size_t budget = (size_t)227 * 1024 - 1024 - 256;
   const size_t ares = p.resident ? (size_t)(p.Kq / TL_BK) * TL_OP : 0, stage = p.resident ? TL_OP : 2 * TL_OP;
-  p.stages = (int)std::min<size_t>(TL_MAX_STAGES, (budget - ares) / stage);
+  p.stages = (int)std::min<size_t>(TL_MAX_STAGES, (budget - ares) / stage / 2 * 2);   // even: see the issuers
   p.per = (p.K <= 64) ? 1 : 2;
   const int64_t ldo = round_up(p.M, 8);
   if (!encode_2d(&p.tmA, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (uint64_t)p.M, (uint64_t)3 * p.Kq, (uint64_t)ldo * 2, 64,
