@@ -120,7 +120,8 @@ typedef struct qlr_ctx qlr_ctx;
 int qlr_create(qlr_ctx** ctx, int device, void* stream);
 /* Synchronise, free the workspace and the context.  ctx may be NULL. */
 int qlr_destroy(qlr_ctx* ctx);
-/* Change the stream later calls are issued on. */
+/* Change the stream later calls are issued on.  All calls but qlr_qcomplete_update share the workspace, and
+ * calls on the old stream may still be using it: make the new stream wait for them first. */
 int qlr_set_stream(qlr_ctx* ctx, void* stream);
 /* Make sure the workspace holds at least `bytes` bytes (cudaMalloc now, never inside a call). */
 int qlr_reserve(qlr_ctx* ctx, size_t bytes);
@@ -379,7 +380,13 @@ int qlr_residual_norm(qlr_ctx* ctx, const qlr_qmat* A, const qlr_qmat* Q, int si
  * mask_ld >= n, non-zero = observed.  U: m x k and V: n x k column-major in the dtype of C (only
  * their first k columns are read); S: device FP64, k values.  k = 0 (U, S, V may be NULL) writes
  * the starting point P_Omega(M), zero at the unobserved entries.  The rank-k product is formed
- * tile by tile in registers (FP32 for F32, FP64 for F64) and never stored.
+ * tile by tile and never stored: F64 in FP64; F32 in FP32, or from m n k of about 15e6 on (k <= 256) on
+ * the tensor cores, every operand entry split into three BF16 values and FP32 sums (no further from the
+ * exact product than FP32 multiply-adds).  The splits (at most ~61 MB for n <= 10000, k <= 50) live in
+ * memory of their own, not in the workspace: allocated with cudaMalloc on first need, grown on demand
+ * (which waits for the update before), freed with the context; updates on several streams are ordered
+ * by an event.  A call on a capturing stream, or one that finds no memory, uses the FP32 pipes
+ * instead, whose results differ within FP32 rounding.
  * Errors: QLR_EINVAL (null pointers, layouts, dtypes), QLR_ESHAPE (sizes, k < 0),
  * QLR_EUNSUPPORTED (more than 65535 * 32 rows).
  */

@@ -346,15 +346,46 @@ size_t lowrank_ws(int64_t m, int64_t n, int k, int p, int v, int algo, int compu
   return b;
 }
 
-// The masked update; FP32 updates on the tensor cores where the workspace holds their operands.
-int masked_update(qlr_ctx* ctx, const qlr::CompleteArgs& a, int dtype) {
-  if (dtype == QLR_F32 && qlr::masked_update_tc_wanted(a.m, a.n, a.k) &&
-      qlr_try_ws(ctx, qlr::masked_update_tc_ws(a.m, a.n, a.k))) {
-    WsArena ws(ctx->ws, ctx->ws_bytes);
+// The masked update with the operands' splits in `buf`; on the FP32 (FP64) pipe where there is no room.
+int masked_update(qlr_ctx* ctx, const qlr::CompleteArgs& a, int dtype, void* buf, size_t bytes) {
+  if (dtype == QLR_F32 && qlr::masked_update_tc_wanted(a.m, a.n, a.k) && bytes >= qlr::masked_update_tc_ws(a.m, a.n, a.k)) {
+    WsArena ws(buf, bytes);
     const int rc = qlr::masked_update_tc(ctx, a, ws);
     if (rc != QLR_ENOMEM) return rc;
   }
   return qlr::complete_update(ctx, a, dtype);
+}
+
+// Memory of its own for an update's splits, ready for use on the context's stream: an update then races
+// with no other call, whatever stream or graph that runs on, and frees nothing a graph holds.  False when
+// there is none: no memory, or a capturing stream (whose graph may be replayed beside later updates).
+bool update_scratch(qlr_ctx* ctx, size_t bytes) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &st) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (st != cudaStreamCaptureStatusNone) return false;
+  if (!ctx->upd_done && cudaEventCreateWithFlags(&ctx->upd_done, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->upd_done = nullptr;
+    return false;
+  }
+  if (ctx->upd_bytes < bytes) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // another thread's capture is not disturbed
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    void* p = nullptr;
+    const bool ok = cudaMalloc(&p, bytes) == cudaSuccess;
+    if (ok && ctx->upd) {
+      cudaEventSynchronize(ctx->upd_done);
+      cudaFree(ctx->upd);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!ok) { cudaGetLastError(); return false; }
+    ctx->upd = p;
+    ctx->upd_bytes = bytes;
+  } else if (cudaStreamWaitEvent(ctx->stream, ctx->upd_done, 0) != cudaSuccess) {   // an update on another stream
+    cudaGetLastError();
+    return false;
+  }
+  return true;
 }
 
 }  // namespace
@@ -422,22 +453,6 @@ int qlr_ensure_ws(qlr_ctx* ctx, size_t bytes) {
   return QLR_OK;
 }
 
-bool qlr_try_ws(qlr_ctx* ctx, size_t bytes) {
-  if (ctx->ws_bytes >= bytes) return true;
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(ctx->stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
-  }
-  void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); return false; }
-  if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) { cudaFree(p); return false; }
-  if (ctx->ws) cudaFree(ctx->ws);
-  ctx->ws = p;
-  ctx->ws_bytes = bytes;
-  return true;
-}
-
 extern "C" {
 
 int qlr_create(qlr_ctx** out, int device, void* stream) {
@@ -488,6 +503,8 @@ int qlr_destroy(qlr_ctx* ctx) {
   resolve_pending(ctx);
   for (auto e : ctx->ev_pool) cudaEventDestroy(e);
   if (ctx->ws) cudaFree(ctx->ws);
+  if (ctx->upd) cudaFree(ctx->upd);
+  if (ctx->upd_done) cudaEventDestroy(ctx->upd_done);
   if (ctx->d_err) cudaFree(ctx->d_err);
   delete ctx;
   return QLR_OK;
@@ -777,7 +794,12 @@ int qlr_qcomplete_update(qlr_ctx* ctx, const qlr_qmat* M, const uint8_t* mask, i
   qlr::CompleteArgs a;
   QLR_TRY(complete_args(M, mask, mask_ld, U, S, V, k, C, a));
   DeviceGuard g(ctx->device);
-  return masked_update(ctx, a, C->dtype);
+  if (C->dtype != QLR_F32 || !qlr::masked_update_tc_wanted(a.m, a.n, a.k) ||
+      !update_scratch(ctx, qlr::masked_update_tc_ws(a.m, a.n, a.k)))
+    return qlr::complete_update(ctx, a, C->dtype);
+  const int rc = masked_update(ctx, a, C->dtype, ctx->upd, ctx->upd_bytes);
+  QLR_CUDA_TRY(cudaEventRecord(ctx->upd_done, ctx->stream));
+  return rc;
 }
 
 int qlr_qcomplete(qlr_ctx* ctx, const qlr_qmat* M, const uint8_t* mask, int64_t mask_ld, int k, int p, int passes,
@@ -792,7 +814,7 @@ int qlr_qcomplete(qlr_ctx* ctx, const qlr_qmat* M, const uint8_t* mask, int64_t 
   QLR_TRY(qlr::complete_update(ctx, start, C->dtype));                        // C = P_Omega(M)
   for (int it = 0; it < iters; ++it) {
     QLR_TRY(lowrank_impl(ctx, C, k, p, passes, algo, omega, opts, U, S, V));   // eq. Step1
-    QLR_TRY(masked_update(ctx, update, C->dtype));                     // eq. Step2
+    QLR_TRY(masked_update(ctx, update, C->dtype, ctx->ws, ctx->ws_bytes));     // eq. Step2
   }
   return QLR_OK;
 }

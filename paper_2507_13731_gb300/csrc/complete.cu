@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(CM_THREADS) masked_copy_kernel(const CompleteA
 
 int complete_update(qlr_ctx* ctx, const CompleteArgs& a, int dtype) {
   if (a.m == 0 || a.n == 0) return QLR_OK;
-  if ((a.m + 31) / 32 > 65535) return QLR_EUNSUPPORTED;
+  if (a.m > COMPLETE_MAX_ROWS) return QLR_EUNSUPPORTED;
   const int tm = dtype == QLR_F64 ? 8 : 32, tn = dtype == QLR_F64 ? 32 : 64;
   const int64_t gy = (a.m + tm - 1) / tm, gx = (a.n + tn - 1) / tn;
   if (gx * gy > 0x7fffffff) return QLR_EUNSUPPORTED;

@@ -16,6 +16,11 @@ struct qlr_ctx {
   int* d_err = nullptr;          // device error word: first QLR_E* code recorded by a kernel
   void* ws = nullptr;            // workspace
   size_t ws_bytes = 0;
+  // Operand splits of qlr_qcomplete_update, which shares no memory with the other calls; `upd_done` is
+  // recorded behind the last use.
+  void* upd = nullptr;
+  size_t upd_bytes = 0;
+  cudaEvent_t upd_done = nullptr;
   int num_sms = 0;
   // launch statistics
   int64_t launches[QLR_KID_COUNT] = {};
@@ -56,9 +61,6 @@ struct WsArena {
 };
 
 int qlr_ensure_ws(qlr_ctx* ctx, size_t bytes);
-// The same for a workspace that the call can do without: false, with the present workspace kept,
-// when it cannot grow (stream capture, no memory).
-bool qlr_try_ws(qlr_ctx* ctx, size_t bytes);
 
 // Failing CUDA calls are reported on stderr when QLR_DEBUG_CUDA is set in the environment.
 void qlr_report_cuda(cudaError_t e, const char* expr, const char* file, int line);
@@ -245,6 +247,7 @@ struct CompleteArgs {
   int64_t m, n;
   int k;
 };
+constexpr int64_t COMPLETE_MAX_ROWS = (int64_t)65535 * 32;
 int complete_update(qlr_ctx* ctx, const CompleteArgs& a, int dtype);
 // Failure-detection self test (selftest.cu): a bounded mbarrier wait that times out.
 int selftest_wait_timeout(qlr_ctx* ctx);

@@ -551,9 +551,10 @@ int tall_gemm(qlr_ctx* ctx, const qlr_qmat& T, const double* const S[4], int64_t
   return rc;
 }
 
-// 24.4 against 21.8 us at m n k = 1e7, 27.8 / 35.1 at 3e7, 62 / 238 at 4096 x 4096, k = 8.
+// 24.4 against 21.8 us at m n k = 1e7, 27.8 / 35.1 at 3e7, 62 / 238 at 4096 x 4096, k = 8.  No more rows than
+// the other forms take, so that what is refused does not depend on the form.
 bool masked_update_tc_wanted(int64_t m, int64_t n, int k) {
-  return k >= 1 && k <= TALL_MAX_L && m < (1LL << 31) && n < (1LL << 31) && m * n * k >= (int64_t)15000000 &&
+  return k >= 1 && k <= TALL_MAX_L && m <= COMPLETE_MAX_ROWS && n < (1LL << 31) && m * n * k >= (int64_t)15000000 &&
          get_encode() != nullptr;
 }
 size_t masked_update_tc_ws(int64_t m, int64_t n, int k) {
