@@ -1179,7 +1179,7 @@ static int block_jacobi_cluster(int device, int l) {
   const size_t smem = block_jacobi_smem(l, bw, JP_MAX, sizeof(T), JB_THREADS);
   if (bw <= JB_THREADS / 32 &&
       cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
+      qlr_allow_smem(kern) == QLR_OK) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(JP_MAX, 1, 1);
     cfg.blockDim = dim3(JB_THREADS, 1, 1);
@@ -1227,7 +1227,7 @@ static int core_tsvd_t(qlr_ctx* ctx, int l, const double* R, int k, double* L, d
     const int threads = wide ? JB_THREADS_WIDE : JB_THREADS;
     const size_t smem = block_jacobi_smem(l, bw, jp, sizeof(T), threads);
     const int replay = (l + threads / 32 - 1) / (threads / 32);   // CTAs with rows of V
-    QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QLR_TRY(qlr_allow_smem(kern));
     cudaLaunchConfig_t cfg = {};
     if (jp > JP) QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cfg.gridDim = dim3(jp * (1 + (replay + jp - 1) / jp), 1, 1);
@@ -1253,7 +1253,7 @@ static int core_tsvd_t(qlr_ctx* ctx, int l, const double* R, int k, double* L, d
     const size_t smem = (size_t)4 * sizeof(T) * l * std::max(l, nwarps);
     auto kern = l <= 16 ? jacobi_small_kernel<T, 1> : l <= 32 ? jacobi_small_kernel<T, 2>
                 : l <= 48 ? jacobi_small_kernel<T, 3> : jacobi_small_kernel<T, 4>;
-    QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QLR_TRY(qlr_allow_smem(kern));
     KTimer kt(ctx, QLR_KID_JACOBI);
     QLR_CUDA_TRY(cudaMemsetAsync(pg, 0, sizeof(Progress), ctx->stream));
     kern<<<1 + (l + nwarps - 1) / nwarps, threads, smem, ctx->stream>>>(R, l, W, V, JMAX_SWEEPS, tol, sig, sweeps, rlog, pg,
@@ -1264,8 +1264,7 @@ static int core_tsvd_t(qlr_ctx* ctx, int l, const double* R, int k, double* L, d
     const size_t one = ll4 * sizeof(T);
     const bool w_smem = one <= 220 * 1024;
     const size_t smem = w_smem ? one : 0;
-    if (smem > 0)
-      QLR_CUDA_TRY(cudaFuncSetAttribute(jacobi_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 0) QLR_TRY(qlr_allow_smem(jacobi_kernel<T>));
     {
       KTimer kt(ctx, QLR_KID_JACOBI);
       jacobi_kernel<T><<<1, JT, smem, ctx->stream>>>(R, l, W, w_smem, JMAX_SWEEPS, tol, sig, sweeps, rlog, ctx->d_err);
@@ -1276,7 +1275,7 @@ static int core_tsvd_t(qlr_ctx* ctx, int l, const double* R, int k, double* L, d
       KTimer kt(ctx, QLR_KID_JACOBI);
       const size_t rs = (size_t)4 * 4 * l * sizeof(T);
       // static shared memory comes on top of the dynamic size: always opt in
-      QLR_CUDA_TRY(cudaFuncSetAttribute(jacobi_replay_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs));
+      QLR_TRY(qlr_allow_smem(jacobi_replay_kernel<T>));
       jacobi_replay_kernel<T><<<(l + 3) / 4, 128, rs, ctx->stream>>>(l, rlog, sweeps, V);
       qlr_count_launch();
     }
@@ -1292,7 +1291,7 @@ static int core_tsvd_t(qlr_ctx* ctx, int l, const double* R, int k, double* L, d
   QLR_CUDA_TRY(cudaGetLastError());
   const size_t rsm = (size_t)8 * l * sizeof(double);
   // static shared memory comes on top of the dynamic size: always opt in
-  QLR_CUDA_TRY(cudaFuncSetAttribute(refine_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
+  QLR_TRY(qlr_allow_smem(refine_kernel<T>));
   {   // R's left vectors are the replayed rotations V, its right vectors W's columns (W = R^H)
     KTimer kt(ctx, QLR_KID_REFINE);
     refine_kernel<T><<<k, 256, rsm, ctx->stream>>>(R, l, V, W, order, k, L, S, Rt);
@@ -1308,7 +1307,7 @@ int jacobi_grouped(qlr_ctx* ctx, const JacobiGroupArgs* d_args, int count, int l
   if (count <= 0) return QLR_OK;
   if (lmax > kBatchMaxL) return QLR_EUNSUPPORTED;
   const size_t smem = jacobi_grouped_smem(lmax);
-  QLR_CUDA_TRY(cudaFuncSetAttribute(jacobi_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  QLR_TRY(qlr_allow_smem(jacobi_grouped_kernel));
   KTimer kt(ctx, QLR_KID_JACOBI);
   jacobi_grouped_kernel<<<count, JG_THREADS, smem, ctx->stream>>>(d_args, JMAX_SWEEPS, ctx->d_err);
   qlr_count_launch();

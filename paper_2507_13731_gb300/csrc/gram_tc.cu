@@ -591,7 +591,7 @@ int gram_tc(qlr_ctx* ctx, const qlr_qmat& Y, double* G, WsArena& ws) {
       static_cast<const float*>(Y.plane[3]), m, l, Y.ld, d.L4p, d.mp, S, ex);
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
-  QLR_CUDA_TRY(cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem(7)));
+  QLR_TRY(qlr_allow_smem(gram_tc_kernel));
   const int nitems = d.ntiles * d.nchunks, sms = ctx->num_sms > 0 ? ctx->num_sms : 148;
   gram_tc_kernel<<<(unsigned)std::min(nitems, sms), GTHREADS, gsmem(7), ctx->stream>>>(prm, d.ntiles, nitems);
   qlr_count_launch();
@@ -643,7 +643,7 @@ int gram_tc_grouped(qlr_ctx* ctx, const void* d_probs, const int4* slice, int n_
   gram_slice_grouped_kernel<<<n_slice, 256, 0, ctx->stream>>>(probs, slice);
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
-  QLR_CUDA_TRY(cudaFuncSetAttribute(gram_tc_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem(8)));
+  QLR_TRY(qlr_allow_smem(gram_tc_grouped_kernel));
   gram_tc_grouped_kernel<<<std::min(n_mma, ctx->num_sms > 0 ? ctx->num_sms : 148), GTHREADS, gsmem(8), ctx->stream>>>(
       probs, mma, n_mma, ctx->d_err);
   qlr_count_launch();

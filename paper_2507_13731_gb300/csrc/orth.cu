@@ -1856,7 +1856,7 @@ int chol_f32_grouped(qlr_ctx* ctx, const CholGroupArgs* d_args, int count, int l
   if (count <= 0) return QLR_OK;
   if (lmax > kBatchMaxL) return QLR_EUNSUPPORTED;
   const size_t smem = chol_f32_grouped_smem(lmax);
-  QLR_CUDA_TRY(cudaFuncSetAttribute(chol_f32_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  QLR_TRY(qlr_allow_smem(chol_f32_grouped_kernel));
   KTimer kt(ctx, QLR_KID_CHOL);
   chol_f32_grouped_kernel<<<count, CF_THREADS, smem, ctx->stream>>>(d_args, ctx->d_err);
   qlr_count_launch();
@@ -1868,7 +1868,7 @@ int chol_df_grouped(qlr_ctx* ctx, const CholGroupArgs* d_args, int count, int lm
   if (count <= 0) return QLR_OK;
   if (lmax > kBatchMaxL) return QLR_EUNSUPPORTED;
   const size_t smem = chol_df_grouped_smem(lmax);
-  QLR_CUDA_TRY(cudaFuncSetAttribute(chol_df_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  QLR_TRY(qlr_allow_smem(chol_df_grouped_kernel));
   KTimer kt(ctx, QLR_KID_CHOL);
   chol_df_grouped_kernel<<<count, CG_THREADS, smem, ctx->stream>>>(d_args, ctx->d_err);
   qlr_count_launch();
@@ -2068,17 +2068,17 @@ int tri_inv(qlr_ctx* ctx, int l, const double* R, double* Rinv, const double* Di
     split_d32_kernel<<<gs, 256, 0, ctx->stream>>>(R, Rh, Rl, nr, Dinv_all, Dh, Dl, nd, run_if);
     qlr_count_launch();
     // 8 l floats: the same bytes as the FP64 form's 4 l doubles
-    QLR_CUDA_TRY(cudaFuncSetAttribute(tri_inv_blocked_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QLR_TRY(qlr_allow_smem(tri_inv_blocked_df_kernel));
     tri_inv_blocked_df_kernel<<<l, 256, smem, ctx->stream>>>(Rh, Rl, Dh, Dl, Rinv, l, run_if);
     qlr_count_launch();
   } else if (Dinv_all) {
     // static shared memory comes on top of the dynamic size: always opt in
-    QLR_CUDA_TRY(cudaFuncSetAttribute(tri_inv_blocked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QLR_TRY(qlr_allow_smem(tri_inv_blocked_kernel));
     tri_inv_blocked_kernel<<<l, 256, smem, ctx->stream>>>(R, Dinv_all, Rinv, l, run_if);
     qlr_count_launch();
   } else {
     // static shared memory comes on top of the dynamic size: always opt in
-    QLR_CUDA_TRY(cudaFuncSetAttribute(tri_inv_col_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QLR_TRY(qlr_allow_smem(tri_inv_col_kernel));
     tri_inv_col_kernel<<<l, 256, smem, ctx->stream>>>(R, Rinv, l);
     qlr_count_launch();
   }

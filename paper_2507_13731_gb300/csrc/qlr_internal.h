@@ -73,6 +73,13 @@ void qlr_report_cuda(cudaError_t e, const char* expr, const char* file, int line
     }                                                             \
   } while (0)
 
+// Lets a kernel be launched with any amount of dynamic shared memory that a block can have beside the
+// kernel's static one, on the current device.  The attribute belongs to the kernel, not to the caller: were it
+// set to each launch's own size, another thread's context could lower it between this call and the launch.
+int qlr_allow_smem_kernel(const void* kern);
+template <class F>
+int qlr_allow_smem(F* kern) { return qlr_allow_smem_kernel(reinterpret_cast<const void*>(kern)); }
+
 #define QLR_TRY(expr)                               \
   do {                                              \
     int r_ = (expr);                                \

@@ -1233,12 +1233,12 @@ int launch_kernel(qlr_ctx* ctx, const Plan& pl, const TcParams& prm, int kid) {
     if (pl.wide) return launch_kernel<KIND, AMODE, true>(ctx, pl, prm, kid);
   }
   auto kern = sketch_tc_kernel<KIND, AMODE, WIDE>;
-  QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
+  QLR_TRY(qlr_allow_smem(kern));
   KTimer kt(ctx, kid);
   const int threads = (KIND == K_TF32X3 || AMODE == A_T || prm.rn) ? TC_THREADS_WIDE : TC_THREADS;
   if (pl.grid_sk > 0) {
     auto sk = sketch_tc_streamk_kernel<KIND, AMODE, WIDE>;
-    QLR_CUDA_TRY(cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
+    QLR_TRY(qlr_allow_smem(sk));
     sk<<<pl.grid_sk, threads, pl.smem, ctx->stream>>>(prm);
     qlr_count_launch();
     QLR_CUDA_TRY(cudaGetLastError());
@@ -1533,7 +1533,7 @@ int launch_grouped(qlr_ctx* ctx, const GroupedSketch& gs) {
     auto pk = sketch_tc_persistent_kernel<KIND, AMODE, false>;
     if constexpr (AMODE == A_K && KIND != K_TF32X3)
       if (gs.wide) pk = sketch_tc_persistent_kernel<KIND, AMODE, true>;
-    QLR_CUDA_TRY(cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs.smem));
+    QLR_TRY(qlr_allow_smem(pk));
     KTimer kt(ctx, QLR_KID_SKETCH_TC);
     pk<<<(unsigned)gs.grid, TC_THREADS, gs.smem, ctx->stream>>>(static_cast<const TcParams*>(gs.d_probs), gs.d_items,
                                                                gs.nitems, gs.nb_max, gs.stages, gs.apl, gs.fd, gs.tmem_cols,
@@ -1543,7 +1543,7 @@ int launch_grouped(qlr_ctx* ctx, const GroupedSketch& gs) {
     return QLR_OK;
   }
   auto kern = sketch_tc_grouped_kernel<KIND, AMODE>;
-  QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs.smem));
+  QLR_TRY(qlr_allow_smem(kern));
   KTimer kt(ctx, QLR_KID_SKETCH_TC);
   kern<<<(unsigned)gs.nitems, TC_THREADS, gs.smem, ctx->stream>>>(static_cast<const TcParams*>(gs.d_probs), gs.d_items);
   qlr_count_launch();

@@ -477,7 +477,7 @@ int run_gemm(qlr_ctx* ctx, TallArgs& p, const __nv_bfloat16* A, const __nv_bfloa
     return QLR_ECUDA;
   const size_t smem = ares + p.stages * stage + 1024 + 256;
   auto kern = tall_gemm_kernel<MASKED>;
-  QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  QLR_TRY(qlr_allow_smem(kern));
   const int64_t tiles = (int64_t)p.mtiles * p.ntiles;
   const unsigned grid = (unsigned)std::min<int64_t>(tiles, ctx->num_sms > 0 ? ctx->num_sms : 148);
   kern<<<grid, TL_THREADS, smem, ctx->stream>>>(p);

@@ -1,12 +1,33 @@
 // Elementwise helpers on quaternion matrices: dtype conversion / copy, zero fill.
 #include <cstdio>
 #include <cstdlib>
+#include <mutex>
 
 #include "qlr_internal.h"
 
 void qlr_report_cuda(cudaError_t e, const char* expr, const char* file, int line) {
   static const bool on = std::getenv("QLR_DEBUG_CUDA") != nullptr;
   if (on) std::fprintf(stderr, "qlr: %s failed at %s:%d: %s\n", expr, file, line, cudaGetErrorString(e));
+}
+
+int qlr_allow_smem_kernel(const void* kern) {
+  static std::mutex mu;
+  static std::vector<std::pair<const void*, int>> limits;   // one entry per kernel of this library
+  int limit = 0;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    for (const auto& e : limits)
+      if (e.first == kern) limit = e.second;
+    if (limit == 0) {
+      cudaFuncAttributes fa;
+      QLR_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
+      limit = 227 * 1024 - (int)fa.sharedSizeBytes;
+      limits.emplace_back(kern, limit);
+    }
+  }
+  // on every call (the same value): a device, or its context after a reset, may not have seen it
+  QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+  return QLR_OK;
 }
 
 size_t qlr_dtype_size(int dtype) {
