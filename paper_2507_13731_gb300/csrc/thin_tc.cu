@@ -5,8 +5,11 @@
 //
 // Arithmetic.  An FP32 value is the sum of three BF16 values, x = x0 + x1 + x2 (each the rounding
 // to nearest of what the earlier ones leave: 8 bits each, 24 in all), so a product of two FP32
-// values is the sum of the six products x_i y_j with i + j <= 2 up to ~2^-26 relative, with FP32's
-// full exponent range.  The tensor cores' FP32 accumulation truncates (each MMA that adds into an
+// values is the sum of the six products x_i y_j with i + j <= 2 up to ~2^-26 relative.  From
+// TINY = 2^-100 on all three are normal BF16 numbers.  A tile whose operands hold smaller entries that
+// count, or entries that are not finite (a split's 0 times an infinity is a NaN that FP32 does not
+// give), or whose sums may come near FP32's largest number (x0 may lie 2^-9 above x), is formed by FP32
+// multiply-adds in the epilogue instead: the split kernels note what they see.  The tensor cores' FP32 accumulation truncates (each MMA that adds into an
 // accumulator loses half an ulp of it on average, always toward zero), so the reduction is cut into
 // chunks of 32 elements (16 where it is at most 64 long), each in a fresh accumulator: the
 // corrections first, 2^-8 of the sum or less, then the one or two MMAs of x0 y0.  The epilogue
@@ -70,8 +73,35 @@ struct TallArgs {
   int64_t ldm;
   const uint8_t* mask;
   int64_t ldk;
+  // the operands as given, for tiles formed in FP32, and what the split kernels found in them
+  const float* t[4];            // tall operand, column-major
+  int64_t ldt;
+  const double* s[4];           // small FP64 factor, column-major; masked update: U and S
+  int64_t lds;
+  const float* u[4];
+  int64_t ldu;
+  const double* sigma;
+  const uint8_t* aflags;        // [512-row block][column of the tall operand]: largest biased exponent, 255 also
+                                // for entries below TINY
+  const uint4* bflags;          // [column tile][32-column block of the reduction]: columns with entries below
+                                // TINY, columns with entries that dwarf such, largest biased exponent
   int* err;
 };
+constexpr float TINY = 7.888609e-31f, DWARF = 1.3234890e-23f;   // 2^-100, 2^-76
+// Operands below 2^(ea - 126) and 2^(eb - 126): a sum of 4 l <= 2^10 products stays below 2^126.
+constexpr unsigned EXP_SUM_MAX = 126 + 252 - 10;
+constexpr int TL_MAX_RB = TALL_MAX_L / 32;                      // 32-column blocks of the reduction
+constexpr int SPLIT_ROWS = 512;                                 // rows per CTA of the split kernel
+__device__ __forceinline__ bool is_tiny(float x) { return x != 0.f && fabsf(x) < TINY; }
+
+// Signs of the real product, bit 4 c + d: T_c X_{c xor d} enters output plane d negatively.
+constexpr uint32_t neg_bits(std::initializer_list<std::pair<int, int>> cd) {
+  uint32_t m = 0;
+  for (const auto& e : cd) m |= 1u << (4 * e.first + e.second);
+  return m;
+}
+constexpr uint32_t NEG_THIN = neg_bits({{1, 0}, {2, 0}, {3, 0}, {3, 1}, {1, 2}, {2, 3}});   // T S, eq. 1
+constexpr uint32_t NEG_MASKED = neg_bits({{1, 1}, {3, 1}, {1, 2}, {2, 2}, {2, 3}, {3, 3}});  // u conj(v), T = V, X = U S
 
 // x = s0 + s1 + s2.  A value that rounds beyond BF16's range is truncated instead; a non-finite
 // value is kept whole in s0.
@@ -84,29 +114,54 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16 (&s)[3]) {
 }
 
 // Tall operand T (rows x l, column-major planes): out[s][4 r + c][row], rows padded to Kq with
-// zero reduction rows.  Two matrix rows per thread.
+// zero reduction rows.  A thread takes two matrix rows of one column's four planes.
 struct SplitArgs {
   const float* t[4];
   int64_t ld, rows, ldo;
   int l, Kq;
   __nv_bfloat16* out;
+  uint8_t* flags;
 };
-__global__ void __launch_bounds__(256) tall_split_kernel(const SplitArgs a) {
-  const int kk = blockIdx.y, r = kk / 4, c = kk % 4;
-  const int64_t i = 2 * ((int64_t)blockIdx.x * 256 + threadIdx.x);
-  if (i >= a.ldo) return;
-  float x0 = 0.f, x1 = 0.f;
+__global__ void __launch_bounds__(SPLIT_ROWS / 2) tall_split_kernel(const SplitArgs a) {
+  __shared__ unsigned wmax[SPLIT_ROWS / 64];
+  const int r = blockIdx.y;
+  const int64_t i = (int64_t)blockIdx.x * SPLIT_ROWS + 2 * threadIdx.x;
+  float x[4][2] = {};
   if (r < a.l) {
-    const float* src = (c == 0 ? a.t[0] : c == 1 ? a.t[1] : c == 2 ? a.t[2] : a.t[3]) + (int64_t)r * a.ld;
-    if (i < a.rows) x0 = src[i];
-    if (i + 1 < a.rows) x1 = src[i + 1];
-  }
-  __nv_bfloat16 s0[3], s1[3];
-  split3(x0, s0);
-  split3(x1, s1);
 #pragma unroll
-  for (int s = 0; s < 3; ++s)
-    *reinterpret_cast<__nv_bfloat162*>(a.out + ((size_t)s * a.Kq + kk) * a.ldo + i) = __nv_bfloat162(s0[s], s1[s]);
+    for (int c = 0; c < 4; ++c) {
+      const float* src = a.t[c] + (int64_t)r * a.ld;
+      if (i < a.rows) x[c][0] = src[i];
+      if (i + 1 < a.rows) x[c][1] = src[i + 1];
+    }
+  }
+  float mx = 0.f;
+  bool odd = false;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const float v = x[e / 2][e % 2];
+    mx = fmaxf(mx, fabsf(v));
+    odd = odd || is_tiny(v) || isnan(v);
+  }
+  const unsigned m = __reduce_max_sync(0xffffffffu, odd ? 0x7f800000u : __float_as_uint(mx));
+  if (threadIdx.x % 32 == 0) wmax[threadIdx.x / 32] = m;
+  if (i < a.ldo) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      __nv_bfloat16 s0[3], s1[3];
+      split3(x[c][0], s0);
+      split3(x[c][1], s1);
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+        *reinterpret_cast<__nv_bfloat162*>(a.out + ((size_t)s * a.Kq + 4 * r + c) * a.ldo + i) = __nv_bfloat162(s0[s], s1[s]);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned b = 0;
+    for (int w = 0; w < SPLIT_ROWS / 64; ++w) b = max(b, wmax[w]);
+    a.flags[(size_t)blockIdx.x * (a.Kq / 4) + r] = (uint8_t)(b >> 23);
+  }
 }
 
 // Expanded factor: out[s][128 nt + 64 h + 16 d + jj][4 r + c] = sign(c, d) X_{c xor d}(r, 32 nt + 16 h + jj):
@@ -123,11 +178,13 @@ struct ExpandArgs {
   int64_t N;                    // valid output columns
   int Kq;
   int64_t rows;                 // rows of one split
-  uint32_t neg;                 // bit 4 c + d: negative sign
+  uint32_t neg;                 // NEG_THIN or NEG_MASKED
   __nv_bfloat16* out;
+  uint4* flags;
 };
 __global__ void __launch_bounds__(256) tall_expand_kernel(const ExpandArgs a) {
   __shared__ float X[4][32][33];   // plane, r, column
+  __shared__ unsigned tiny_cols[8], big_cols[8], wmax[8];
   const int t = threadIdx.x;
   const int64_t j0 = (int64_t)blockIdx.x * TL_J;
   const int r0 = blockIdx.y * 32;
@@ -142,6 +199,26 @@ __global__ void __launch_bounds__(256) tall_expand_kernel(const ExpandArgs a) {
     X[q][rr][jj] = v;
   }
   __syncthreads();
+  {   // a lane per column, four r a warp
+    bool tiny = false, odd = false;
+    float mx = 0.f;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const float v = X[e / 4][4 * (t / 32) + e % 4][t % 32];
+      tiny = tiny || is_tiny(v);
+      odd = odd || isnan(v);
+      mx = fmaxf(mx, fabsf(v));
+    }
+    const unsigned tb = __ballot_sync(0xffffffffu, tiny), bb = __ballot_sync(0xffffffffu, mx >= DWARF);
+    const unsigned mb = __reduce_max_sync(0xffffffffu, odd ? 0x7f800000u : __float_as_uint(mx));
+    if (t % 32 == 0) { tiny_cols[t / 32] = tb; big_cols[t / 32] = bb; wmax[t / 32] = mb; }
+    __syncthreads();
+    if (t == 0) {
+      uint4 f = make_uint4(0u, 0u, 0u, 0u);
+      for (int w = 0; w < 8; ++w) { f.x |= tiny_cols[w]; f.y |= big_cols[w]; f.z = max(f.z, wmax[w] >> 23); }
+      a.flags[(size_t)blockIdx.x * TL_MAX_RB + blockIdx.y] = f;
+    }
+  }
   const int rr = t % 32;
   if (4 * (r0 + rr) >= a.Kq) return;
   for (int w = t / 32; w < TL_N; w += 8) {
@@ -339,10 +416,23 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
   } else {
     // ---------------- epilogue: 8 warps, a lane quarter and half the columns each ----------------
     const int q = warp & 3, half = warp >> 2;
-    int mt = (int)(t0 / p.ntiles), nt = (int)(t0 % p.ntiles), b = 0;
+    int mt = (int)(t0 / p.ntiles), nt = (int)(t0 % p.ntiles), b = 0, cur = -1;
     uint32_t bph = 0;
+    unsigned ea = 0;                                   // largest biased exponent of these rows
     bool ok = true;
     for (int left = (int)(t1 - t0); left > 0 && ok; --left) {
+      // what the split kernels found: loads in flight while the MMAs run
+      unsigned tiny_cols = 0, big_cols = 0, eb = 0, rows4 = 0;
+      if (32 * lane < p.Kq / 4) {
+        const uint4 f = p.bflags[(size_t)nt * TL_MAX_RB + lane];
+        tiny_cols = f.x; big_cols = f.y; eb = f.z;
+      }
+      const bool fresh = mt != cur;
+      if (fresh) {
+        const unsigned* af = reinterpret_cast<const unsigned*>(p.aflags + (size_t)(mt / (SPLIT_ROWS / TL_M)) * (p.Kq / 4));
+        for (int w = lane; w < p.Kq / 16; w += 32) rows4 = __vmaxu4(rows4, af[w]);
+      }
+      cur = mt;
       const int64_t row = (int64_t)mt * TL_M + q * 32 + lane, j0 = (int64_t)nt * TL_J + half * 16;
       const int nch = (ksteps_of(nt) + per - 1) / per;
       if (++nt == p.ntiles) { nt = 0; ++mt; }
@@ -376,7 +466,40 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
         if (++b == TL_ACC) { b = 0; bph ^= 1u; }
       }
       if (!ok) break;
+      if (fresh) {
+        const unsigned r4 = __vmaxu4(rows4, rows4 >> 16);
+        ea = __reduce_max_sync(0xffffffffu, __vmaxu4(r4, r4 >> 8) & 255u);
+      }
+      eb = __reduce_max_sync(0xffffffffu, eb);
+      const unsigned tc = __reduce_or_sync(0xffffffffu, tiny_cols) & ~__reduce_or_sync(0xffffffffu, big_cols);
+      const bool again = tc != 0 || ea == 255u || eb == 255u || ea + eb > EXP_SUM_MAX;
       if (!row_ok) continue;
+      if (again) {   // FP32 multiply-adds on the operands as given (the sums' values are not used)
+        constexpr uint32_t neg = MASKED ? NEG_MASKED : NEG_THIN;
+#pragma unroll
+        for (int e = 0; e < 64; ++e) v[e / 16][e % 16] = 0.f;
+        const int rend = p.upper ? (int)min((int64_t)p.K / 4, j0 + 16) : p.K / 4;
+#pragma unroll 1
+        for (int r = 0; r < rend; ++r) {
+          float t[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) t[c] = p.t[c][(int64_t)r * p.ldt + row];
+          const float sg = MASKED ? (float)p.sigma[r] : 0.f;
+#pragma unroll
+          for (int jj = 0; jj < 16; ++jj) {
+            if (jj >= nj) continue;
+            float x[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              x[c] = MASKED ? p.u[c][(int64_t)r * p.ldu + j0 + jj] * sg : (float)p.s[c][(j0 + jj) * p.lds + r];
+#pragma unroll
+            for (int d = 0; d < 4; ++d)
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                v[d][jj] = fmaf(((neg >> (4 * c + d)) & 1u) ? -t[c] : t[c], x[c ^ d], v[d][jj]);
+          }
+        }
+      }
       // pointers are stepped by the pitch: 64-bit index products for every entry made this
       // epilogue the bound (50 instructions an entry: 211 us at 4096 x 4096, k = 30)
       if (MASKED) {   // C(i, j): i = output column, j = row of the tall operand
@@ -445,21 +568,31 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
 }
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
-size_t a_bytes(int64_t rows, int64_t l) { return (size_t)3 * round_up(4 * l, TL_BK) * round_up(rows, 8) * 2; }
-size_t b_bytes(int64_t N, int64_t l) { return (size_t)3 * round_up(N, TL_J) * 4 * round_up(4 * l, TL_BK) * 2; }
+// The operands' splits, and with what was found in them behind (multiples of 16 bytes).
+size_t a_split(int64_t rows, int64_t l) { return (size_t)3 * round_up(4 * l, TL_BK) * round_up(rows, 8) * 2; }
+size_t b_split(int64_t N, int64_t l) { return (size_t)3 * round_up(N, TL_J) * 4 * round_up(4 * l, TL_BK) * 2; }
+size_t a_bytes(int64_t rows, int64_t l) {
+  return a_split(rows, l) + (size_t)(round_up(rows, SPLIT_ROWS) / SPLIT_ROWS) * (round_up(4 * l, TL_BK) / 4);
+}
+size_t b_bytes(int64_t N, int64_t l) { return b_split(N, l) + (size_t)(round_up(N, TL_J) / TL_J) * TL_MAX_RB * sizeof(uint4); }
 
 // Split the tall operand (rows [0, rows) of its planes) into `out`.
-void run_split(cudaStream_t st, const void* const t[4], int64_t ld, int64_t rows, int l, __nv_bfloat16* out) {
+void run_split(cudaStream_t st, const void* const t[4], int64_t ld, int64_t rows, int l, char* out, TallArgs& p) {
   SplitArgs a{};
   for (int c = 0; c < 4; ++c) a.t[c] = static_cast<const float*>(t[c]);
-  a.ld = ld; a.rows = rows; a.ldo = round_up(rows, 8); a.l = l; a.Kq = (int)round_up(4 * l, TL_BK); a.out = out;
-  tall_split_kernel<<<dim3((unsigned)((a.ldo / 2 + 255) / 256), (unsigned)a.Kq), 256, 0, st>>>(a);
+  a.ld = ld; a.rows = rows; a.ldo = round_up(rows, 8); a.l = l; a.Kq = (int)round_up(4 * l, TL_BK);
+  a.out = reinterpret_cast<__nv_bfloat16*>(out);
+  a.flags = reinterpret_cast<uint8_t*>(out + a_split(rows, l));
+  for (int c = 0; c < 4; ++c) p.t[c] = a.t[c];
+  p.ldt = ld;
+  p.aflags = a.flags;
+  tall_split_kernel<<<dim3((unsigned)((rows + SPLIT_ROWS - 1) / SPLIT_ROWS), (unsigned)(a.Kq / 4)), SPLIT_ROWS / 2, 0, st>>>(a);
   qlr_count_launch();
 }
 
 // Fill in the tile plan and the tensor maps and launch.
 template <bool MASKED>
-int run_gemm(qlr_ctx* ctx, TallArgs& p, const __nv_bfloat16* A, const __nv_bfloat16* B, int l) {
+int run_gemm(qlr_ctx* ctx, TallArgs& p, const char* A, const char* B, int l) {
   p.K = 4 * l;
   p.Kq = (int)round_up(p.K, TL_BK);
   p.mtiles = (int)((p.M + TL_M - 1) / TL_M);
@@ -486,22 +619,19 @@ int run_gemm(qlr_ctx* ctx, TallArgs& p, const __nv_bfloat16* A, const __nv_bfloa
   return QLR_OK;
 }
 
-int run_expand(cudaStream_t st, ExpandArgs& e, int l, int64_t N, __nv_bfloat16* out) {
+int run_expand(cudaStream_t st, ExpandArgs& e, int l, int64_t N, char* out, TallArgs& p) {
   e.l = l;
   e.N = N;
   e.Kq = (int)round_up(4 * l, TL_BK);
   e.rows = round_up(N, TL_J) * 4;
-  e.out = out;
+  e.out = reinterpret_cast<__nv_bfloat16*>(out);
+  e.flags = reinterpret_cast<uint4*>(out + b_split(N, l));
+  for (int c = 0; c < 4; ++c) { p.s[c] = e.s[c]; p.u[c] = e.u[c]; }
+  p.lds = e.lds; p.ldu = e.ldu; p.sigma = e.sigma; p.bflags = e.flags;
   tall_expand_kernel<<<dim3((unsigned)((N + TL_J - 1) / TL_J), (unsigned)((e.Kq + 127) / 128)), 256, 0, st>>>(e);
   qlr_count_launch();
   QLR_CUDA_TRY(cudaGetLastError());
   return QLR_OK;
-}
-
-uint32_t bits(std::initializer_list<std::pair<int, int>> cd) {
-  uint32_t m = 0;
-  for (const auto& e : cd) m |= 1u << (4 * e.first + e.second);
-  return m;
 }
 
 // Panels of the masked update: the expanded factor of a panel of rows of C stays in L2 while the
@@ -529,19 +659,19 @@ int tall_gemm(qlr_ctx* ctx, const qlr_qmat& T, const double* const S[4], int64_t
               bool upper, qlr_qmat& C, WsArena& ws) {
   const int l = (int)T.cols;
   const size_t mark = ws.off;
-  auto* A = ws.take<__nv_bfloat16>(a_bytes(T.rows, l) / 2);
-  auto* B = ws.take<__nv_bfloat16>(b_bytes(N, l) / 2);
+  char* A = ws.take<char>(a_bytes(T.rows, l));
+  char* B = ws.take<char>(b_bytes(N, l));
   if (!ws.ok) { ws.ok = true; ws.off = mark; return QLR_ENOMEM; }
   KTimer kt(ctx, QLR_KID_APPLY);
-  run_split(ctx->stream, T.plane, T.ld, T.rows, l, A);
+  TallArgs p;
+  memset(&p, 0, sizeof(p));
+  run_split(ctx->stream, T.plane, T.ld, T.rows, l, A, p);
   ExpandArgs e{};
   for (int c = 0; c < 4; ++c) e.s[c] = S[c];
   e.lds = lds;
-  e.neg = bits({{1, 0}, {2, 0}, {3, 0}, {3, 1}, {1, 2}, {2, 3}});      // T_c S_{c xor d}, eq. 1
-  int rc = run_expand(ctx->stream, e, l, N, B);
+  e.neg = NEG_THIN;
+  int rc = run_expand(ctx->stream, e, l, N, B, p);
   if (rc == QLR_OK) {
-    TallArgs p;
-    memset(&p, 0, sizeof(p));
     p.M = T.rows; p.N = N; p.upper = upper ? 1 : 0;
     for (int c = 0; c < 4; ++c) p.c[c] = static_cast<float*>(C.plane[c]);
     p.ldc = C.ld; p.alpha = alpha; p.beta = beta; p.err = ctx->d_err;
@@ -564,8 +694,8 @@ size_t masked_update_tc_ws(int64_t m, int64_t n, int k) {
 int masked_update_tc(qlr_ctx* ctx, const CompleteArgs& a, WsArena& ws) {
   const size_t mark = ws.off;
   const int64_t pr = panel_rows(a.m, a.k), pc = std::min<int64_t>(a.n, PANEL_COLS);
-  auto* A = ws.take<__nv_bfloat16>(a_bytes(pc, a.k) / 2);
-  auto* B = ws.take<__nv_bfloat16>(b_bytes(pr, a.k) / 2);
+  char* A = ws.take<char>(a_bytes(pc, a.k));
+  char* B = ws.take<char>(b_bytes(pr, a.k));
   if (!ws.ok) { ws.ok = true; ws.off = mark; return QLR_ENOMEM; }
   KTimer kt(ctx, QLR_KID_COMPLETE);
   int rc = QLR_OK;
@@ -573,18 +703,18 @@ int masked_update_tc(qlr_ctx* ctx, const CompleteArgs& a, WsArena& ws) {
     const int64_t nc = std::min(pc, a.n - j0);
     const void* v[4];
     for (int c = 0; c < 4; ++c) v[c] = static_cast<const float*>(a.V[c]) + j0;
-    run_split(ctx->stream, v, a.ldv, nc, a.k, A);
+    TallArgs tall;
+    memset(&tall, 0, sizeof(tall));
+    run_split(ctx->stream, v, a.ldv, nc, a.k, A, tall);
     for (int64_t i0 = 0; i0 < a.m && rc == QLR_OK; i0 += pr) {
       const int64_t nr = std::min(pr, a.m - i0);
       ExpandArgs e{};
       for (int c = 0; c < 4; ++c) e.u[c] = static_cast<const float*>(a.U[c]) + i0;
       e.ldu = a.ldu; e.sigma = a.S;
-      // u conj(v): V_c U_{c xor d} with the conjugate's signs
-      e.neg = bits({{1, 1}, {3, 1}, {1, 2}, {2, 2}, {2, 3}, {3, 3}});
-      rc = run_expand(ctx->stream, e, a.k, nr, B);
+      e.neg = NEG_MASKED;
+      TallArgs p = tall;
+      rc = run_expand(ctx->stream, e, a.k, nr, B, p);
       if (rc != QLR_OK) break;
-      TallArgs p;
-      memset(&p, 0, sizeof(p));
       p.M = nc; p.N = nr;
       for (int c = 0; c < 4; ++c) {
         p.c[c] = static_cast<float*>(a.C[c]) + i0 * a.ldc + j0;
