@@ -702,14 +702,6 @@ __device__ __forceinline__ d32 d32_rsqrt3(d32 d) {
   const float t = __fmul_rn(y, c), te = __fmaf_rn(y, c, -t);          // y c exactly
   return d32_add({y, 0.f}, {t, __fmaf_rn(y, cl, te)});
 }
-__device__ __forceinline__ d32 d32_rcp(d32 d) {
-  d32 y = {__frcp_rn(d.h), 0.f};
-  for (int it = 0; it < 2; ++it) {   // y <- y + y (1 - d y)
-    const d32 r = d32_add({1.f, 0.f}, d32_neg(d32_mul(d, y)));
-    y = d32_add(y, d32_mul(y, r));
-  }
-  return y;
-}
 // A quaternion of double-FP32 numbers: components (real, i, j, k) of the high and low parts.
 struct dq {
   float4 h, l;
@@ -748,6 +740,61 @@ __device__ __forceinline__ void cc_st_async2f(uint32_t raddr, float a, float b, 
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(raddr), "f"(a),
                "f"(b), "r"(rbar)
                : "memory");
+}
+
+// One doubling of the inverse X of an upper-triangular CB x CB quaternion block D (planes): from the
+// inverses of its S x S diagonal blocks to those of the 2 S x 2 S ones, X_IJ = -X_II (D_IJ X_JJ).  Four
+// lanes an entry where sums are long.  Eight short products, each dense over the warps, instead of CB
+// dependent substitution steps: the FP64 pipe (under two multiply-adds per SM and cycle) and a dependent FP64
+// operation's latency are the bound.
+template <int S>
+__device__ __forceinline__ void cc_inverse_doubling(const double (&D)[4][CB][CB + 1], double (&X)[4][CB][CB + 1],
+                                                    double (&T)[4][CB / 2 * CB / 2]) {
+  constexpr int PARTS = S >= 4 ? 4 : 1, ENT = CB / 2 * S;   // entries of all blocks X_IJ
+  const int t = threadIdx.x, part = t % PARTS, e = t / PARTS;
+  const int i = e % S, j = (e / S) % S, I0 = e / (S * S) * 2 * S, J0 = I0 + S;   // within the block, its corners
+  const bool on = e < ENT;
+  auto madd = [](Quat<double>& acc, const Quat<double>& a, const Quat<double>& b) {
+    acc.w = fma(-a.z, b.z, fma(-a.y, b.y, fma(-a.x, b.x, fma(a.w, b.w, acc.w))));
+    acc.x = fma(-a.z, b.y, fma(a.y, b.z, fma(a.x, b.w, fma(a.w, b.x, acc.x))));
+    acc.y = fma(a.z, b.x, fma(a.y, b.w, fma(-a.x, b.z, fma(a.w, b.y, acc.y))));
+    acc.z = fma(a.z, b.w, fma(-a.y, b.x, fma(a.x, b.y, fma(a.w, b.z, acc.z))));
+  };
+  auto total = [&](Quat<double>& q) {
+#pragma unroll
+    for (int o = PARTS / 2; o > 0; o >>= 1) {
+      q.w += __shfl_xor_sync(0xffffffffu, q.w, o);
+      q.x += __shfl_xor_sync(0xffffffffu, q.x, o);
+      q.y += __shfl_xor_sync(0xffffffffu, q.y, o);
+      q.z += __shfl_xor_sync(0xffffffffu, q.z, o);
+    }
+  };
+  const bool warp_on = (t / 32) * 32 / PARTS < ENT;   // whole warps
+  Quat<double> acc = {0, 0, 0, 0};
+  if (warp_on) {
+    if (on)
+      for (int k = part; k <= j; k += PARTS)
+        madd(acc, {D[0][I0 + i][J0 + k], D[1][I0 + i][J0 + k], D[2][I0 + i][J0 + k], D[3][I0 + i][J0 + k]},
+             {X[0][J0 + k][J0 + j], X[1][J0 + k][J0 + j], X[2][J0 + k][J0 + j], X[3][J0 + k][J0 + j]});
+    total(acc);
+    if (on && part == 0) { T[0][e] = acc.w; T[1][e] = acc.x; T[2][e] = acc.y; T[3][e] = acc.z; }
+  }
+  __syncthreads();
+  if (warp_on) {
+    acc = {0, 0, 0, 0};
+    if (on)
+      for (int k = i + part; k < S; k += PARTS) {
+        const int o = e - i + k;   // T(k, j) of the same block
+        madd(acc, {X[0][I0 + i][I0 + k], X[1][I0 + i][I0 + k], X[2][I0 + i][I0 + k], X[3][I0 + i][I0 + k]},
+             {T[0][o], T[1][o], T[2][o], T[3][o]});
+      }
+    total(acc);
+    if (on && part == 0) {
+      X[0][I0 + i][J0 + j] = -acc.w; X[1][I0 + i][J0 + j] = -acc.x;
+      X[2][I0 + i][J0 + j] = -acc.y; X[3][I0 + i][J0 + j] = -acc.z;
+    }
+  }
+  __syncthreads();
 }
 
 __global__ void __launch_bounds__(CC_THREADS, 1) chol_cluster_df_kernel(const double* __restrict__ G, double* __restrict__ R,
@@ -932,47 +979,30 @@ __global__ void __launch_bounds__(CC_THREADS, 1) chol_cluster_df_kernel(const do
   }
   __threadfence();
   cluster.sync();
-  // Inverses of the diagonal blocks, 16 lanes per column (eight warps: all 16 columns at once): lane r
-  // holds entry r of the column, x_i = acc_i / r_ii is broadcast and lanes r < i subtract R_ri x_i --
-  // no barrier and no FP64 (a block-wide FP64 substitution took 36 thousand cycles, 18 of 112 us at
-  // l = 60).
-  __shared__ dq D[CB][CB + 1];
+  // inverses of the diagonal blocks, in FP64
+  __shared__ double D[4][CB][CB + 1], X[4][CB][CB + 1], T[4][CB / 2 * CB / 2];
   const int nblk = (l + CB - 1) / CB;
   for (int J = c; J < nblk; J += nc) {
     const int j0 = J * CB, b = min(CB, l - j0);
     for (int e = t; e < CB * CB; e += CC_THREADS) {
       const int i = e % CB, jj = e / CB;
-      dq q;
-      for (int cp = 0; cp < 4; ++cp)
-        dq_set(q, cp, (i < b && jj < b && i <= jj) ? d32_from(__ldcg(R + cp * ll + (size_t)(j0 + jj) * l + j0 + i))
-                                                   : d32{0.f, 0.f});
-      D[i][jj] = q;
+      for (int cp = 0; cp < 4; ++cp) {
+        double v = (i < b && jj < b && i <= jj) ? __ldcg(R + cp * ll + (size_t)(j0 + jj) * l + j0 + i) : 0.0;
+        if (i >= b && i == jj && cp == 0) v = 1.0;
+        D[cp][i][jj] = v;
+        X[cp][i][jj] = (i == jj && cp == 0) ? 1.0 / v : 0.0;
+      }
     }
     __syncthreads();
-    const int r = lane & 15, jj = 2 * warp + (lane >> 4);
-    const d32 rp = (r < b) ? d32_rcp(dq_get(D[r][r], 0)) : d32{0.f, 0.f};
-    dq x;
-    x.h = make_float4(r == jj ? 1.f : 0.f, 0.f, 0.f, 0.f);
-    x.l = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = b - 1; i >= 0; --i) {
-      if (r == i && i <= jj)
-        for (int cp = 0; cp < 4; ++cp) dq_set(x, cp, d32_mul(dq_get(x, cp), rp));
-      dq xi;
-      for (int cp = 0; cp < 4; ++cp) {
-        const d32 v = dq_get(x, cp);
-        dq_set(xi, cp, {__shfl_sync(0xffffffffu, v.h, i, 16), __shfl_sync(0xffffffffu, v.l, i, 16)});
-      }
-      if (r < i && i <= jj) {
-        dq m = D[r][i];                       // x - m xi = x - conj(conj(m)) xi
-        m.h.y = -m.h.y; m.h.z = -m.h.z; m.h.w = -m.h.w;
-        m.l.y = -m.l.y; m.l.z = -m.l.z; m.l.w = -m.l.w;
-        x = dq_cfms(x, m, xi);
-      }
-    }
+    cc_inverse_doubling<1>(D, X, T);
+    cc_inverse_doubling<2>(D, X, T);
+    cc_inverse_doubling<4>(D, X, T);
+    cc_inverse_doubling<8>(D, X, T);
     double* Dinv = Dinv_all + (size_t)J * 4 * CB * CB;
-    if (r < b && jj < b)
-      for (int cp = 0; cp < 4; ++cp)
-        Dinv[(size_t)cp * b * b + (size_t)jj * b + r] = (r <= jj) ? d32_to(dq_get(x, cp)) : 0.0;
+    for (int e = t; e < b * b; e += CC_THREADS) {
+      const int i = e % b, jj = e / b;
+      for (int cp = 0; cp < 4; ++cp) Dinv[(size_t)cp * b * b + (size_t)jj * b + i] = X[cp][i][jj];
+    }
     __syncthreads();
   }
 }
