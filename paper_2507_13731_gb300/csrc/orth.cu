@@ -1180,8 +1180,8 @@ __global__ void __launch_bounds__(256) tri_inv_blocked_kernel(const double* __re
 // F = Phi(E - F^H F), Phi(X) = strict upper part of X plus half its (real) diagonal, a fixed point
 // reached by iterating from F = Phi(E) (the error shrinks like |E|^(n+1)).  The inverse is
 // (I + F)^{-1} = I + D with D = -F - F D (the Neumann series I - F + F^2 - ...), iterated from
-// D = -F.  Each step is a triangular product spread over all SMs -- no serial pivots.  Both
-// iterations contract with a rate of at most 4 l max|E|, and stop when the next step could change no
+// D = -F.  Each step is a triangular product spread over all SMs -- no serial pivots.  The iterations
+// contract with rates of at most 9 and 4.5 l max|E|, and stop when the next step could change no
 // entry by more than SERIES_TOL (far below the FP64 resolution of I + F).
 // One cooperative launch runs everything, a barrier over its CTAs between two steps: as 16 launches
 // (most of them finding their iteration converged) the series took 206 us at l = 180 and 49 us at
@@ -1198,15 +1198,16 @@ __global__ void __launch_bounds__(256) tri_inv_blocked_kernel(const double* __re
 // under the 2^-45-class error of the Gram itself), and the steps stop being FP64-bound.  FP64
 // sketches accumulate in FP64.
 constexpr double SERIES_MAX = 5e-3;
-constexpr double SERIES_TOL = 1e-18;
+constexpr double SERIES_TOL = 2e-18;
 constexpr int SERIES_ITERS = 6, NEUMANN_ITERS = 7;   // the first Neumann step is D = -F
 constexpr int SPLIT = 16;   // lanes per entry: sums as short per-lane chains plus a shuffle tree
 
 struct SeriesArgs {
   const double* G;
   // quaternion vectors of TA, l x l each: E, the sums F^H F and F D (their entry's owner only), F by
-  // columns (two, taking turns) and by rows, D by columns
-  void *e, *s1, *s2, *fc[2], *fr, *dc[2];
+  // columns (two, taking turns) and by rows, D by columns; for TA = float also what E and F leave when
+  // they are rounded to FP32 (owner only): F and D are each rounded once, from FP64-class values
+  void *e, *s1, *s2, *fc[2], *fr, *dc[2], *elo, *flo;
   double *R2, *R2inv;
   unsigned* mx;                  // FP32 bits: [0] max|E|, [1 ..] each step's largest change (zeroed)
   unsigned* arrived;             // the barrier's count (zeroed)
@@ -1214,6 +1215,17 @@ struct SeriesArgs {
   int* err;
   int l;
 };
+// (hi + lo) - x as a value of TA and the rest.
+__device__ __forceinline__ void series_diff(float hi, float lo, float x, float& v, float& rest) {
+  const float s = __fsub_rn(hi, x), b = __fsub_rn(s, hi);
+  const float e = __fadd_rn(__fsub_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fadd_rn(x, b)), lo);
+  v = __fadd_rn(s, e);
+  rest = __fsub_rn(e, __fsub_rn(v, s));
+}
+__device__ __forceinline__ void series_diff(double hi, double, double x, double& v, double& rest) {
+  v = hi - x;
+  rest = 0.0;
+}
 template <class TA> struct SeriesVec;
 template <> struct SeriesVec<float> { using V = float4; };
 template <> struct SeriesVec<double> { using V = double4; };
@@ -1263,6 +1275,9 @@ __global__ void __launch_bounds__(SERIES_THREADS) series_kernel(const SeriesArgs
   V* s1 = static_cast<V*>(a.s1);
   V* s2 = static_cast<V*>(a.s2);
   V* fr = static_cast<V*>(a.fr);
+  V* el = static_cast<V*>(a.elo);   // unused (null) for TA = double
+  V* fl = static_cast<V*>(a.flo);
+  constexpr bool LO = sizeof(TA) == 4;
   unsigned bar = 0;
   auto raise = [&](unsigned* m, float v) {   // the warp's largest value, one atomic
 #pragma unroll
@@ -1296,19 +1311,22 @@ __global__ void __launch_bounds__(SERIES_THREADS) series_kernel(const SeriesArgs
     if (ij.x == ij.y) e.w -= 1.0;
     const V v = vec((TA)e.w, (TA)e.x, (TA)e.y, (TA)e.z);
     ev[o] = v;
+    if (LO) el[o] = vec((TA)(e.w - (double)v.x), (TA)(e.x - (double)v.y), (TA)(e.y - (double)v.z), (TA)(e.z - (double)v.w));
     s1[o] = s2[o] = vec(0, 0, 0, 0);
     static_cast<V*>(a.fc[0])[o] = (ij.x == ij.y) ? vec((TA)0.5 * v.x, 0, 0, 0) : v;
-    const float m4 = fmaxf(fmaxf(fabsf((float)v.x), fabsf((float)v.y)), fmaxf(fabsf((float)v.z), fabsf((float)v.w)));
-    mx = (m4 <= mx) ? mx : m4;   // a NaN stays
+    // a NaN in any component counts as infinite (fmaxf would drop it)
+    for (const float f : {(float)v.x, (float)v.y, (float)v.z, (float)v.w}) mx = isnan(f) ? INFINITY : fmaxf(mx, fabsf(f));
   }
-  raise(a.mx, isnan(mx) ? INFINITY : mx);
+  raise(a.mx, mx);
   if (!series_barrier(a, bar++)) return;
   const float emax = largest(a.mx);
   const bool chol = !((double)emax * l <= SERIES_MAX);
   if (gt == 0) *a.use_chol = chol ? 1 : 0;
   if (chol) return;
-  // a step's change times this bounds the next one's
-  const float rate = 4.f * (float)l * emax;
+  // A step's change times this bounds the next one's, component by component: a change of F enters both
+  // factors of F^H F (8 l max|F|, four products a component), one of D only F D (4 l max|F|); max|F| may
+  // exceed max|E| by less than an eighth.
+  const float rate = 9.f * (float)l * emax, rate_d = 4.5f * (float)l * emax;
   // One step: sum(i, j) by the entry's lanes, kept in `prev` by its owner, who writes next(i, j, sum);
   // the largest change of a sum goes to m.
   auto step = [&](unsigned* m, V* prev, auto sum, auto next) {
@@ -1337,8 +1355,19 @@ __global__ void __launch_bounds__(SERIES_THREADS) series_kernel(const SeriesArgs
     raise(m, ch);
   };
   auto phi = [&](int i, int j, const Quat<TA>& s) {   // Phi(E - s)(i, j)
-    const V e = ev[(size_t)j * l + i];
-    return (i == j) ? vec((TA)0.5 * (e.x - s.w), 0, 0, 0) : vec(e.x - s.w, e.y - s.x, e.z - s.y, e.w - s.z);
+    const size_t o = (size_t)j * l + i;
+    const V e = ev[o], lo = LO ? el[o] : vec(0, 0, 0, 0);
+    V v, r;
+    series_diff(e.x, lo.x, s.w, v.x, r.x);
+    series_diff(e.y, lo.y, s.x, v.y, r.y);
+    series_diff(e.z, lo.z, s.y, v.z, r.z);
+    series_diff(e.w, lo.w, s.z, v.w, r.w);
+    if (i == j) {
+      v = vec((TA)0.5 * v.x, 0, 0, 0);
+      r = vec((TA)0.5 * r.x, 0, 0, 0);
+    }
+    if (LO) fl[o] = r;
+    return v;
   };
   // F <- Phi(E - F^H F), (F^H F)_ij = sum_{t <= i} conj(F_ti) F_tj
   int cur = 0;
@@ -1388,12 +1417,18 @@ __global__ void __launch_bounds__(SERIES_THREADS) series_kernel(const SeriesArgs
            return acc;
          },
          [&](int i, int j, const Quat<TA>& s) {
-           const V f = Ff[(size_t)j * l + i];
-           Dn[(size_t)j * l + i] = vec(-f.x - s.w, -f.y - s.x, -f.z - s.y, -f.w - s.z);
+           const size_t o = (size_t)j * l + i;
+           const V f = Ff[o], lo = LO ? fl[o] : vec(0, 0, 0, 0);
+           V v, r;                                           // -(f + s)
+           series_diff(-f.x, -lo.x, s.w, v.x, r.x);
+           series_diff(-f.y, -lo.y, s.x, v.y, r.y);
+           series_diff(-f.z, -lo.z, s.y, v.z, r.z);
+           series_diff(-f.w, -lo.w, s.z, v.w, r.w);
+           Dn[o] = v;
          });
     cur ^= 1;
     if (!series_barrier(a, bar++)) return;
-    if ((double)largest(m) * rate <= SERIES_TOL) break;
+    if ((double)largest(m) * rate_d <= SERIES_TOL) break;
   }
   // R2 = I + F and R2^{-1} = I + D in FP64 from E and the sums, by their entries' owners (16 lanes
   // take the four components of R2, R2inv and their zero mirror images)
@@ -2140,6 +2175,8 @@ static int series_factor(qlr_ctx* ctx, int l, const double* G, double* R2, doubl
   SeriesArgs a{};
   a.G = G;
   for (void** v : {&a.e, &a.s1, &a.s2, &a.fc[0], &a.fc[1], &a.fr, &a.dc[0], &a.dc[1]}) *v = ws.take<char>(ll * vsz);
+  if (f32acc)
+    for (void** v : {&a.elo, &a.flo}) *v = ws.take<char>(ll * vsz);
   a.mx = ws.take<unsigned>(NMAX + 1);
   a.arrived = a.mx + NMAX;
   a.use_chol = ws.take<int>(1);
