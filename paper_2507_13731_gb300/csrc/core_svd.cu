@@ -101,10 +101,10 @@ __device__ inline unsigned await_progress(const Progress* pg, unsigned have, int
 }
 
 // A sweep whose rotations all had cosine (of the pair before it) and sine at most thr leaves every
-// cosine within l thr^2: its own pair's is zero, and each of the up to l later rotations of either
-// column mixes in at most sine times cosine.  thr^2 = tol / l makes that the tolerance.
+// cosine within 2 l thr^2: its own pair's is zero, and each of the up to l later rotations of either of
+// its two columns mixes in at most sine times cosine.  thr^2 = tol / (2 l) makes that the tolerance.
 template <class T>
-__device__ __forceinline__ T last_sweep_threshold2(T tol, int l) { return tol / (T)l; }
+__device__ __forceinline__ T last_sweep_threshold2(T tol, int l) { return tol / (T)(2 * l); }
 
 // Reciprocal and reciprocal square root for the rotation parameters: the hardware approximations
 // in float (a few ulp; every rotation is applied to W and V, or logged and replayed, exactly as
