@@ -70,9 +70,11 @@ __device__ __forceinline__ void rr_pair(int lp, int r, int i, int& p, int& q) {
 
 // How far the log is written, for the replaying CTAs of the same launch: `count` units published
 // (release, after a barrier behind the records' stores), `done` set after the last of them.  The
-// CTA (or cluster) that sweeps has the lowest block indices and waits for nobody; a replaying CTA's
-// wait is bounded.
-struct Progress { unsigned count, done; };
+// CTA (or cluster) that sweeps is the one that draws the first ticket, whatever its index (CUDA promises
+// no order in which blocks start): it is running when the others begin to wait for it, and waits for
+// nobody.  A replaying CTA's wait is bounded as well.
+constexpr int MAX_CLUSTERS = 8;
+struct Progress { unsigned count, done, tickets, ticket_of[MAX_CLUSTERS]; };   // count, done, tickets zeroed
 __device__ __forceinline__ void publish(unsigned* p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -329,9 +331,12 @@ __global__ void __launch_bounds__(480) jacobi_small_kernel(const double* __restr
   const int t = threadIdx.x, lane = t % 32, warp = t / 32, nwarps = blockDim.x / 32;
   const int lp = l + (l & 1), np = lp / 2, rounds = lp - 1;
   const size_t ll = (size_t)l * l;
-  if (blockIdx.x > 0) {
+  __shared__ unsigned ticket;
+  if (t == 0) ticket = atomicAdd(&pg->tickets, 1u);
+  __syncthreads();
+  if (ticket > 0) {
     // ---------------- replay: one warp per row of V, a lane per pair of the round ----------------
-    const int row = (blockIdx.x - 1) * nwarps + warp;
+    const int row = ((int)ticket - 1) * nwarps + warp;
     if (row >= l) return;
     V4* vr = W + (size_t)warp * l;
     for (int j = lane; j < l; j += 32) stq<T>(vr + j, j == row ? (T)1 : (T)0, 0, 0, 0);
@@ -699,7 +704,7 @@ __device__ void jacobi_block_replay(int l, int bw, int jp, int cta, const T* __r
                                     T* __restrict__ Vout, unsigned char* smem, int* err);
 
 // Rows per lane RPL: the two columns of a pair stay in registers between the dot products and
-// the rotation (l <= 32 RPL).  The first cluster of jp CTAs sweeps, the others replay.
+// the rotation (l <= 32 RPL).  The cluster of jp CTAs with the first ticket sweeps, the others replay.
 template <class T, int RPL, int NT>
 __global__ void __launch_bounds__(NT, 1) jacobi_block_kernel(const double* __restrict__ R, int l, int bw, int jp,
                                                                    T* __restrict__ W, T* __restrict__ Vout,
@@ -708,13 +713,17 @@ __global__ void __launch_bounds__(NT, 1) jacobi_block_kernel(const double* __res
                                                                    int* __restrict__ sweeps_out, T* __restrict__ sig_out,
                                                                    Progress* __restrict__ pg, int* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if ((int)blockIdx.x >= jp) {   // whole clusters: no cluster barrier is left waiting
-    jacobi_block_replay<T>(l, bw, jp, (int)blockIdx.x - jp, rlog, pg, Vout, smem_raw, err);
+  cg::cluster_group cluster = cg::this_cluster();
+  const int p = (int)cluster.block_rank();
+  unsigned* my_ticket = &pg->ticket_of[blockIdx.x / jp];
+  if (p == 0 && threadIdx.x == 0) *my_ticket = atomicAdd(&pg->tickets, 1u);
+  cluster.sync();
+  const int ticket = (int)__ldcg(my_ticket);
+  if (ticket > 0) {              // whole clusters: no cluster barrier is left waiting
+    jacobi_block_replay<T>(l, bw, jp, (ticket - 1) * jp + p, rlog, pg, Vout, smem_raw, err);
     return;
   }
   T* S = reinterpret_cast<T*>(smem_raw);          // [4][2 bw][l]: plane, local column, row
-  cg::cluster_group cluster = cg::this_cluster();
-  const int p = (int)cluster.block_rank();
   const int t = threadIdx.x, lane = t % 32, warp = t / 32, nwarps = NT / 32;
   const size_t ll = (size_t)l * l;
   const int JPR = jp;                             // cluster size
@@ -1230,6 +1239,7 @@ static int core_tsvd_t(qlr_ctx* ctx, int l, const double* R, int k, double* L, d
     const int threads = wide ? JB_THREADS_WIDE : JB_THREADS;
     const size_t smem = block_jacobi_smem(l, bw, jp, sizeof(T), threads);
     const int replay = (l + threads / 32 - 1) / (threads / 32);   // CTAs with rows of V
+    if ((replay + jp - 1) / jp >= MAX_CLUSTERS) return QLR_EUNSUPPORTED;   // 256 rows: at most 4 clusters
     QLR_TRY(qlr_allow_smem(kern));
     cudaLaunchConfig_t cfg = {};
     if (jp > JP) QLR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
