@@ -186,11 +186,13 @@ int gemm_simt(qlr_ctx* ctx, const GemmArgs& g);
 int gram_f64_partials(qlr_ctx* ctx, const qlr_qmat& Y, int64_t chunks, int64_t rpc, double* part);
 
 // tcgen05 sketch products (see sketch_tc.cu)
-int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qmat& Y, int compute, WsArena& ws);
+// allow_fd = false: the plain form of the operand's staging, which needs the least scratch.
+int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qmat& Y, int compute, WsArena& ws,
+              bool allow_fd = true);
 size_t sketch_tc_ws(int64_t rows_in, int64_t l, int num_sms);
 // Exact scratch bytes sketch_tc takes for this product with a budget of num_sms stream-K CTAs
 // (staged thin operand, stream-K partial tiles; 256-byte aligned slices).
-size_t sketch_tc_need(int op, int64_t M, int64_t K, int l, int compute, int num_sms);
+size_t sketch_tc_need(int op, const qlr_qmat& A, const qlr_qmat& X, int compute, int num_sms, bool allow_fd);
 bool sketch_tc_supported(int op, const qlr_qmat& A, const qlr_qmat& X, int compute);
 
 // Grouped tensor-core sketch over many problems (one launch for the staging of every X and one

@@ -1578,18 +1578,25 @@ size_t sketch_tc_ws(int64_t rows_in, int64_t l, int num_sms) {
   return (size_t)2 * 4 * ldo * rows * 4 + (size_t)2 * (num_sms + 8) * 4 * TBM * 128 * 4 + 65536 + 4096;
 }
 
-size_t sketch_tc_need(int op, int64_t M, int64_t K, int l, int compute, int num_sms) {
-  const Plan pl = make_plan(compute, op, M, K, l, num_sms);   // a full quaternion A: the largest staging
-  const int64_t ldo = (K + 7) / 8 * 8;
+static Plan plan_of(int op, const qlr_qmat& A, const qlr_qmat& X, int compute, int num_sms, bool allow_fd) {
+  const bool n = op == QLR_OP_N;
+  return make_plan(compute, op, n ? A.rows : A.cols, n ? A.cols : A.rows, (int)X.cols, num_sms, true,
+                   A.plane[0] == nullptr ? 3 : 4, allow_fd && X.dtype == QLR_F32);
+}
+
+size_t sketch_tc_need(int op, const qlr_qmat& A, const qlr_qmat& X, int compute, int num_sms, bool allow_fd) {
+  const Plan pl = plan_of(op, A, X, compute, num_sms, allow_fd);
+  const int64_t ldo = (X.rows + 7) / 8 * 8;
   const size_t xesz = (pl.kind == K_BF16) ? 2 : 4;
-  const size_t xb = staged_x_bytes(pl.fd, 4, ldo, l, pl.nb, pl.ncb, xesz);
+  const size_t xb = staged_x_bytes(pl.fd, pl.apl, ldo, (int)X.cols, pl.nb, pl.ncb, xesz);
   size_t b = align256(xb);
   if (pl.kind == K_TF32X3) b += align256(xb);
   if (pl.grid_sk > 0) b += align256((size_t)2 * pl.grid_sk * 4 * TBM * pl.nb * sizeof(float));
   return b;
 }
 
-int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qmat& Y, int compute, WsArena& ws) {
+int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qmat& Y, int compute, WsArena& ws,
+              bool allow_fd) {
   if (!sketch_tc_supported(op, A, X, compute)) return QLR_EUNSUPPORTED;
   if (op != QLR_OP_N && op != QLR_OP_H) return QLR_EINVAL;
   const int64_t M = (op == QLR_OP_N) ? A.rows : A.cols;
@@ -1598,8 +1605,7 @@ int sketch_tc(qlr_ctx* ctx, int op, const qlr_qmat& A, const qlr_qmat& X, qlr_qm
   if (M == 0 || l == 0) return QLR_OK;
   if (K == 0) return zero_qmat(ctx, Y);
   if (X.dtype != QLR_F32 && !(compute == QLR_COMPUTE_BF16 && X.dtype == QLR_BF16)) return QLR_EINVAL;
-  const Plan pl = make_plan(compute, op, M, K, l, ctx->num_sms > 0 ? ctx->num_sms : 148, true,
-                            A.plane[0] == nullptr ? 3 : 4, X.dtype == QLR_F32);
+  const Plan pl = plan_of(op, A, X, compute, ctx->num_sms > 0 ? ctx->num_sms : 148, allow_fd);
   if (pl.stages < 2) return QLR_EUNSUPPORTED;
   size_t mark = ws.off;
   // stage the thin operand with a 16-byte aligned column pitch
