@@ -644,8 +644,9 @@ __global__ void __launch_bounds__(KIND == K_BF16 ? TC_THREADS : TC_THREADS_WIDE,
 }
 
 // The output tiles that stream-K reduced in pieces: Y = the sum of the pieces' partials in slot order.
-// blockIdx.x is the tile, blockIdx.y four of its 4 nb columns; a thread per row, up to 32 loads in
-// flight.  (The last CTA of a tile to finish did this before, 16 columns at a time while the others had
+// blockIdx.x is the tile or, where tiles are more than cuts (few of them are split then), the cut between two
+// CTAs' ranges, whose tile the first cut inside it takes; blockIdx.y four of the tile's 4 nb columns; a thread
+// per row, up to 32 loads in flight.  Over all tiles it started a million CTAs for 151 split ones at 10^6 rows.  (The last CTA of a tile to finish did this before, 16 columns at a time while the others had
 // left: 80 of 85 us at 1500 x 600 x 100, 12 tiles of 12 pieces.)
 constexpr int RED_COLS = 4, RED_AHEAD = 8;
 struct ReduceArgs {
@@ -653,13 +654,20 @@ struct ReduceArgs {
   float* y[4];
   int64_t ldy, M;
   int l, nb, ncb, kiters, mtiles, cgroup, grid;
+  int by_cut;
 };
 __global__ void __launch_bounds__(TBM) sketch_reduce_kernel(const ReduceArgs a) {
   const int NG = (a.cgroup && a.ncb > 1) ? a.ncb : 1;
   const StreamK sk{a.kiters, (int64_t)a.mtiles * (a.ncb / NG) * a.kiters, a.grid / NG};
   // tile t of the list (of its column block's list in groups)
   const int coff = NG > 1 ? (int)blockIdx.x % NG : 0;
-  const int64_t t = (int64_t)blockIdx.x / NG, K = a.kiters;
+  const int64_t K = a.kiters;
+  int64_t t = (int64_t)blockIdx.x / NG;
+  if (a.by_cut) {
+    const int64_t c = t + 1, x = sk.start(c);
+    t = x / K;
+    if (x == t * K || sk.start(c - 1) > t * K) return;
+  }
   const int cb = NG > 1 ? coff : (int)(t % a.ncb), mt = (int)(NG > 1 ? t : t / a.ncb);
   const int64_t c0 = sk.owner(t * K), c1 = sk.owner((t + 1) * K - 1);
   const int nseg = (int)(c1 - c0 + 1);
@@ -1247,7 +1255,10 @@ int launch_kernel(qlr_ctx* ctx, const Plan& pl, const TcParams& prm, int kid) {
     for (int c = 0; c < 4; ++c) ra.y[c] = prm.y[c];
     ra.ldy = prm.ldy; ra.M = prm.M; ra.l = prm.l; ra.nb = prm.nb; ra.ncb = prm.ncb; ra.kiters = prm.kiters;
     ra.mtiles = prm.mtiles; ra.cgroup = prm.cgroup; ra.grid = pl.grid_sk;
-    sketch_reduce_kernel<<<dim3((unsigned)(pl.mtiles * pl.ncb), (unsigned)(4 * ((pl.nb + RED_COLS - 1) / RED_COLS))), TBM, 0,
+    const int ng = (pl.cgroup && pl.ncb > 1) ? pl.ncb : 1, cuts = pl.grid_sk - ng, tiles = pl.mtiles * pl.ncb;
+    ra.by_cut = cuts < tiles ? 1 : 0;
+    if (cuts == 0) return QLR_OK;   // one CTA (of each column block): nothing is split
+    sketch_reduce_kernel<<<dim3((unsigned)std::min(cuts, tiles), (unsigned)(4 * ((pl.nb + RED_COLS - 1) / RED_COLS))), TBM, 0,
                            ctx->stream>>>(ra);
   } else {
     kern<<<dim3((unsigned)pl.ncb, (unsigned)pl.mtiles, 1u), threads, pl.smem, ctx->stream>>>(prm);
