@@ -562,19 +562,26 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
           }
           if (!valid_row) continue;
           const bool accumulate = !first && !pv.ttotal;     // global running sum
+          // pointers stepped by the pitch: 64-bit products for every entry bound the tall sketches of
+          // short reductions (pure 10^6 x 256 x 60 TF32: 1249 us, now 1133)
+          float* const col = dst + (int64_t)(cc + (sg.nseg == 1 ? j0 : 0)) * stride;
+          const int ncol = sg.nseg == 1 ? min(nb - cc, pv.l - j0 - cc) : nb - cc;
+          // one pointer for all entries: the compiler would keep 32 of them and spill
+          auto step = [&](float*& o) {
+            o += stride;
+            asm volatile("" : "+l"(o));
+          };
           float old[32];
           if (accumulate) {
+            float* o = col;
 #pragma unroll
-            for (int jj = 0; jj < 32; ++jj) {
-              const bool in = (cc + jj < nb) && (sg.nseg > 1 || j0 + cc + jj < pv.l);
-              old[jj] = in ? dst[(int64_t)(cc + jj) * stride + (sg.nseg == 1 ? (int64_t)j0 * stride : 0)] : 0.f;
-            }
+            for (int jj = 0; jj < 32; ++jj, step(o)) old[jj] = jj < ncol ? *o : 0.f;
           }
+          float* o = col;
 #pragma unroll
-          for (int jj = 0; jj < 32; ++jj) {
-            const bool in = (cc + jj < nb) && (sg.nseg > 1 || j0 + cc + jj < pv.l);
+          for (int jj = 0; jj < 32; ++jj, step(o)) {
             const float v = __uint_as_float(jj < 16 ? r0[jj] : r1[jj - 16]);
-            if (in) dst[(int64_t)(cc + jj) * stride + (sg.nseg == 1 ? (int64_t)j0 * stride : 0)] = accumulate ? old[jj] + v : v;
+            if (jj < ncol) *o = accumulate ? old[jj] + v : v;
           }
         }
       }
