@@ -248,16 +248,11 @@ __device__ __forceinline__ void issue_stage(uint32_t lead, const StageDescs& D, 
 }
 
 // ---------------------------------------------------------------------------------------
-// A contiguous piece of one output tile's reduction: stages [it0, it1).  A tile reduced in
-// nseg > 1 pieces (stream-K) has them from CTAs c0 .. c0 + nseg - 1 of its group; piece o writes
-// its partial to slot 2 ((c0 + o) cs + coff) + (o == 0 ? b0 : 0) (b0 = 1 when the tile starts
-// inside CTA c0's range, as that CTA's second piece), and sketch_reduce_kernel adds the partials in
-// slot order.  A group is every CTA (cs = 1, coff = 0), or, with column-block groups,
-// the CTAs coff, coff + cs, coff + 2 cs, ... of one column block (cs = the number of blocks).
+// A contiguous piece of one output tile's reduction: stages [it0, it1).  Of a tile reduced in
+// nseg > 1 pieces (stream-K) each writes its partial to its slot, and sketch_reduce_kernel adds them.
 struct Seg {
-  int it0, it1, slot, nseg, c0, b0;
+  int it0, it1, slot, nseg;
   int more;   // another piece follows in this CTA: keep the right to allocate TMEM
-  int cs = 1, coff = 0;
 };
 
 // One output tile (column block cb, row tile mt) over the reduction piece sg.
@@ -603,7 +598,7 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
 // One CTA per output tile, the whole reduction.
 template <int KIND, int AMODE, bool WIDE>
 __global__ void __launch_bounds__(KIND == K_BF16 ? TC_THREADS : TC_THREADS_WIDE, 1) sketch_tc_kernel(const __grid_constant__ TcParams p) {
-  sketch_tile<KIND, AMODE, WIDE>(p, blockIdx.x, blockIdx.y, Seg{0, p.kiters, 0, 1, 0, 0, 0});
+  sketch_tile<KIND, AMODE, WIDE>(p, blockIdx.x, blockIdx.y, Seg{0, p.kiters, 0, 1, 0});
 }
 
 // Stream-K: the reduction stages of all tiles, taken in tile order, are cut into gridDim.x equal
@@ -640,8 +635,7 @@ __global__ void __launch_bounds__(KIND == K_BF16 ? TC_THREADS : TC_THREADS_WIDE,
     const int64_t c0 = sk.owner(t * K), c1 = sk.owner((t + 1) * K - 1);
     const int b0 = (sk.start(c0) < t * K) ? 1 : 0;
     const int more = (pos + (it1 - it0) < end) ? 1 : 0;
-    const Seg sg{it0, it1, (int)(2 * (c * NG + cbg) + (c == c0 ? b0 : 0)), (int)(c1 - c0 + 1), (int)c0, b0, more,
-                 NG, cbg};
+    const Seg sg{it0, it1, (int)(2 * (c * NG + cbg) + (c == c0 ? b0 : 0)), (int)(c1 - c0 + 1), more};
     if (!first) __syncthreads();
     const int mt = (NG > 1) ? (int)t : (int)t / p.ncb;
     sketch_tile<KIND, AMODE, WIDE>(p, (NG > 1) ? cbg : (int)t - mt * p.ncb, mt, sg);
@@ -724,7 +718,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) sketch_tc_grouped_kernel(const 
         asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&p.tmXlo[q]) : "memory");
     }
   }
-  sketch_tile<KIND, AMODE>(p, it.z, it.y, Seg{0, p.kiters, 0, 1, 0, 0, 0});
+  sketch_tile<KIND, AMODE>(p, it.z, it.y, Seg{0, p.kiters, 0, 1, 0});
 }
 
 // Persistent grouped form: gridDim.x CTAs (one per SM) walk the item list, CTA b taking items
