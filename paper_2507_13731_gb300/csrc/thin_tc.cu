@@ -256,6 +256,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
   uint64_t* acc_empty = acc_full + TL_ACC;       // [TL_ACC]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + TL_ACC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  unsigned* seen = tmem_slot + 2;                // [3] over the whole operands: largest exponents, tiny entries
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const int64_t tiles = (int64_t)p.mtiles * p.ntiles;
   const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
@@ -270,6 +271,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
     mbar_init(adone, TL_ISSUERS);
     for (int b = 0; b < TL_ACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], TL_EPI); }
     *abort_flag = 0;
+    seen[0] = seen[1] = seen[2] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -420,21 +422,33 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
     uint32_t bph = 0;
     unsigned ea = 0;                                   // largest biased exponent of these rows
     bool ok = true;
+    // What the split kernels found, over the whole operands, while the first tile is on its way: tiles are
+    // looked at one by one only if there is something to find (their 16 bytes a tile cost 6 % of an update of
+    // rank 8).
+    const int rblocks = (p.Kq + 4 * 32 - 1) / (4 * 32);
+    bool look;
+    {
+      unsigned a4 = 0, be = 0, tiny = 0;
+      const unsigned* af = reinterpret_cast<const unsigned*>(p.aflags);
+      const int64_t words = (p.M + SPLIT_ROWS - 1) / SPLIT_ROWS * (p.Kq / 16);
+      for (int64_t i = threadIdx.x; i < words; i += 32 * TL_EPI) a4 = __vmaxu4(a4, af[i]);
+      for (int i = threadIdx.x; i < p.ntiles * rblocks; i += 32 * TL_EPI) {
+        const uint4 f = p.bflags[(size_t)(i / rblocks) * TL_MAX_RB + i % rblocks];
+        tiny |= f.x;
+        be = max(be, f.z);
+      }
+      a4 = __vmaxu4(a4, a4 >> 16);
+      a4 = __reduce_max_sync(0xffffffffu, __vmaxu4(a4, a4 >> 8) & 255u);
+      be = __reduce_max_sync(0xffffffffu, be);
+      tiny = __reduce_or_sync(0xffffffffu, tiny);
+      if (lane == 0) { atomicMax(&seen[0], a4); atomicMax(&seen[1], be); atomicOr(&seen[2], tiny); }
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * TL_EPI) : "memory");
+      look = seen[0] == 255u || seen[1] == 255u || seen[2] != 0 || seen[0] + seen[1] > EXP_SUM_MAX;
+    }
     for (int left = (int)(t1 - t0); left > 0 && ok; --left) {
-      // what the split kernels found: loads in flight while the MMAs run
-      unsigned tiny_cols = 0, big_cols = 0, eb = 0, rows4 = 0;
-      if (32 * lane < p.Kq / 4) {
-        const uint4 f = p.bflags[(size_t)nt * TL_MAX_RB + lane];
-        tiny_cols = f.x; big_cols = f.y; eb = f.z;
-      }
-      const bool fresh = mt != cur;
-      if (fresh) {
-        const unsigned* af = reinterpret_cast<const unsigned*>(p.aflags + (size_t)(mt / (SPLIT_ROWS / TL_M)) * (p.Kq / 4));
-        for (int w = lane; w < p.Kq / 16; w += 32) rows4 = __vmaxu4(rows4, af[w]);
-      }
-      cur = mt;
       const int64_t row = (int64_t)mt * TL_M + q * 32 + lane, j0 = (int64_t)nt * TL_J + half * 16;
       const int nch = (ksteps_of(nt) + per - 1) / per;
+      const int tmt = mt;
       if (++nt == p.ntiles) { nt = 0; ++mt; }
       const bool row_ok = row < p.M;
       const int nj = (int)max((int64_t)0, min((int64_t)16, p.N - j0));   // valid columns of this warp's 16
@@ -466,13 +480,21 @@ __global__ void __launch_bounds__(TL_THREADS, 1) tall_gemm_kernel(const __grid_c
         if (++b == TL_ACC) { b = 0; bph ^= 1u; }
       }
       if (!ok) break;
-      if (fresh) {
-        const unsigned r4 = __vmaxu4(rows4, rows4 >> 16);
-        ea = __reduce_max_sync(0xffffffffu, __vmaxu4(r4, r4 >> 8) & 255u);
+      bool again = false;
+      if (look) {
+        if (tmt != cur) {
+          unsigned a4 = 0;
+          const unsigned* af = reinterpret_cast<const unsigned*>(p.aflags + (size_t)(tmt / (SPLIT_ROWS / TL_M)) * (p.Kq / 4));
+          for (int w = lane; w < p.Kq / 16; w += 32) a4 = __vmaxu4(a4, af[w]);
+          a4 = __vmaxu4(a4, a4 >> 16);
+          ea = __reduce_max_sync(0xffffffffu, __vmaxu4(a4, a4 >> 8) & 255u);
+          cur = tmt;
+        }
+        const uint4 f = lane < rblocks ? p.bflags[(size_t)(j0 / TL_J) * TL_MAX_RB + lane] : make_uint4(0u, 0u, 0u, 0u);
+        const unsigned eb = __reduce_max_sync(0xffffffffu, f.z);
+        const unsigned tc = __reduce_or_sync(0xffffffffu, f.x) & ~__reduce_or_sync(0xffffffffu, f.y);
+        again = tc != 0 || ea == 255u || eb == 255u || ea + eb > EXP_SUM_MAX;
       }
-      eb = __reduce_max_sync(0xffffffffu, eb);
-      const unsigned tc = __reduce_or_sync(0xffffffffu, tiny_cols) & ~__reduce_or_sync(0xffffffffu, big_cols);
-      const bool again = tc != 0 || ea == 255u || eb == 255u || ea + eb > EXP_SUM_MAX;
       if (!row_ok) continue;
       if (again) {   // FP32 multiply-adds on the operands as given (the sums' values are not used)
         constexpr uint32_t neg = MASKED ? NEG_MASKED : NEG_THIN;
