@@ -516,8 +516,27 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
       const uint32_t tbase = tmem + (uint32_t)(4 * nb);   // running sum (pv.ttotal)
       const bool to_total = pv.ttotal && !last;             // this chunk only updates the TMEM sum
       const bool add_total = pv.ttotal && !first;           // the TMEM sum enters this chunk's values
+      if (to_total) {   // the four planes' columns lie together, 4 nb a multiple of 64
 #pragma unroll 1
-      for (int d = 0; d < 4; ++d) {
+        for (int cc = 32 * eh; cc < 4 * nb; cc += 32 * EPI) {
+          const uint32_t lane_off = ((uint32_t)(q * 32) << 16) + (uint32_t)cc;
+          uint32_t r[32];
+          tmem_ld32_issue(abase + lane_off, r);
+          if (add_total) {
+            uint32_t s[32];
+            tmem_ld32_issue(tbase + lane_off, s);
+            tmem_wait_ld();
+#pragma unroll
+            for (int jj = 0; jj < 32; ++jj) r[jj] = __float_as_uint(__uint_as_float(s[jj]) + __uint_as_float(r[jj]));
+          } else {
+            tmem_wait_ld();
+          }
+          tmem_st32(tbase + lane_off, r);
+        }
+        tmem_wait_st();
+      }
+#pragma unroll 1
+      for (int d = 0; d < 4 && !to_total; ++d) {
         // the output plane d of this tile: Y itself (a whole tile) or this piece's partial slot
         float* dst;
         int64_t stride;
@@ -550,21 +569,16 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
               r1[jj] = __float_as_uint(__uint_as_float(s1[jj]) + __uint_as_float(r1[jj]));
             }
           }
-          if (to_total) {
-            tmem_st16(tbase + lane_off, r0);
-            if (cc + 16 < nb) tmem_st16(tbase + lane_off + 16, r1);
-            continue;
-          }
           if (!valid_row) continue;
           const bool accumulate = !first && !pv.ttotal;     // global running sum
-          // pointers stepped by the pitch: 64-bit products for every entry bound the tall sketches of
-          // short reductions (pure 10^6 x 256 x 60 TF32: 1249 us, now 1133)
           float* const col = dst + (int64_t)(cc + (sg.nseg == 1 ? j0 : 0)) * stride;
           const int ncol = sg.nseg == 1 ? min(nb - cc, pv.l - j0 - cc) : nb - cc;
-          // one pointer for all entries: the compiler would keep 32 of them and spill
+          // One pointer stepped by the pitch, kept to one by an empty asm: the registers of 384 threads do not
+          // hold 32 of them, and a 64-bit product for every entry bound the tall sketches of short
+          // reductions (pure 10^6 x 256 x 60 TF32: 1249 us, now 1078).  BF16's 256 threads hold them.
           auto step = [&](float*& o) {
             o += stride;
-            asm volatile("" : "+l"(o));
+            if (KIND != K_BF16) asm("" : "+l"(o));
           };
           float old[32];
           if (accumulate) {
@@ -574,13 +588,19 @@ __device__ __forceinline__ void sketch_tile(const TcParams& p, const int cb, con
           }
           float* o = col;
 #pragma unroll
-          for (int jj = 0; jj < 32; ++jj, step(o)) {
-            const float v = __uint_as_float(jj < 16 ? r0[jj] : r1[jj - 16]);
+          for (int jj = 0; jj < 16; ++jj, step(o)) {
+            const float v = __uint_as_float(r0[jj]);
             if (jj < ncol) *o = accumulate ? old[jj] + v : v;
+          }
+          if (ncol > 16) {
+#pragma unroll
+            for (int jj = 0; jj < 16; ++jj, step(o)) {
+              const float v = __uint_as_float(r1[jj]);
+              if (16 + jj < ncol) *o = accumulate ? old[16 + jj] + v : v;
+            }
           }
         }
       }
-      if (to_total) tmem_wait_st();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tmem_empty[b]);   // this chunk's accumulator may be overwritten
