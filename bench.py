@@ -152,18 +152,21 @@ def peak_for(compute: str):
     return None, None, 1, None
 
 
-def sketch_roofline(flops: float, nbytes: float, ms: float, launches: int, compute: str, traffic=None):
+def sketch_roofline(flops: float, nbytes: float, ms: float, launches: int, compute: str, traffic=None, sketches=None):
     """Roofline object of the sketch launches of a timed region: achieved = algorithmic work of all
-    launches / their summed CUDA-event time; bound = the roof the work meets first."""
+    launches / their summed CUDA-event time; bound = the roof the work meets first.  A sketch whose
+    reduction is split counts two launches (the product and the addition of its pieces): the averages
+    and the figures "per launch" are those of one of the `sketches` products, its addition included."""
+    n = max(sketches or launches, 1)
     pk, src = _peaks()
     hbm = pk.get("hbm_gbs", 6800.0)
     peak, unit, products, note = peak_for(compute)
     sec = ms / 1e3
     t_hbm = nbytes / (hbm * 1e9)
     t_ops = flops * products / (peak * 1e12) if peak else 0.0
-    out = {"kernel": "sketch_tc" if compute != "F32" else "sketch_simt", "launches": launches,
-           "avg_ms": round(ms / max(launches, 1), 5), "algorithmic_flops_per_launch": flops / max(launches, 1),
-           "algorithmic_bytes_per_launch": nbytes / max(launches, 1), "traffic": traffic}
+    out = {"kernel": "sketch_tc" if compute != "F32" else "sketch_simt", "launches": launches, "sketches": n,
+           "avg_ms": round(ms / n, 5), "algorithmic_flops_per_launch": flops / n,
+           "algorithmic_bytes_per_launch": nbytes / n, "traffic": traffic}
     if t_hbm >= t_ops:
         ach = nbytes / sec / 1e9
         out.update({"bound": "hbm", "achieved": round(ach, 2), "peak": round(hbm, 1), "unit": "GB/s",
@@ -398,7 +401,7 @@ def mixed_precision_leg(dev, golden, reps=3):
         if nl:
             fl, nb = sketch_work(P.m, P.n, [P.k + P.p] * 4 * n, False, 2 if mode == "BF16" else 4)
             ent["sketch"] = sketch_roofline(fl, nb, kms, nl, mode,
-                                            traffic_for("sketch_tc_bf16_c3") if mode == "BF16" else None)
+                                            traffic_for("sketch_tc_bf16_c3") if mode == "BF16" else None, 4 * n)
         ent["kernels_ms_per_qsvd"] = {k: round(t / n, 3) for k, (c, t) in st.items() if c}
         out[mode] = ent
     rc = ctx.sync()
@@ -1036,7 +1039,8 @@ def main():
             if not nl:
                 continue
             flops, nbytes = sketch_work(HM, HN, ws_ * args.steps, True, 4)
-            r = sketch_roofline(flops, nbytes, kms, nl, comp, traffic_for(f"{kid}_{comp.lower()}_c4"))
+            r = sketch_roofline(flops, nbytes, kms, nl, comp, traffic_for(f"{kid}_{comp.lower()}_c4"),
+                                len(ws_) * args.steps)
             r.update({"class": kid, "compute": comp, "pass_widths": ws_, "class_share": round(kms / total_ms, 4)})
             roofs.append(r)
         roof = dict(max(roofs, key=lambda r: r["class_share"]))   # the sketch class with most time

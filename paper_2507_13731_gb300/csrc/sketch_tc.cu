@@ -25,9 +25,8 @@
 // positions are counters (the integer divisions they replace took 300 of a stage's 1700 cycles in
 // plain TF32), and the whole warp runs its loop with one elected lane issuing (see umma_bf16).
 // Measured (Y = A X and Z = A^H W together, with the staging; one lane with divisions, with counters,
-// and now with the choice of form below): 3xTF32 4096 x 4096 x 110 761, 630, 525 us, BF16 16384 x
-// 8192 x 220 1638, 1522, 1277 us, TF32 pure 20000 x 10000 x 60 1431, 1348, 1201 us, rounded TF32
-// x 180 5021, 4736, 3796 us.
+// and now): 3xTF32 4096 x 4096 x 110 761, 630, 483 us, BF16 16384 x 8192 x 220 1638, 1522, 1261 us,
+// TF32 pure 20000 x 10000 x 60 1431, 1348, 1189 us, rounded TF32 x 180 5021, 4736, 3650 us.
 //
 // Precision modes: BF16 (kind::f16, A stored BF16, X rounded to BF16), TF32 (kind::tf32, one
 // product on FP32 data, which the tensor cores truncate to TF32), rounded TF32 (one product, A and
