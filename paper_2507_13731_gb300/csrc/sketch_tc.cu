@@ -1231,7 +1231,8 @@ Plan make_plan(int compute, int op, int64_t M, int64_t K, int l, int num_sms, bo
   // their accumulators truncate, so other cuts give other results.
   int64_t cuts = 0;
   if (pl.kind == K_TF32X3 || pl.rn) cuts = std::min<int64_t>(num_sms / tiles, pl.kiters);
-  if (cuts > 1 && pl.kiters < 24 * cuts) pl.grid_sk = (int)(tiles * cuts);
+  const bool equal = cuts > 1 && pl.kiters < 24 * cuts;
+  if (equal) pl.grid_sk = (int)(tiles * cuts);
   else if (g > tiles) pl.grid_sk = (int)g;
   else if (tiles > num_sms && tiles % num_sms != 0 && g == num_sms) pl.grid_sk = num_sms;
   else pl.grid_sk = 0;
@@ -1242,6 +1243,14 @@ Plan make_plan(int compute, int op, int64_t M, int64_t K, int l, int num_sms, bo
     pl.cgroup = true;
   }
   pl.flush = (pl.kind == K_TF32X3) ? X3_FLUSH_STAGES : pl.rn ? RN_FLUSH_K / pl.bk : 0;
+  // Where equal pieces leave SMs idle they are longer than the ranges they stand for, and the truncation grows
+  // with the length: 3xTF32 then takes a piece of more than 8 stages in two chunks.  Pure 6000 x 500 x 100:
+  // 3.6e-6 in ranges, 4.2e-6 in pieces, 2.3e-6 in two chunks of them (132, 62 and 70 us; blocks of at most
+  // 64 columns, summed in TMEM, take no longer).  Rounded operands are off by a hundred times as much.
+  if (equal && pl.kind == K_TF32X3 && num_sms % tiles != 0) {
+    const int piece = (int)((pl.kiters + cuts - 1) / cuts);
+    if (piece > 8) pl.flush = (piece + 1) / 2;
+  }
   // chunk sums in TMEM next to the chunk accumulator when both fit (column blocks <= 64), else in
   // the output with two chunk buffers
   pl.ttotal = (pl.flush > 0 && 8 * pl.nb <= 512) ? 1 : 0;
