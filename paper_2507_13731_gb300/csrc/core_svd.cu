@@ -275,7 +275,8 @@ __global__ void __launch_bounds__(JT) jacobi_kernel(const double* __restrict__ R
 // between the dot products and the rotation; every pair of a round at once; quaternions as one
 // 16- or 32-byte vector.  In FP64 the six dot products are reduced in transposed form (8 additions
 // a lane instead of 24).  Measured (sweeps, replay and
-// refinement, before and now): FP32 l = 40 736 and 363 us; FP64 l = 15 1144 and 447 us.
+// refinement, before and now): FP32 l = 40 736 and 363 us; FP64 l = 15, whole
+// calls, 1188 and 491 us.
 template <class T> struct Q4;
 template <> struct Q4<float> { using V = float4; using H = float2; };
 template <> struct Q4<double> { using V = double4; using H = double2; };

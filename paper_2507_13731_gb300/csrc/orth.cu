@@ -1185,7 +1185,7 @@ __global__ void __launch_bounds__(256) tri_inv_blocked_kernel(const double* __re
 // entry by more than SERIES_TOL (far below the FP64 resolution of I + F).
 // One cooperative launch runs everything, a barrier over its CTAs between two steps: as 16 launches
 // (most of them finding their iteration converged) the series took 206 us at l = 180 and 49 us at
-// l = 60 plus the gaps between them, now 88 and 31 (l = 40: 40 and 14).  The factors that a step multiplies are kept as
+// l = 60 plus the gaps between them, now 98 and 32.  The factors that a step multiplies are kept as
 // quaternion vectors in the accumulation type, F in both orders, so every lane reads consecutive
 // 16-byte (FP64: 32-byte) entries.
 // When l * max|E_ij| exceeds SERIES_MAX the kernel raises `use_chol` and leaves; the blocked Cholesky

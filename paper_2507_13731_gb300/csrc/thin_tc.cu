@@ -29,13 +29,15 @@
 // issuer spends 500 more on barriers and commits, with the pipe idle: two issuing warps take the
 // stages in turn.
 //
-// Bound and measurements (CUDA events, GB300): the masked update writes 16 bytes per entry for
-// 6 * 32 k flops.  At 20000 x 10000, k = 50 the six products are 0.83 ms of tensor time and the
-// writes 0.5 ms; it takes 1.9 ms against 9.0 ms on the FP32 pipe (4096 x 4096, k = 30: 115 against
-// 575 us), what is left being the operands' L2 reads (64 bytes per SM and cycle at the full MMA
-// rate).  Q = Y R^{-1} at 20000 x 180: 118 us with the splits against 250.  Error against 64 bits at
-// 4096 x 4096: 7.1e-8 (k = 30) and 7.9e-8 (k = 50) relative, FP32 fused multiply-adds 1.1e-7 and
-// 1.4e-7.
+// Bound and measurements (CUDA events, GB300, whole calls): the masked update writes 16 bytes per entry
+// for 6 * 32 k flops.  At 20000 x 10000, k = 50 the six products are 0.83 ms of tensor time and the
+// writes 0.5 ms; it takes 1.83 ms against 9.03 ms on the FP32 pipe (4096 x 4096, k = 30: 123 against
+// 457 us).  No unit is at its limit (k = 30: tensor pipe active 39 % of the time, DRAM 52 %, L2 37 %); MMAs
+// and stores take turns within a CTA.  Q = Y R^{-1} at 20000 x 180: 115 us with the splits against 255.
+// Error against 64 bits, random operands: 8.5e-8 (4096 x 4096, k = 30) and 8.9e-8 (20000 x 10000, k = 50)
+// relative, FP32 fused multiply-adds 1.5e-7 and more.  About 5e-8 of it is truncation, always toward zero: a
+// product that follows another truncating one adds to its error rather than averaging out.  (Chunks of 16
+// elements at any length: 4e-8, but up to 24 % more error in all from k = 100 on, and 4 to 9 % more time.)
 #include <algorithm>
 #include <cstring>
 #include <type_traits>
@@ -670,8 +672,8 @@ int64_t panel_rows(int64_t m, int k) {
 namespace qlr {
 
 // The line lies where three launches on the tensor cores and one on the FP32 pipe take the same
-// time: 367 against 353 us for a CholeskyQR2 at rows N l = 18e6, 421 / 421 at 36e6, 543 / 551 at
-// 24e6 (l = 110), 2040 / 2310 at 20000 x 180.
+// time: 410 against 418 us for a CholeskyQR2 at rows N l = 24e6 (l = 110), 323 / 322 at 36e6 (l = 60),
+// 434 / 445 at 36e6 (l = 110), 405 / 423 at 72e6 (l = 60), 1465 / 1753 at 20000 x 180.
 bool tall_gemm_wanted(int64_t rows, int64_t N, int l) {
   return l >= 1 && l <= TALL_MAX_L && N >= 1 && rows < (1LL << 31) - TL_M && N < (1LL << 28) && rows * N * l >= (int64_t)24000000 && get_encode() != nullptr;
 }
@@ -703,8 +705,8 @@ int tall_gemm(qlr_ctx* ctx, const qlr_qmat& T, const double* const S[4], int64_t
   return rc;
 }
 
-// 24.4 against 21.8 us at m n k = 1e7, 27.8 / 35.1 at 3e7, 62 / 238 at 4096 x 4096, k = 8.  No more rows than
-// the other forms take, so that what is refused does not depend on the form.
+// On warm operands 24.4 against 21.8 us at m n k = 1e7 and 27.8 / 35.1 at 3e7; with L2 flushed and 30 % observed
+// 37.5 / 54.4 at 1.6e7, 47.8 / 97.4 at 3e7, 131 / 415 at 4096 x 4096, k = 8.  No more rows than the other forms take, so that what is refused does not depend on the form.
 bool masked_update_tc_wanted(int64_t m, int64_t n, int k) {
   return k >= 1 && k <= TALL_MAX_L && m <= COMPLETE_MAX_ROWS && n < (1LL << 31) && m * n * k >= (int64_t)15000000 &&
          get_encode() != nullptr;
